@@ -8,124 +8,286 @@
 // entry point computes, for every sub-cluster (k, h), the count, the sum of x and the
 // sum of x x^T of the points labelled (z = k, zbar = h), using only the caller's
 // buffers and a fixed scratch array that lives in this library's device image.  The
-// scratch (NA_G x 2 NA_KMAX x NA_EMAX doubles = 5.6 MiB) is held by every GPU that
+// scratch (32 x 2 NA_KMAX x NA_EMAX doubles = 5.6 MiB) is held by every GPU that
 // loads the library until the process exits.
 #include <cuda.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "dpmm_internal.cuh"
 
 namespace dpmm {
 
-constexpr int NA_G = 32;      // CTAs of the partial pass (one scratch slice each)
-constexpr int NA_KMAX = 16;   // clusters
-constexpr int NA_DMAX = 32;   // dimension
-constexpr int NA_P = 128;     // points per tile
+constexpr int NA_RANGES = 32;  // the points are cut into this many ranges, each into tiles
+constexpr int NA_KMAX = 16;    // clusters
+constexpr int NA_DMAX = 32;    // dimension
+constexpr int NA_P = 128;      // points per tile
 constexpr int NA_EMAX = 16 * (((NA_DMAX + 4) / 4) * ((NA_DMAX + 4) / 4 + 1) / 2);  // 720 entries
+constexpr int NA_W = 8;        // warps per block
+constexpr int NA_Q = 4;        // tiles whose labels a warp scans at a time
+constexpr int NA_D = 8;        // rows in flight per warp
+constexpr int NA_ROW = 52;     // floats of a staged row: x, then its first d / 2 + 1 values again
+constexpr size_t NA_SCRATCH = (size_t)32 * 2 * NA_KMAX * NA_EMAX;  // doubles
 
-static __device__ __align__(256) double g_na_scratch[(size_t)NA_G * 2 * NA_KMAX * NA_EMAX];
+static __device__ __align__(256) double g_na_scratch[NA_SCRATCH];
 
-// Pass 1: CTA g owns slice g (2K slots x E).  It clears the slice, then, tile by
-// tile, groups the tile's points by slot (stable ranks) and adds each slot's 4x4
-// register-block sums of xt xt^T (xt = [x, 1]) into its slice, in FP64.
-__global__ void __launch_bounds__(256) na_partial_kernel(const float* __restrict__ X, int64_t N, int d,
-                                                         const int32_t* __restrict__ z,
-                                                         const uint8_t* __restrict__ zbar, int K,
-                                                         StatLayout L, int G, double* scratch) {
-    __shared__ float xs[NA_P * (NA_DMAX + 4)];
-    __shared__ int slot[NA_P], order[NA_P], cnt[2 * NA_KMAX + 2];
-    __shared__ float red[256 * 16];
-    const int tid = threadIdx.x, nt = blockDim.x, g = blockIdx.x;
-    const int S = 2 * K, dp = L.dp, nblk = L.nblk, E = L.E;
-    double* slice = scratch + (size_t)g * S * E;
-    for (int e = tid; e < S * E; e += nt) slice[e] = 0.0;  // the array keeps the last call's contents
-    const int64_t R = (N + G - 1) / G, p0 = (int64_t)g * R, p1 = min(N, p0 + R);
-    const int ngrp = max(1, nt / nblk);
-    const bool worker = tid < nblk * ngrp;
-    const int myblk = worker ? tid % nblk : 0, grp = worker ? tid / nblk : 0;
-    int jb = 0, lb = 0;
-    L.blk_coords(myblk, jb, lb);
-    for (int64_t base = p0; base < p1; base += NA_P) {
-        const int np = (int)min((int64_t)NA_P, p1 - base);
-        __syncthreads();
-        if (tid < np) {
-            const int64_t i = base + tid;
-            float* xr = xs + tid * dp;
-            for (int j = 0; j < d; ++j) xr[j] = X[i * d + j];
-            xr[d] = 1.f;
-            for (int j = d + 1; j < dp; ++j) xr[j] = 0.f;
-            const int zi = z[i], hi = zbar[i];
-            // a label outside [0, K) x {0, 1} goes to the discard slot S and is not counted
-            slot[tid] = (zi >= 0 && zi < K && hi <= 1) ? 2 * zi + hi : S;
-        }
-        if (tid <= S + 1) cnt[tid] = 0;
-        __syncthreads();
-        if (tid < np) {  // stable position of this point among the tile's points of its slot
-            int s = slot[tid], r = 0;
-            for (int q = 0; q < tid; ++q) r += slot[q] == s;
-            order[tid] = r;
-            atomicAdd(&cnt[s + 1], 1);
-        }
-        __syncthreads();
-        if (tid == 0)
-            for (int s = 0; s <= S; ++s) cnt[s + 1] += cnt[s];
-        __syncthreads();
-        if (tid < np) {
-            int pos = cnt[slot[tid]] + order[tid];
-            order[tid] = pos;  // reuse: position of point tid in slot order
-        }
-        __syncthreads();
-        // inverse permutation into slot[] (points in slot order)
-        int mypos = tid < np ? order[tid] : -1;
-        __syncthreads();
-        if (tid < np) slot[mypos] = tid;
-        __syncthreads();
-        for (int s = 0; s < S; ++s) {
-            const int qs = cnt[s], qe = cnt[s + 1];
-            if (qs == qe) continue;  // uniform across the block
-            float acc[16];
-#pragma unroll
-            for (int e = 0; e < 16; ++e) acc[e] = 0.f;
-            if (worker)
-                for (int q = qs + grp; q < qe; q += ngrp) {
-                    const float* xr = xs + slot[q] * dp;
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) acc[u * 4 + v] += xr[jb * 4 + u] * xr[lb * 4 + v];
-                }
-            if (worker)
-#pragma unroll
-                for (int e = 0; e < 16; ++e) red[tid * 16 + e] = acc[e];
-            __syncthreads();
-            for (int e = tid; e < nblk * 16; e += nt) {
-                const int b = e >> 4, q = e & 15;
-                double v = 0.0;
-                for (int gg = 0; gg < ngrp; ++gg) v += (double)red[(gg * nblk + b) * 16 + q];
-                slice[(size_t)s * E + e] += v;
-            }
-            __syncthreads();
-        }
-    }
+// Two FP32 values in one register pair: the packed instructions do two lanes' work each.
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 f2_pack(float a, float b) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 f2_unpack(f2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
+    f2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
 }
 
-// Pass 2: sum the slices in CTA order (deterministic) and unpack n, sum x, sum x x^T.
-__global__ void na_combine_kernel(StatLayout L, int G, int K, const double* scratch, double* n_out, double* sx_out,
-                                  double* sxx_out) {
-    const int s = blockIdx.x, d = L.d, S = 2 * K, E = L.E;
-    auto M = [&](int j, int l) {
-        const int e = L.ent(j, l);
-        double v = 0.0;
-        for (int g = 0; g < G; ++g) v += scratch[((size_t)g * S + s) * E + e];
-        return v;
-    };
-    for (int q = threadIdx.x; q < d * d; q += blockDim.x) {
-        const int j = q / d, l = q % d;
-        sxx_out[(size_t)s * d * d + q] = j <= l ? M(j, l) : M(l, j);
+// Two sums, each an FP32 pair: s + c is the sum so far to about 48 bits.
+struct NaPair {
+    f2 s, c;
+    __device__ void zero() { s = c = 0ull; }
+    __device__ void add(f2 a) {  // two-sum: s + a = t + err exactly
+        const f2 t = f2_add(s, a), bb = f2_sub(t, s);
+        c = f2_add(c, f2_add(f2_sub(s, f2_sub(t, bb)), f2_sub(a, bb)));
+        s = t;
     }
-    for (int j = threadIdx.x; j < d; j += blockDim.x) sx_out[(size_t)s * d + j] = M(j, d);
-    if (threadIdx.x == 0) n_out[s] = M(d, d);
+    __device__ double2 value() const {
+        const float2 x = f2_unpack(s), y = f2_unpack(c);
+        return make_double2((double)x.x + (double)y.x, (double)x.y + (double)y.y);
+    }
+    __device__ bool bad() const {
+        const float2 x = f2_unpack(s), y = f2_unpack(c);
+        return !isfinite(x.x) || !isfinite(y.x) || !isfinite(x.y) || !isfinite(y.y);
+    }
+};
+struct NaDouble {
+    double2 v;
+    __device__ void zero() { v = make_double2(0.0, 0.0); }
+    __device__ void add(f2 a) {
+        const float2 x = f2_unpack(a);
+        v.x += (double)x.x;
+        v.y += (double)x.y;
+    }
+    __device__ double2 value() const { return v; }
+    __device__ bool bad() const { return false; }
+};
+
+struct NaArgs {
+    const float* X;
+    int64_t N;
+    int d;
+    const int32_t* z;
+    const uint8_t* zbar;
+    int K, G;    // slices
+    int W;       // FP32 groups of a tile's points of one slot
+    double* scratch;
+};
+
+// The sums of one slot: sum x_j x_(j + t mod d) for t = 0 .. d / 2 (every unordered pair of
+// features once, lane j), sum x_j, and the count.  ES doubles per (slice, slot).
+__host__ __device__ inline int na_entries(int d) { return (d / 2 + 2) * d + 1; }
+
+// Pass 1: block (s, g) sums the points of slot s = 2k + h among the tiles of slice g, each
+// warp in tiles of its own.  A warp scans four tiles' labels by ballots (every slot's block
+// reads them: 5 bytes a point from L2) and then takes its slot's own rows one after another,
+// so X crosses DRAM once: lane j holds x_j, and its partners x_(j + t) come from the row
+// staged in shared memory, eight rows being loaded while eight are added up.
+// What bounds it is the precision: a tile's points of one slot are summed in FP32 (point q
+// in group q mod W), and the groups' sums are added to about 48 bits.  In FP64 that is one
+// conversion and one add per entry and group on a pipe of two lanes an SM (2.3 ms at
+// d = 32, N = 1e6); as an FP32 pair it is six FP32 adds and one more.  A pair that
+// overflows or meets an infinity or NaN makes the block start over in FP64.
+// Measured at d = 32, K = 16, N = 1e6: 0.29 ms (fmaheavy pipe about 70% busy); 0.46 ms as 4 x 4 register blocks over staged
+// tiles (290 million instructions, half of them loops over tiles of four points); 21.4 ms for
+// 32 blocks that took a tile's 32 slots in turn, two block barriers each.
+template <int T, typename Acc>  // T: odd, at least d / 2 + 1
+__device__ __forceinline__ bool na_block(const NaArgs& a, float* row, int* list, double* red) {
+    constexpr int NP = (T + 1) / 2;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int d = a.d, S = 2 * a.K, s = blockIdx.x, g = blockIdx.y, W = a.W;
+    Acc acc[NP];  // t = 2 p and 2 p + 1; the last one's second: sum x_j
+#pragma unroll
+    for (int p = 0; p < NP; ++p) acc[p].zero();
+    unsigned long long count = 0;
+    const int wm = 65536 / W + 1;  // n * wm >> 16 = n / W for 0 <= n <= 128, W <= 256
+    const int64_t R = (a.N + NA_RANGES - 1) / NA_RANGES;
+    const unsigned Tr = (unsigned)((R + NA_P - 1) / NA_P), tiles = NA_RANGES * Tr;  // tiles per range, in all
+    const unsigned per = (tiles + a.G - 1) / a.G, ta = g * per, tb = min(tiles, ta + per);
+    const int64_t base = (int64_t)(ta / Tr) * R + (ta % Tr) * NA_P;  // the slice's first point
+    const float* Xb = a.X + base * d + (lane < d ? lane : 0);
+    float* mine = row + lane;
+    const bool again = lane < d && lane <= d / 2;  // x_j is x_(j + d) of the wrapped row
+    for (unsigned t0 = ta + NA_Q * warp; t0 < tb; t0 += NA_Q * NA_W) {
+        int zi[NA_Q][NA_P / 32], hi[NA_Q][NA_P / 32], off[NA_Q];
+#pragma unroll
+        for (int u = 0; u < NA_Q; ++u) {
+            const unsigned t = t0 + u, r = t / Tr;
+            const int64_t i0 = (int64_t)r * R + (int64_t)(t % Tr) * NA_P;
+            const int64_t i1 = t < tb ? min(min(a.N, (int64_t)(r + 1) * R), i0 + NA_P) : 0;
+            off[u] = (int)(i0 - base);
+#pragma unroll
+            for (int q = 0; q < NA_P / 32; ++q) {
+                const int64_t i = i0 + 32 * q + lane;
+                zi[u][q] = i < i1 ? __ldg(a.z + i) : -1;
+                hi[u][q] = i < i1 ? (int)__ldg(a.zbar + i) : 2;
+            }
+        }
+        // the slot's points of the four tiles, group by group; the sign bit marks a group's first
+        int n = 0;
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < NA_Q; ++u) {
+            unsigned m[NA_P / 32];
+            int nu = 0;
+#pragma unroll
+            for (int q = 0; q < NA_P / 32; ++q) {  // labels outside [0, K) x {0, 1} match no slot
+                m[q] = __ballot_sync(0xffffffffu, zi[u][q] == (s >> 1) && hi[u][q] == (s & 1));
+                nu += __popc(m[q]);
+            }
+            const int nq = nu * wm >> 16, nr = nu - nq * W;
+            int r0 = 0;
+#pragma unroll
+            for (int q = 0; q < NA_P / 32; ++q) {
+                if ((m[q] >> lane) & 1u) {
+                    const int r = r0 + __popc(m[q] & ((1u << lane) - 1u));
+                    const int k = r * wm >> 16, gr = r - k * W;  // r / W and r mod W
+                    list[n + gr * nq + min(gr, nr) + k] = (off[u] + 32 * q + lane) | (k == 0 ? 0x80000000 : 0);
+                }
+                r0 += __popc(m[q]);
+            }
+            n += nu;
+        }
+        count += n;
+        __syncwarp();
+        float x[NA_D];
+        auto fetch = [&](int q0) {
+#pragma unroll
+            for (int q = 0; q < NA_D; ++q)
+                x[q] = q0 + q < n ? __ldg(Xb + (int64_t)(list[q0 + q] & 0x7fffffff) * d) : 0.f;
+        };
+        fetch(0);
+        f2 f[NP];
+#pragma unroll
+        for (int p = 0; p < NP; ++p) f[p] = 0ull;
+        for (int q0 = 0; q0 < n; q0 += NA_D) {
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < NA_D; ++q) {
+                if (lane < d) mine[q * NA_ROW] = x[q];
+                if (again) mine[q * NA_ROW + d] = x[q];
+            }
+            __syncwarp();
+            if (q0 + NA_D < n) fetch(q0 + NA_D);
+            for (int q = 0; q < min(NA_D, n - q0); ++q) {
+                const float* v = mine + q * NA_ROW;
+                f2 pr[NP];
+#pragma unroll
+                for (int p = 0; p < NP; ++p) pr[p] = f2_pack(v[2 * p], p + 1 < NP ? v[2 * p + 1] : 1.f);
+                const f2 xj = f2_pack(v[0], v[0]);
+                if (list[q0 + q] < 0) {  // a new group: the last one's sums are complete
+#pragma unroll
+                    for (int p = 0; p < NP; ++p) {
+                        acc[p].add(f[p]);
+                        f[p] = f2_mul(xj, pr[p]);
+                    }
+                } else {
+#pragma unroll
+                    for (int p = 0; p < NP; ++p) f[p] = f2_fma(xj, pr[p], f[p]);
+                }
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < NP; ++p) acc[p].add(f[p]);
+    }
+    bool bad = false;
+#pragma unroll
+    for (int p = 0; p < NP; ++p) bad = bad || acc[p].bad();
+    if (__syncthreads_or(lane < d && bad)) return false;
+    // the warps' sums in warp order: red[warp][t][j], then the counts
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        const double2 v = acc[p].value();
+        red[(warp * (T + 1) + 2 * p) * 32 + lane] = v.x;
+        red[(warp * (T + 1) + 2 * p + 1) * 32 + lane] = v.y;
+    }
+    double* cnt = red + NA_W * (T + 1) * 32;
+    if (lane == 0) cnt[warp] = (double)count;
+    __syncthreads();
+    const int ES = na_entries(d), ns = d / 2 + 1;
+    double* out = a.scratch + ((size_t)g * S + s) * ES;
+    for (int e = threadIdx.x; e < ES; e += 32 * NA_W) {
+        const int t = e / d, j = e % d;
+        double v = 0.0;
+        for (int w = 0; w < NA_W; ++w)
+            v += e == ES - 1 ? cnt[w] : red[(w * (T + 1) + (t < ns ? t : T)) * 32 + j];
+        out[e] = v;
+    }
+    return true;
+}
+
+template <int T>
+__global__ void __launch_bounds__(32 * NA_W, 2) na_partial_kernel(NaArgs a) {
+    constexpr int LIST = NA_Q * NA_P, RED = NA_W * (T + 1) * 32 + NA_W;
+    constexpr size_t BYTES = (size_t)NA_W * (LIST * 4 + NA_D * NA_ROW * 4);
+    __shared__ __align__(16) unsigned char sm[BYTES > RED * 8 ? BYTES : RED * 8];
+    int* list = (int*)sm + (threadIdx.x >> 5) * LIST;
+    float* row = (float*)((int*)sm + NA_W * LIST) + (threadIdx.x >> 5) * (NA_D * NA_ROW);
+    for (int e = threadIdx.x & 31; e < NA_D * NA_ROW; e += 32) row[e] = 0.f;  // what no feature fills
+    __syncwarp();
+    if (na_block<T, NaPair>(a, row, list, (double*)sm)) return;
+    for (int e = threadIdx.x & 31; e < NA_D * NA_ROW; e += 32) row[e] = 0.f;
+    __syncthreads();
+    na_block<T, NaDouble>(a, row, list, (double*)sm);
+}
+
+// Pass 2: the slices' sums of 32 entries of slot s, eight partial sums each (slice g in
+// partial sum g mod 8, added in order: deterministic), unpacked to n, sum x, sum x x^T.
+__global__ void __launch_bounds__(256) na_combine_kernel(int d, int G, int K, const double* scratch, double* n_out,
+                                                         double* sx_out, double* sxx_out) {
+    __shared__ double part[8][32];
+    const int s = blockIdx.x, S = 2 * K, ES = na_entries(d);
+    const int e = blockIdx.y * 32 + (threadIdx.x & 31), p = threadIdx.x >> 5;
+    double v = 0.0;
+    if (e < ES)
+        for (int g = p; g < G; g += 8) v += scratch[((size_t)g * S + s) * ES + e];
+    part[p][threadIdx.x & 31] = v;
+    __syncthreads();
+    if (p != 0 || e >= ES) return;
+    v = 0.0;
+    for (int q = 0; q < 8; ++q) v += part[q][threadIdx.x];
+    const int t = e / d, j = e % d;
+    if (e == ES - 1) {
+        n_out[s] = v;
+    } else if (t > d / 2) {
+        sx_out[(size_t)s * d + j] = v;
+    } else if (2 * t < d || j < t) {  // t = d / 2 meets every pair twice
+        const int l = (j + t) % d;
+        sxx_out[((size_t)s * d + j) * d + l] = v;
+        sxx_out[((size_t)s * d + l) * d + j] = v;
+    }
 }
 
 // The scratch address is looked up (cudaGetSymbolAddress) once per device and per
@@ -179,19 +341,36 @@ extern "C" dpmm_status dpmm_suffstats_noalloc(const float* X, int64_t N, int d, 
         }
         scratch = (double*)g_na_cache[dev].ptr;
     }
+    cudaStream_t s = (cudaStream_t)stream;
+    // slices: about eight blocks per SM over the 2K slots (two are resident at a time, and a
+    // large cluster's blocks take longer than a small one's), as the scratch allows (39 at
+    // d = 32, K = 16), each of at least 32 tiles, one scan of every warp
+    const int ES = na_entries(d);
+    const int64_t tiles = (N + NA_P - 1) / NA_P;
+    const int64_t want = (1216 + 2 * K - 1) / (2 * K), fit = (int64_t)(NA_SCRATCH / ((size_t)2 * K * ES));
+    NaArgs a;
+    a.X = X;
+    a.N = N;
+    a.d = d;
+    a.z = z;
+    a.zbar = zbar;
+    a.K = K;
+    a.G = (int)std::max<int64_t>(1, std::min(std::min(want, fit), (tiles + NA_Q * NA_W - 1) / (NA_Q * NA_W)));
+    // as many FP32 groups as 256 threads hold 4 x 4 register blocks of the padded triangle
     StatLayout L;
     L.init(d, STAT_FULL);
-    cudaStream_t s = (cudaStream_t)stream;
-    int G = NA_G;
+    a.W = std::max(1, 256 / L.nblk);
+    a.scratch = scratch;
     // launched with cudaLaunchKernel, whose return value is this launch's own error (an
     // error left behind by an unrelated earlier launch is neither reported nor cleared)
-    void* a1[] = {(void*)&X, (void*)&N, (void*)&d, (void*)&z, (void*)&zbar, (void*)&K, (void*)&L, (void*)&G,
-                  (void*)&scratch};
-    if (cudaLaunchKernel((const void*)na_partial_kernel, dim3(NA_G), dim3(256), a1, 0, s) != cudaSuccess)
-        return DPMM_ECUDA;
+    const void* fn = d <= 4 ? (const void*)na_partial_kernel<3>
+                   : d <= 8 ? (const void*)na_partial_kernel<5>
+                   : d <= 16 ? (const void*)na_partial_kernel<9> : (const void*)na_partial_kernel<17>;
+    void* a1[] = {(void*)&a};
+    if (cudaLaunchKernel(fn, dim3(2 * K, a.G), dim3(32 * NA_W), a1, 0, s) != cudaSuccess) return DPMM_ECUDA;
     const double* cs = scratch;
-    void* a2[] = {(void*)&L, (void*)&G, (void*)&K, (void*)&cs, (void*)&n_out, (void*)&sx_out, (void*)&sxx_out};
-    if (cudaLaunchKernel((const void*)na_combine_kernel, dim3(2 * K), dim3(128), a2, 0, s) != cudaSuccess)
+    void* a2[] = {(void*)&d, (void*)&a.G, (void*)&K, (void*)&cs, (void*)&n_out, (void*)&sx_out, (void*)&sxx_out};
+    if (cudaLaunchKernel((const void*)na_combine_kernel, dim3(2 * K, (ES + 31) / 32), dim3(256), a2, 0, s) != cudaSuccess)
         return DPMM_ECUDA;
     return DPMM_OK;
 }
