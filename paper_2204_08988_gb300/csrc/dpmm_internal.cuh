@@ -266,7 +266,8 @@ struct dpmm_ctx {
     double *p_logw = nullptr, *p_mu = nullptr, *p_W = nullptr, *p_logdetW = nullptr, *p_c = nullptr,
            *p_logtheta = nullptr;
     float *q_mu = nullptr, *q_W = nullptr, *q_c = nullptr, *q_b = nullptr, *q_logtheta = nullptr;
-    double* p_b = nullptr;   // b = mu^T W per slot (FP64, TF32-rounded W on the TF32 path)
+    // FP64 path: q_mu is mu - mu of slot 0, q_b the norms of W's columns, q_c that of q_mu
+    double* p_b = nullptr;   // b = mu^T W per slot (TF32 path: FP64 sums, TF32-rounded W)
     void* tc_img = nullptr;  // tensor-core operand image of the cluster parameters
     size_t tc_img_bytes = 0;
     void* tcs_img = nullptr;  // tensor-core sub-cluster factor images (K_max x 10 KB)
@@ -283,6 +284,7 @@ struct dpmm_ctx {
     int* hist = nullptr;     // K_max x T_tiles
     int* tot = nullptr;      // K_max + 1: totals, then starts
     int* idx = nullptr;      // N: points sorted by cluster
+    bool sorted = false;     // idx holds a permutation of the points (a sort has run on these data)
     int G2 = 0;              // most ranges of the sub-label/statistics step (records capacity)
     int Gr = 1;              // ranges used for the current data: about one per 512 points, at most G2
     double* records = nullptr;  // (G2 + K_max) x 2 x E

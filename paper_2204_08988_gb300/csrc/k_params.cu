@@ -496,7 +496,7 @@ __global__ void dirichlet_norm_f32_kernel(int d, const int* dK, const double* lo
 
 // FP32 mirrors of the drawn parameters for the reduced-precision paths, and the
 // shift the next statistics are accumulated with (the cluster's drawn mean).
-__global__ void derive_kernel(int kind, int d, int tf32, const int* dK, const double* p_logw, const double* p_mu,
+__global__ void derive_kernel(int kind, int d, int tf32, int fp64, const int* dK, const double* p_logw, const double* p_mu,
                               const double* p_W, const double* p_c, const double* p_logtheta, float* q_mu,
                               float* q_W, float* q_c, float* q_b, double* p_b, float* q_logtheta, double* shift_new,
                               float* shift32) {
@@ -521,18 +521,30 @@ __global__ void derive_kernel(int kind, int d, int tf32, const int* dK, const do
             }
         }
         for (int j = tid; j < d; j += nt) {
-            q_mu[(size_t)s * d + j] = (float)mu[j];
+            if (fp64) {  // for the FP32 enclosures of the FP64 label step: mu - mu_0 and ||W_j||
+                q_mu[(size_t)s * d + j] = (float)(mu[j] - p_mu[j]);
+                float n2 = 0.f;
+#pragma unroll 8
+                for (int l = 0; l < d; ++l) {
+                    const float w = (float)W[l * d + j];
+                    if (l <= j) n2 = fmaf(w, w, n2);
+                }
+                q_b[(size_t)s * d + j] = sqrtf(n2);
+            } else {
+                q_mu[(size_t)s * d + j] = (float)mu[j];
+            }
             // b_j = sum_l mu_l W_lj (l <= j: W is upper triangular), with W as the tensor
             // cores see it, in the order l = 0, 1, ...; a fixed trip count lets the loads of
             // several rows be in flight at once (the FMA chain is the only serial part)
-            double b = 0.0;
+            if (tf32) {
+                double b = 0.0;
 #pragma unroll 8
-            for (int l = 0; l < d; ++l) {
-                const double w = W[l * d + j], m = mu[l];
-                if (l <= j) b = fma(m, tf32 ? (double)round_tf32((float)w) : w, b);
+                for (int l = 0; l < d; ++l) {
+                    const double w = W[l * d + j], m = mu[l];
+                    if (l <= j) b = fma(m, (double)round_tf32((float)w), b);
+                }
+                p_b[(size_t)s * d + j] = b;  // read by the tensor-core image builds
             }
-            q_b[(size_t)s * d + j] = (float)b;
-            p_b[(size_t)s * d + j] = b;  // read by the tensor-core image builds
             if (s % 3 == 0) {
                 shift_new[(size_t)(s / 3) * d + j] = (double)(float)mu[j];
                 shift32[(size_t)(s / 3) * d + j] = (float)mu[j];
@@ -542,7 +554,16 @@ __global__ void derive_kernel(int kind, int d, int tf32, const int* dK, const do
         const int j0 = blockIdx.y * 4096, j1 = min(d, j0 + 4096);
         for (int j = j0 + tid; j < j1; j += nt) q_logtheta[(size_t)s * d + j] = (float)p_logtheta[(size_t)s * d + j];
     }
-    if (tid == 0 && blockIdx.y == 0) q_c[s] = (float)p_c[s];
+    if (tid == 0 && blockIdx.y == 0 && !fp64) q_c[s] = (float)p_c[s];
+    if (fp64 && kind == DPMM_PRIOR_NIW && tid < 32) {  // ||mu - mu_0||
+        float n2 = 0.f;
+        for (int j = tid; j < d; j += 32) {
+            const float m = (float)(p_mu[(size_t)s * d + j] - p_mu[j]);
+            n2 = fmaf(m, m, n2);
+        }
+        for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+        if (tid == 0) q_c[s] = sqrtf(n2);
+    }
 }
 
 static StatView make_sv(dpmm_ctx* c) { return StatView{c->stats, c->st}; }
@@ -633,7 +654,7 @@ cudaError_t launch_params(dpmm_ctx* c, uint64_t seed) {
 cudaError_t launch_derive(dpmm_ctx* c) {
     prof_begin(c, "derive");
     const dim3 dgrid(3 * c->K_max, c->kind == DPMM_PRIOR_NIW ? 1 : (c->d + 4095) / 4096);
-    derive_kernel<<<dgrid, 128, 0, c->stream>>>(c->kind, c->d, c->prec == DPMM_PREC_TF32, c->dK, c->p_logw, c->p_mu, c->p_W, c->p_c,
+    derive_kernel<<<dgrid, 128, 0, c->stream>>>(c->kind, c->d, c->prec == DPMM_PREC_TF32, c->prec == DPMM_PREC_FP64_PLAIN, c->dK, c->p_logw, c->p_mu, c->p_W, c->p_c,
                                                        c->p_logtheta, c->q_mu, c->q_W, c->q_c, c->q_b, c->p_b,
                                                        c->q_logtheta, c->shift_new, c->shift32);
     prof_end(c, "derive");

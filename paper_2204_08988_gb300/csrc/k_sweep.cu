@@ -25,6 +25,15 @@ __device__ inline T ldx(const XT* p) { return (T)(*p); }
 template <>
 __device__ inline float ldx<float, __nv_bfloat16>(const __nv_bfloat16* p) { return __bfloat162float(*p); }
 
+__device__ __forceinline__ void mw_cp16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
 template <typename T>
 struct ParamView {
     const T* W;      // slots x d x d
@@ -131,6 +140,507 @@ __global__ void __launch_bounds__(256) labels_simt_kernel(int kind, int d, int x
         }
     }
     if (live) z[i] = zb;
+    }
+}
+
+// An FP64 Gumbel value to within GUMBEL_APPROX, in FP32 arithmetic: e = -log u from u, or
+// from 1 - u (exact in the 53-bit integer) when u is above 1/2, to a few FP32 roundings, so
+// log e is off by about 4e-7 and, for |log e| <= 37, its own rounding by 4e-6.
+constexpr double GUMBEL_APPROX = 1e-4;
+__device__ inline float gumbel_approx(uint32_t a, uint32_t b) {
+    const unsigned long long m = 2ull * (((unsigned long long)(a >> 6) << 26) | (b >> 6)) + 1ull;
+    const float s = 1.1102230246251565e-16f;  // 2^-53
+    const float e = m < (1ull << 52) ? -logf((float)m * s) : -log1pf(-(float)((1ull << 53) - m) * s);
+    return -logf(e);
+}
+
+template <typename T>
+__device__ inline T gmin();  // below every Gumbel value of the precision
+template <>
+__device__ inline double gmin<double>() { return -3.7; }
+template <>
+__device__ inline float gmin<float>() { return -3.f; }
+
+// ------------------------------------------------------------------ Gaussian labels, small d
+// z_i = argmax_k [s_ik + G_ik] for d <= 16 (FP32) or d <= 8 (FP64).  The sums are short there,
+// and what bounds the step is the chain of latencies of one point's K clusters; so L lanes share
+// a point (clusters sub, sub + L, ...), as many as the points leave room for.  All clusters'
+// parameters are staged in shared memory once per block, rows and columns padded with zeros
+// to DV (a zero adds nothing to a sum).  A first pass finds the two best scores: if the second
+// cannot win whatever the Gumbel values (monotone rounding makes the bounds hold for the
+// rounded sums), the label is known.  Otherwise the clusters within reach of the best score
+// are drawn; in FP64 by an FP32 value first (gumbel_approx), FP64 logarithms being taken for
+// those it cannot tell apart.
+// Measured: FP64, d = 2, K = 10, N = 10,000: 27 us, from 62 us with one thread per point
+// and FP64 draws; FP32, d = 8, K = 12, N = 100,003: 25 us, from 35 us.
+template <typename T, int DV, int L>
+__global__ void __launch_bounds__(256) labels_small_kernel(int d, int xs, int64_t N, const T* __restrict__ X,
+                                                           ParamView<T> pv, const int* dK, const uint32_t* diter,
+                                                           uint64_t seed, int32_t* z) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    constexpr int PER = DV * DV + DV + 1;  // W, mu, c; odd: lanes of different clusters use different banks
+    T* sp = (T*)smraw;
+    const int K = *dK, tid = threadIdx.x, sub = tid % L;
+    for (int e = tid; e < K * PER; e += 256) {
+        const int k = e / PER, r = e % PER;
+        const size_t s = 3 * (size_t)k;
+        T v = 0;
+        if (r < DV * DV) {
+            const int l = r / DV, j = r % DV;
+            if (l <= j && j < d) v = pv.W[s * d * d + l * d + j];
+        } else if (r < DV * DV + DV) {
+            if (r - DV * DV < d) v = pv.mu[s * d + (r - DV * DV)];
+        } else {
+            v = pv.c[s];
+        }
+        sp[e] = v;
+    }
+    __syncthreads();
+    const Key key{seed, diter[0], diter[1], diter[2]};
+    const int64_t step = (int64_t)gridDim.x * (256 / L);
+    for (int64_t i0 = (int64_t)blockIdx.x * (256 / L) + (tid & ~31) / L; i0 < N; i0 += step) {  // uniform in a warp
+        const int64_t ir = i0 + (tid & 31) / L;
+        const bool live = ir < N;
+        const int64_t i = live ? ir : N - 1;
+        T x[DV];
+#pragma unroll
+        for (int j = 0; j < DV; ++j) x[j] = j < d ? X[i * xs + j] : (T)0;
+        auto score = [&](int k) -> T {
+            const T* P = sp + k * PER;
+            T q = 0;
+            T t[DV];
+#pragma unroll
+            for (int j = 0; j < DV; ++j) t[j] = x[j] - P[DV * DV + j];
+#pragma unroll
+            for (int j = 0; j < DV; ++j) {
+                T y = 0;
+#pragma unroll
+                for (int l = 0; l <= j; ++l) y = fma(P[l * DV + j], t[l], y);
+                q = fma(y, y, q);
+            }
+            return P[PER - 1] - (T)0.5 * q;
+        };
+        T best = -INFINITY, second = -INFINITY;
+        int kb = 0;
+        for (int k = sub; k < K; k += L) {
+            const T s = score(k);
+            if (s > best) {
+                second = best;
+                best = s;
+                kb = k;
+            } else if (s > second) {
+                second = s;
+            }
+        }
+#pragma unroll
+        for (int o = 1; o < L; o <<= 1) {
+            const T ob = __shfl_xor_sync(0xffffffffu, best, o), os = __shfl_xor_sync(0xffffffffu, second, o);
+            const int ok = __shfl_xor_sync(0xffffffffu, kb, o);
+            second = max(min(best, ob), max(second, os));
+            if (ob > best || (ob == best && ok < kb)) {
+                best = ob;
+                kb = ok;
+            }
+        }
+        const T reach = best + gmin<T>();
+        const bool need = second > -INFINITY && !(second + gmax<T>() < reach);
+        if (__any_sync(0xffffffffu, need)) {
+            T vb = -INFINITY, vs = -INFINITY;  // the best value and the runner-up
+            int kv = 0;
+            uint32_t w[4];
+            auto words = [&](int k) { key.block((uint32_t)i, TAG_Z, (uint32_t)(k >> 1), w); };
+            if (need)
+                for (int k = sub; k < K; k += L) {
+                    const T s = score(k);
+                    if (!(s > -INFINITY) || s + gmax<T>() < reach) continue;
+                    words(k);
+                    T v;
+                    if constexpr (sizeof(T) == 8) v = s + (T)((k & 1) ? gumbel_approx(w[2], w[3]) : gumbel_approx(w[0], w[1]));
+                    else v = s + ((k & 1) ? gumbel_of<T>(w[2], w[3]) : gumbel_of<T>(w[0], w[1]));
+                    if (v > vb) {
+                        vs = vb;
+                        vb = v;
+                        kv = k;
+                    } else if (v > vs) {
+                        vs = v;
+                    }
+                }
+            auto reduce = [&]() {
+#pragma unroll
+                for (int o = 1; o < L; o <<= 1) {
+                    const T ob = __shfl_xor_sync(0xffffffffu, vb, o), os = __shfl_xor_sync(0xffffffffu, vs, o);
+                    const int ok = __shfl_xor_sync(0xffffffffu, kv, o);
+                    vs = max(min(vb, ob), max(vs, os));
+                    if (ob > vb || (ob == vb && ok < kv)) {
+                        vb = ob;
+                        kv = ok;
+                    }
+                }
+            };
+            reduce();
+            if constexpr (sizeof(T) == 8) {
+                const T cut = vb - 4 * GUMBEL_APPROX;
+                const bool near = need && vs >= cut;
+                if (__any_sync(0xffffffffu, near)) {
+                    const int keep = kv;
+                    vb = vs = -INFINITY;
+                    if (near)
+                        for (int k = sub; k < K; k += L) {
+                            const T s = score(k);
+                            if (!(s > -INFINITY) || s + gmax<T>() < reach) continue;
+                            words(k);
+                            if (s + (T)((k & 1) ? gumbel_approx(w[2], w[3]) : gumbel_approx(w[0], w[1])) < cut) continue;
+                            const T v = s + ((k & 1) ? gumbel_of<T>(w[2], w[3]) : gumbel_of<T>(w[0], w[1]));
+                            if (v > vb) {
+                                vb = v;
+                                kv = k;
+                            }
+                        }
+                    reduce();
+                    if (!near) kv = keep;
+                }
+            }
+            if (need) kb = kv;
+        }
+        if (live && sub == 0) z[i] = kb;
+    }
+}
+
+// ------------------------------------------------------------------ Gaussian labels in FP64
+// z_i = argmax_k [s_ik + G_ik], s_ik = c_k - 1/2 ||W_k^T (x_i - mu_k)||^2, one thread per
+// point.  What bounds the step is the FP64 pipe (two lanes an SM): scoring every cluster
+// takes K d^2 / 2 FP64 multiply-adds a point and two FP64 logarithms a draw.  So every
+// score is first enclosed in FP32, [L_ik, U_ik] with the bounds derived below, and a cluster
+// whose U + (largest Gumbel value) is below the best L + (smallest) is left out: it cannot
+// win whatever is drawn.  If one cluster is left, it is the label.  Otherwise the ones left
+// are scored in FP64, their Gumbel values are enclosed in FP32 (gumbel_approx), and FP64
+// logarithms are taken for those that this cannot tell apart.  The labels are those of
+// scoring and drawing everything in FP64.
+// The points are taken in the order of the last counting sort, so that a warp's points
+// mostly have the cluster they had in common; it is enclosed first.  Of every other cluster
+// the last eight columns are tried first (W is upper triangular: column j is x_j given
+// x_0 .. x_j-1, on the tightest scale where j is largest), staged in shared memory one
+// cluster ahead; the few clusters that they leave standing are enclosed in full.
+// Measured at d = 32, K = 20, N = 30,001: 217 us; 1518 us for every score and draw in FP64
+// (with x - mu formed anew for every entry of W), 650 us with FP64 partial sums instead of
+// FP32 enclosures (a warp goes on until all of its 32 points have left the cluster), 225 us
+// with the clusters read from global memory where they are used (one latency after another).
+//
+// Enclosure: with x' = x - mu_0 and mu'_k = mu_k - mu_0 (formed in FP64, rounded to FP32,
+// mu_0 the first cluster's mean: the data need not be centred), t = x' - mu' and the column
+// sum y = sum_l W_l t_l in FP32, y is off by at most (d + 8) 2^-24 sum_l |W_l| (|x'_l| +
+// |mu'_l|): one rounding each of W, x', mu', t, and d + 1 of the sum.  By Cauchy-Schwarz
+// that is at most e = (d + 8) 2^-24 ||W_j|| (||x'|| + ||mu'||), the norms rounded up by 1%.  The
+// rounding of x' and mu' in FP64, 2^-53 (|x| + |mu_0|), enters as 2^-26 (|x_l| + |mu_0l|) added
+// to |x'_l|.  Sums of squares of at most 144 terms are off by 144 x 2^-24 < 1e-5 relative.
+constexpr int NIW_C = 8;  // contenders a thread holds
+constexpr int NIW_B = 8;  // columns at a time
+constexpr int NIW_P = 8;  // clusters a thread puts off
+
+struct Niw64 {
+    int d, xs;
+    int64_t N;
+    const double *X, *W, *mu, *c;  // FP64 data and parameters (slots 3k)
+    const float *qW, *qmu, *qn, *qc;  // FP32: W, mu - mu_0, the norms of W's columns and of mu - mu_0
+    const int* idx;                // order of the points, or null
+    const int* dK;
+    const uint32_t* diter;
+    uint64_t seed;
+    const int* gate;
+    int32_t* z;
+};
+
+// Dynamic shared memory, a column per thread (row stride blockDim + 1): d floats x', d floats
+// t, d doubles x - mu; then the contenders: NIW_C doubles (scores) and, each of blockDim,
+// NIW_C floats U, NIW_C ints, NIW_P shorts; then, per warp, two stages of NIW_B d + d floats (a cluster's
+// last columns of W, mu - mu_0).
+template <bool VEC>  // VEC: d is a multiple of 4, rows of the FP32 W are 16-byte aligned
+__global__ void __launch_bounds__(128) labels_niw64_kernel(Niw64 a) {
+    if (a.gate && *a.gate == 0) return;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int K = *a.dK, d = a.d, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, ld = nt + 1;
+    double* sd = (double*)smraw + tid;                    // x - mu of the cluster in hand, FP64
+    double* csc = (double*)smraw + (size_t)d * ld + tid;  // contenders' FP64 scores
+    float* sx = (float*)((double*)smraw + (size_t)d * ld + NIW_C * nt);
+    float* st = sx + (size_t)d * ld + tid;
+    float* cu = sx + (size_t)2 * d * ld + tid;            // contenders' U, then approximate values
+    int* ck = (int*)(cu - tid + NIW_C * nt) + tid;
+    const int sz = (NIW_B + 1) * d, jl = (d - 1) / NIW_B * NIW_B, wl = d - jl;  // stage, last block of columns
+    short* pend = (short*)(ck - tid + NIW_C * nt) + tid;
+    float* stg = (float*)(pend - tid + NIW_P * nt) + (tid >> 5) * 2 * ((sz + 3) & ~3);
+    auto stage = [&](int k, int b) {  // rows of NIW_B floats, then mu; one group of copies
+        const float* W = a.qW + (size_t)(3 * k) * d * d + jl;
+        const float* mu = a.qmu + (size_t)(3 * k) * d;
+        float* to = stg + b * ((sz + 3) & ~3);
+        if constexpr (VEC) {
+            const int n4 = wl >> 2;  // wl is 4 or 8
+            for (int e = lane; e < d * n4; e += 32) {
+                const int l = n4 == 2 ? e >> 1 : e, u = n4 == 2 ? (e & 1) * 4 : 0;
+                mw_cp16(to + l * NIW_B + u, W + (size_t)l * d + u);
+            }
+            for (int e = lane; e < d >> 2; e += 32) mw_cp16(to + d * NIW_B + 4 * e, mu + 4 * e);
+        } else {
+            for (int e = lane; e < d * wl; e += 32) cp_async4(to + e / wl * NIW_B + e % wl, W + (size_t)(e / wl) * d + e % wl);
+            for (int e = lane; e < d; e += 32) cp_async4(to + d * NIW_B + e, mu + e);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int e = lane; e < 2 * ((sz + 3) & ~3); e += 32) stg[e] = 0.f;  // the columns beyond d
+    __syncwarp();
+    const Key key{a.seed, a.diter[0], a.diter[1], a.diter[2]};
+    const float gam = (float)(d + 8) * 6.0e-8f * 1.02f;  // 2^-24 = 5.96e-8; the norms' 1%
+    const int64_t ntiles = (a.N + nt - 1) / nt;
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int64_t p = tile * nt + tid;
+        const bool live = p < a.N;  // the rest of the last block repeats the last point
+        const int64_t pc = live ? p : a.N - 1, i = a.idx ? (int64_t)a.idx[pc] : pc;
+        const int zi = a.z[i];
+        float nx = 0.f;  // ||x'||, with the FP64 rounding's share
+        __syncwarp();    // a warp stages its own 32 points, four rows at a time
+        for (int r0 = 0; r0 < 32; r0 += 4) {
+            int64_t ir[4];
+            float n2[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) ir[u] = __shfl_sync(0xffffffffu, i, r0 + u);
+            for (int l = lane; l < d; l += 32) {
+                double v[4];
+                const double m0 = a.mu[l];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = a.X[ir[u] * a.xs + l];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const float x = (float)(v[u] - m0), w = fabsf(x) + 1.5e-8f * (fabsf((float)v[u]) + fabsf((float)m0));
+                    sx[l * ld + (tid & ~31) + r0 + u] = x;
+                    n2[u] = fmaf(w, w, n2[u]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                for (int o = 16; o > 0; o >>= 1) n2[u] += __shfl_xor_sync(0xffffffffu, n2[u], o);
+                if (lane == r0 + u) nx = sqrtf(n2[u]);
+            }
+        }
+        __syncwarp();
+        const float* x = sx + tid;
+        const double* xr = a.X + i * a.xs;
+        float low = -INFINITY;  // a cluster below this value cannot win
+        double vb = -INFINITY;  // the best value drawn so far, and its cluster
+        int kb = 0, nc = 0;
+        bool drawn = false, sure = true;
+        // FP64 score of cluster k
+        auto score = [&](int k) -> double {
+            const double* W = a.W + (size_t)(3 * k) * d * d;
+            const double* mu = a.mu + (size_t)(3 * k) * d;
+            double q = 0.0;
+            for (int j = 0; j < d; j += 2) {  // two chains at once; each adds l = 0, 1, ... in order
+                const bool two = j + 1 < d;
+                sd[j * ld] = xr[j] - __ldg(mu + j);
+                if (two) sd[(j + 1) * ld] = xr[j + 1] - __ldg(mu + j + 1);
+                const double* Wa = W + j;
+                const double* Wb = W + (two ? j + 1 : j);
+                double ya = 0.0, yb = 0.0;
+#pragma unroll 8
+                for (int l = 0; l <= j; ++l) {
+                    const double t = sd[l * ld];
+                    ya = fma(__ldg(Wa + l * d), t, ya);
+                    yb = fma(__ldg(Wb + l * d), t, yb);
+                }
+                q = fma(ya, ya, q);
+                if (two) {
+                    yb = fma(__ldg(Wb + (j + 1) * d), sd[(j + 1) * ld], yb);
+                    q = fma(yb, yb, q);
+                }
+            }
+            return __ldg(a.c + 3 * k) - 0.5 * q;
+        };
+        // the contenders' FP64 values against the best one drawn (ties to the lower index)
+        auto draw_all = [&]() {
+            for (int e = 0; e < nc; ++e) {
+                const int k = ck[e * nt];
+                uint32_t w[4];
+                key.block((uint32_t)i, TAG_Z, (uint32_t)(k >> 1), w);
+                const double v = csc[e * nt] + ((k & 1) ? gumbel_of<double>(w[2], w[3]) : gumbel_of<double>(w[0], w[1]));
+                if (v > vb || (v == vb && drawn && k < kb)) {
+                    vb = v;
+                    kb = k;
+                    drawn = true;
+                }
+            }
+            nc = 0;
+        };
+        auto purge = [&]() {  // contenders that later bounds have ruled out
+            int m = 0;
+            for (int e = 0; e < nc; ++e) {
+                if (cu[e * nt] + 37.5f < low) continue;
+                cu[m * nt] = cu[e * nt];
+                ck[m * nt] = ck[e * nt];
+                ++m;
+            }
+            nc = m;
+        };
+        auto score_all = [&]() {  // FP64 scores of the contenders; those without a value are dropped
+            int m = 0;
+            for (int e = 0; e < nc; ++e) {
+                const int k = ck[e * nt];
+                const double sc = score(k);
+                if (!(sc > -INFINITY)) continue;
+                csc[m * nt] = sc;
+                ck[m * nt] = k;
+                ++m;
+            }
+            nc = m;
+        };
+        auto bound = [&](float c) {  // a sum of squares above it leaves cluster k (weight and determinant c) out
+            return 2.f * (c + 37.5f - low + 1e-3f + 1e-6f * fabsf(c)) * 1.00002f + 1e-2f;
+        };
+        auto square = [&](float y, float e, float& qlo, float& qhi) {
+            const float h = fabsf(y) + e, g = fmaxf(fabsf(y) - e, 0.f);
+            qlo = fmaf(g, g, qlo);
+            qhi = fmaf(h, h, qhi);
+        };
+        auto admit = [&](int k, float c, float qlo, float qhi) {
+            const float slack = 1e-3f + 1e-6f * fabsf(c);
+            const float U = c - 0.5f * (qlo * 0.99998f) + slack;
+            float L = c - 0.5f * (qhi * 1.00002f) - slack;
+            if (!(U > -INFINITY) || U + 37.5f < low) return;
+            if (!(fabsf(L) < INFINITY)) {  // nothing known: FP64 decides
+                L = -INFINITY;
+                sure = false;
+            }
+            if (nc == NIW_C) {
+                purge();
+                if (nc == NIW_C) {
+                    score_all();
+                    draw_all();
+                    if (drawn) low = fmaxf(low, (float)vb - 1e-3f - 1e-6f * fabsf((float)vb));
+                }
+            }
+            cu[nc * nt] = U;
+            ck[nc * nt] = k;
+            ++nc;
+            low = fmaxf(low, L - 3.7f);
+        };
+        auto enclose = [&](int k) {  // every column
+            const float* W = a.qW + (size_t)(3 * k) * d * d;
+            const float* mu = a.qmu + (size_t)(3 * k) * d;
+            const float* qn = a.qn + (size_t)(3 * k) * d;
+            const float c = (float)__ldg(a.c + 3 * k), thr = bound(c);
+#pragma unroll 8
+            for (int l = 0; l < d; ++l) st[l * ld] = x[l * ld] - __ldg(mu + l);
+            const float ga = gam * (nx + __ldg(a.qc + 3 * k));
+            float qlo = 0.f, qhi = 0.f;
+            for (int j0 = jl; j0 >= 0; j0 -= NIW_B) {
+                float y[NIW_B];
+#pragma unroll
+                for (int u = 0; u < NIW_B; ++u) y[u] = 0.f;
+                const int le = min(d, j0 + NIW_B);
+#pragma unroll 8
+                for (int l = 0; l < le; ++l) {
+                    const float t = st[l * ld];
+                    float w[NIW_B];
+                    if constexpr (VEC) {
+#pragma unroll
+                        for (int u = 0; u < NIW_B; u += 4) {
+                            const float4 v = j0 + u < d ? __ldg((const float4*)(W + l * d + j0 + u)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                            w[u] = v.x;
+                            w[u + 1] = v.y;
+                            w[u + 2] = v.z;
+                            w[u + 3] = v.w;
+                        }
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < NIW_B; ++u) w[u] = j0 + u < d ? __ldg(W + l * d + j0 + u) : 0.f;
+                    }
+#pragma unroll
+                    for (int u = 0; u < NIW_B; ++u) y[u] = fmaf(l <= j0 + u ? w[u] : 0.f, t, y[u]);
+                }
+#pragma unroll
+                for (int u = 0; u < NIW_B; ++u)
+                    if (j0 + u < d) square(y[u], ga * __ldg(qn + j0 + u), qlo, qhi);
+                if (qlo > thr) return;
+            }
+            admit(k, c, qlo, qhi);
+        };
+        const int hint = zi >= 0 && zi < K ? zi : 0;
+        int np = 1;
+        pend[0] = (short)hint;
+        stage(0, 0);
+        // clusters put off are enclosed in full with the lanes' own ones side by side: the
+        // point's own first of all, the others when a thread holds no more, and at the end
+        for (int k = -1; k <= K; ++k) {
+            if (k < 0 || k == K || np == NIW_P)
+                while (np > 0) enclose(pend[--np * nt]);
+            if (k < 0 || k == K) continue;
+            const float c = (float)__ldg(a.c + 3 * k), mn = __ldg(a.qc + 3 * k);
+            float en[NIW_B];
+#pragma unroll
+            for (int u = 0; u < NIW_B; ++u) en[u] = u < wl ? __ldg(a.qn + (size_t)(3 * k) * d + jl + u) : 0.f;
+            if (k + 1 < K) {
+                stage(k + 1, (k + 1) & 1);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+            __syncwarp();
+            const float* Wl = stg + (k & 1) * ((sz + 3) & ~3);
+            const float* ml = Wl + d * NIW_B;
+            float y[NIW_B];
+#pragma unroll
+            for (int u = 0; u < NIW_B; ++u) y[u] = 0.f;
+#pragma unroll 8
+            for (int l = 0; l < jl; ++l) {
+                const float t = x[l * ld] - ml[l];
+                const float4 w0 = *(const float4*)(Wl + l * NIW_B), w1 = *(const float4*)(Wl + l * NIW_B + 4);
+                y[0] = fmaf(w0.x, t, y[0]);
+                y[1] = fmaf(w0.y, t, y[1]);
+                y[2] = fmaf(w0.z, t, y[2]);
+                y[3] = fmaf(w0.w, t, y[3]);
+                y[4] = fmaf(w1.x, t, y[4]);
+                y[5] = fmaf(w1.y, t, y[5]);
+                y[6] = fmaf(w1.z, t, y[6]);
+                y[7] = fmaf(w1.w, t, y[7]);
+            }
+#pragma unroll
+            for (int v = 0; v < NIW_B; ++v)
+                if (v < wl) {
+                    const float t = x[(jl + v) * ld] - ml[jl + v];
+#pragma unroll
+                    for (int u = v; u < NIW_B; ++u) y[u] = fmaf(Wl[(jl + v) * NIW_B + u], t, y[u]);
+                }
+            const float ga = gam * (nx + mn);
+            float qlo = 0.f, qhi = 0.f;
+#pragma unroll
+            for (int u = 0; u < NIW_B; ++u)
+                if (u < wl) square(y[u], ga * en[u], qlo, qhi);
+            if (k != hint && !(qlo > bound(c))) pend[np++ * nt] = (short)k;
+            __syncwarp();  // the stage is filled again
+        }
+        purge();
+        if (nc == 1 && !drawn && sure) {
+            kb = ck[0];
+        } else if (nc > 0) {
+            score_all();
+            double vmax = vb;
+            for (int e = 0; e < nc; ++e) {
+                const int k = ck[e * nt];
+                uint32_t w[4];
+                key.block((uint32_t)i, TAG_Z, (uint32_t)(k >> 1), w);
+                const float g = (k & 1) ? gumbel_approx(w[2], w[3]) : gumbel_approx(w[0], w[1]);
+                cu[e * nt] = g;
+                vmax = fmax(vmax, csc[e * nt] + (double)g);
+            }
+            int m = 0;  // the contenders that the approximation cannot tell from the best
+            for (int e = 0; e < nc; ++e)
+                if (csc[e * nt] + (double)cu[e * nt] >= vmax - 4 * GUMBEL_APPROX) {
+                    csc[m * nt] = csc[e * nt];
+                    ck[m * nt] = ck[e * nt];
+                    ++m;
+                }
+            nc = m;
+            if (nc == 1 && !(drawn && vb >= vmax - 4 * GUMBEL_APPROX)) kb = ck[0];
+            else draw_all();
+        }
+        if (live) a.z[i] = kb;
     }
 }
 
@@ -387,7 +897,7 @@ __global__ void __launch_bounds__(MAXT) substats_kernel(SubArgs<T> a) {
                 all += (double)red[((size_t)gg * nblk + b) * 32 + q];
                 rr += (double)red[((size_t)gg * nblk + b) * 32 + 16 + q];
             }
-            out[b * 16 + q] = all - rr;       // sub-cluster l
+            out[b * 16 + q] = all;            // sub-cluster l
             out[a.L.E + b * 16 + q] = rr;     // sub-cluster r
         }
 #pragma unroll
@@ -406,9 +916,14 @@ __global__ void __launch_bounds__(MAXT) substats_kernel(SubArgs<T> a) {
             if (a.draw) {
                 uint32_t w[4];
                 key.block((uint32_t)i, TAG_ZBAR, 0, w);
-                T vl = sub_score<T, XT>(a, 3 * k + 1, xr) + gumbel_of<T>(w[0], w[1]);
-                T vr = sub_score<T, XT>(a, 3 * k + 2, xr) + gumbel_of<T>(w[2], w[3]);
-                h = vr > vl ? 1 : 0;
+                const T sl = sub_score<T, XT>(a, 3 * k + 1, xr), sr = sub_score<T, XT>(a, 3 * k + 2, xr);
+                bool near = true;  // FP64: an FP32 Gumbel difference decides where it can
+                if constexpr (sizeof(T) == 8) {
+                    const T diff = (sr - sl) + (T)(gumbel_approx(w[2], w[3]) - gumbel_approx(w[0], w[1]));
+                    near = !(fabs(diff) > 4 * GUMBEL_APPROX);
+                    h = diff > 0 ? 1 : 0;
+                }
+                if (near) h = sr + gumbel_of<T>(w[2], w[3]) > sl + gumbel_of<T>(w[0], w[1]) ? 1 : 0;
                 a.zbar[i] = (uint8_t)h;
             } else {
                 h = a.zbar[i];
@@ -442,15 +957,250 @@ __global__ void __launch_bounds__(MAXT) substats_kernel(SubArgs<T> a) {
                         xj[u] = xr[jb * 4 + u];
                         xl[u] = xr[lb * 4 + u];
                     }
-                    const T hm = hq[q] ? (T)1 : (T)0;
+                    if (hq[q]) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+#pragma unroll
+                            for (int v = 0; v < 4; ++v) accr[u * 4 + v] = fma(xj[u], xl[v], accr[u * 4 + v]);
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+#pragma unroll
+                            for (int v = 0; v < 4; ++v) acc[u * 4 + v] = fma(xj[u], xl[v], acc[u * 4 + v]);
+                    }
+                }
+            }
+        }
+    }
+    if (cur >= 0) flush(cur);
+}
+
+// Gaussian FP64 sub-labels and statistics.  What bounds the step is the FP64 pipe (two lanes
+// an SM): the two sub-cluster scores take d^2 FP64 multiply-adds a point, the sums d^2 / 2.
+// So the scores are enclosed in FP32 first, as in labels_niw64_kernel (the bounds are derived
+// there), and so are the two Gumbel values; only the points whose sub-label these enclosures
+// leave open are scored in FP64, a warp to each (lane j takes column j, adding l = 0, 1, ... in
+// order), so that the sub-labels are those of scoring every point in FP64.  The sums are FP64.
+// Measured at d = 32, K = 20, N = 30,001: 107 us per step; 250 us with every score in FP64,
+// 759 us so and in 59 ranges of 512 points, on 59 of 152 SMs.
+// Dynamic shared memory: P x dp doubles (rows), P floats (norms), P x 4 floats (enclosures),
+// P ints (k), P + 2 ints (runs), P + 1 ints (points left open), P bytes (h), then d x (P + 1)
+// floats (x - mu_0 by coordinate), later the flush buffer G x nblk x 32 doubles.
+struct Sub64 {
+    SubArgs<double> a;
+    const float *qW, *qmu, *qn, *qc;  // FP32: W, mu - mu_0, the norms of W's columns and of mu - mu_0
+};
+
+__host__ __device__ inline size_t sub64_head(int P, int dp) {
+    return ((size_t)P * dp * 8 + (size_t)P * 20 + (size_t)(3 * P + 3) * 4 + P + 15) / 16 * 16;
+}
+
+template <int MAXT>
+__global__ void __launch_bounds__(MAXT) substats_niw64_kernel(Sub64 b) {
+    const SubArgs<double>& a = b.a;
+    if (a.gate && *a.gate == 0) return;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int d = a.d, dp = a.L.dp, P = a.P, G = a.G, nblk = a.L.nblk;
+    double* xs = (double*)smraw;
+    float* nrm = (float*)(xs + (size_t)P * dp);
+    float* enc = nrm + P;        // lower and upper bound of each sub-cluster's score
+    int* kq = (int*)(enc + 4 * P);
+    int* runs = kq + P;          // run starts, P + 1
+    int* nruns = runs + P + 1;
+    int* open = nruns + 1;       // points whose sub-label FP64 decides; the count at P
+    unsigned char* hq = (unsigned char*)(open + P + 1);
+    double* red = (double*)(smraw + sub64_head(P, dp));
+    float* xf = (float*)red;     // used before any flush of the same batch
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+    const int g = blockIdx.x, ldf = P + 1;
+    const int64_t p0 = (int64_t)g * a.R, p1 = min(a.N, p0 + a.R);
+    const Key key{a.seed, a.diter[0], a.diter[1], a.diter[2]};
+    const double* X = (const double*)a.X;
+    const float gam = (float)(d + 8) * 6.0e-8f * 1.02f;
+    __shared__ int wcnt[32];
+
+    const bool worker = tid < nblk * G;
+    const int myblk = worker ? tid % nblk : 0, grp = worker ? tid / nblk : 0;
+    int jb = 0, lb = 0;
+    a.L.blk_coords(myblk, jb, lb);
+    double acc[16], accr[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) acc[e] = accr[e] = 0.0;
+    int cur = -1;
+
+    auto flush = [&](int k) {
+        __syncthreads();
+        if (worker) {
+            double* r = red + ((size_t)grp * nblk + myblk) * 32;
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                r[e] = acc[e];
+                r[16 + e] = accr[e];
+            }
+        }
+        __syncthreads();
+        double* out = a.rec + (size_t)(g + k) * 2 * a.L.E;
+        for (int e = tid; e < nblk * 16; e += nt) {
+            const int bl = e >> 4, q = e & 15;
+            double sl = 0.0, sr = 0.0;
+            for (int gg = 0; gg < G; ++gg) {
+                sl += red[((size_t)gg * nblk + bl) * 32 + q];
+                sr += red[((size_t)gg * nblk + bl) * 32 + 16 + q];
+            }
+            out[bl * 16 + q] = sl;
+            out[a.L.E + bl * 16 + q] = sr;
+        }
+#pragma unroll
+        for (int e = 0; e < 16; ++e) acc[e] = accr[e] = 0.0;
+    };
+
+    for (int64_t base = p0; base < p1; base += P) {
+        const int np = (int)min((int64_t)P, p1 - base);
+        __syncthreads();
+        for (int r = warp; r < np; r += nt >> 5) {  // one warp per row
+            const int i = a.idx[base + r];
+            float n2 = 0.f;
+            for (int l = lane; l < d; l += 32) {
+                const double v = X[(int64_t)i * a.xs + l];
+                xs[(size_t)r * dp + l] = v;
+                if (a.draw) {
+                    const double m0 = a.pv.mu[l];
+                    const float x = (float)(v - m0), w = fabsf(x) + 1.5e-8f * (fabsf((float)v) + fabsf((float)m0));
+                    xf[l * ldf + r] = x;
+                    n2 = fmaf(w, w, n2);
+                }
+            }
+            if (a.draw) {
+                for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+                if (lane == 0) nrm[r] = sqrtf(n2);
+            }
+            if (lane == 0) kq[r] = a.z[i];
+        }
+        if (tid == 0) open[P] = 0;
+        __syncthreads();
+        if (a.draw) {
+            for (int it = tid; it < 2 * np; it += nt) {  // enclosure of sub-cluster h's score of point p
+                const int h = it >= np, p = it - (h ? np : 0), s = 3 * kq[p] + 1 + h;
+                const float* W = b.qW + (size_t)s * d * d;
+                const float* mu = b.qmu + (size_t)s * d;
+                const float* qn = b.qn + (size_t)s * d;
+                const float ga = gam * (nrm[p] + __ldg(b.qc + s));
+                const float* x = xf + p;
+                float qlo = 0.f, qhi = 0.f;
+                for (int j0 = 0; j0 < d; j0 += 4) {
+                    float y[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+                    for (int l = 0; l < min(d, j0 + 4); ++l) {
+                        const float t = x[l * ldf] - __ldg(mu + l);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            y[u] = fmaf(l <= j0 + u && j0 + u < d ? __ldg(W + l * d + j0 + u) : 0.f, t, y[u]);
+                    }
 #pragma unroll
                     for (int u = 0; u < 4; ++u)
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) {
-                            T pr = xj[u] * xl[v];
-                            acc[u * 4 + v] += pr;
-                            accr[u * 4 + v] += hm * pr;
+                        if (j0 + u < d) {
+                            const float e = ga * __ldg(qn + j0 + u), hi = fabsf(y[u]) + e, lo = fmaxf(fabsf(y[u]) - e, 0.f);
+                            qlo = fmaf(lo, lo, qlo);
+                            qhi = fmaf(hi, hi, qhi);
                         }
+                }
+                const float c = (float)__ldg(a.pv.c + s), slack = 1e-3f + 1e-6f * fabsf(c);
+                enc[4 * p + 2 * h] = c - 0.5f * (qhi * 1.00002f) - slack;
+                enc[4 * p + 2 * h + 1] = c - 0.5f * (qlo * 0.99998f) + slack;
+            }
+            __syncthreads();
+        }
+        for (int p = tid; p < np; p += nt) {
+            const int i = a.idx[base + p];
+            int h = 0;
+            if (a.draw) {
+                uint32_t w[4];
+                key.block((uint32_t)i, TAG_ZBAR, 0, w);
+                const float dg = gumbel_approx(w[2], w[3]) - gumbel_approx(w[0], w[1]);
+                const float lo = enc[4 * p + 2] - enc[4 * p + 1] + dg, hi = enc[4 * p + 3] - enc[4 * p] + dg;
+                const float m = 1e-3f + 1e-6f * (fabsf(enc[4 * p]) + fabsf(enc[4 * p + 2]));  // the sums' own rounding
+                if (lo > m) h = 1;
+                else if (hi < -m) h = 0;
+                else open[atomicAdd(&open[P], 1)] = p;
+                a.zbar[i] = (uint8_t)h;
+            } else {
+                h = a.zbar[i];
+            }
+            hq[p] = (unsigned char)h;
+        }
+        __syncthreads();
+        if (a.draw) {
+            const int no = open[P];
+            for (int o = warp; o < no; o += nt >> 5) {
+                const int p = open[o], k = kq[p], i = a.idx[base + p];
+                const double* x = xs + (size_t)p * dp;
+                const double* W0 = a.pv.W + (size_t)(3 * k + 1) * d * d;
+                const double* m0 = a.pv.mu + (size_t)(3 * k + 1) * d;
+                double q0 = 0.0, q1 = 0.0;
+                for (int j0 = 0; j0 < d; j0 += 32) {
+                    const int j = min(j0 + lane, d - 1);
+                    double y0 = 0.0, y1 = 0.0;
+                    for (int l = 0; l < min(d, j0 + 32); ++l) {
+                        const double t0 = x[l] - __ldg(m0 + l), t1 = x[l] - __ldg(m0 + d + l);
+                        if (l <= j) {
+                            y0 = fma(__ldg(W0 + l * d + j), t0, y0);
+                            y1 = fma(__ldg(W0 + (size_t)d * d + l * d + j), t1, y1);
+                        }
+                    }
+                    for (int u = 0; u < min(32, d - j0); ++u) {
+                        const double v0 = __shfl_sync(0xffffffffu, y0, u), v1 = __shfl_sync(0xffffffffu, y1, u);
+                        q0 = fma(v0, v0, q0);
+                        q1 = fma(v1, v1, q1);
+                    }
+                }
+                if (lane == 0) {
+                    uint32_t w[4];
+                    key.block((uint32_t)i, TAG_ZBAR, 0, w);
+                    const double sl = a.pv.c[3 * k + 1] - 0.5 * q0, sr = a.pv.c[3 * k + 2] - 0.5 * q1;
+                    const double diff = (sr - sl) + (double)(gumbel_approx(w[2], w[3]) - gumbel_approx(w[0], w[1]));
+                    int h = diff > 0 ? 1 : 0;
+                    if (!(fabs(diff) > 4 * GUMBEL_APPROX))
+                        h = sr + gumbel_of<double>(w[2], w[3]) > sl + gumbel_of<double>(w[0], w[1]) ? 1 : 0;
+                    a.zbar[i] = (uint8_t)h;
+                    hq[p] = (unsigned char)h;
+                }
+            }
+            __syncthreads();  // the rows are still read above
+        }
+        for (int e = tid; e < np * dp; e += nt) {  // the row less the cluster's centre, then 1, then zeros
+            const int p = e / dp, j = e % dp;
+            xs[e] = j < d ? xs[e] - a.shift[(size_t)kq[p] * d + j] : (j == d ? 1.0 : 0.0);
+        }
+        __syncthreads();
+        find_runs(kq, np, runs, nruns, wcnt);
+        const int nr = *nruns;
+        for (int r = 0; r < nr; ++r) {
+            const int qs = runs[r], qe = runs[r + 1];
+            const int k = kq[qs];
+            if (k != cur) {
+                if (cur >= 0) flush(cur);
+                cur = k;
+            }
+            if (worker) {
+                for (int q = qs + grp; q < qe; q += G) {
+                    const double* xr = xs + (size_t)q * dp;
+                    double xj[4], xl[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        xj[u] = xr[jb * 4 + u];
+                        xl[u] = xr[lb * 4 + u];
+                    }
+                    if (hq[q]) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+#pragma unroll
+                            for (int v = 0; v < 4; ++v) accr[u * 4 + v] = fma(xj[u], xl[v], accr[u * 4 + v]);
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+#pragma unroll
+                            for (int v = 0; v < 4; ++v) acc[u * 4 + v] = fma(xj[u], xl[v], acc[u * 4 + v]);
+                    }
                 }
             }
         }
@@ -1095,11 +1845,6 @@ struct MwArgs {
 constexpr int MW_DEPTH = 16;  // rows in flight per warp (a ring in shared memory)
 constexpr int MW_ROWB = 512;  // bytes per ring slot: d <= 256 BF16 counts
 
-__device__ __forceinline__ void mw_cp16(void* dst, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-
 // BF16 counts (rows 16-byte aligned).  Dynamic shared memory: 8 warps x MW_DEPTH x MW_ROWB.
 __global__ void __launch_bounds__(256, 3) mult_warp_kernel(MwArgs a) {
     if (a.gate && *a.gate == 0) return;
@@ -1341,11 +2086,63 @@ static cudaError_t labels_simt_t(dpmm_ctx* c, uint64_t seed, const int* gate) {
     return cudaGetLastError();
 }
 
+// Gaussian FP64 labels without the score hook.  Blocks of 32 to 128 points: the most that
+// still give every SM two blocks.
+static cudaError_t labels_niw64(dpmm_ctx* c, uint64_t seed, const int* gate) {
+    const int d = c->d;
+    const size_t per = ((size_t)d * d + d + 1) * sizeof(double);  // d too large for labels_simt_kernel: refused here too
+    if ((size_t)32 * (d + 1) * sizeof(double) + per > 200 * 1024) return cudaErrorInvalidValue;
+    const size_t stg = (((NIW_B + 1) * (size_t)d + 3) & ~(size_t)3) * 2 * 4;  // per warp
+    auto bytes = [&](int TB) { return (size_t)d * (TB + 1) * 16 + 16 + (size_t)NIW_C * TB * 16 + (size_t)NIW_P * TB * 2 + (size_t)(TB / 32) * stg; };
+    int TB = 128;
+    while (TB > 32 && (bytes(TB) > 100 * 1024 || c->N < (int64_t)TB * 2 * c->num_sms)) TB /= 2;
+    auto kern = d % 4 == 0 ? labels_niw64_kernel<true> : labels_niw64_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(TB));
+    if (e != cudaSuccess) return e;
+    const int64_t tiles = (c->N + TB - 1) / TB;
+    const int grid = (int)(gate ? std::min<int64_t>(tiles, (int64_t)c->num_sms) : tiles);
+    Niw64 a{d, c->xs, c->N, (const double*)c->X, c->p_W, c->p_mu, c->p_c, c->q_W, c->q_mu, c->q_b,
+            c->q_c, c->sorted ? c->idx : nullptr, c->dK, c->diter, seed, gate, c->z};
+    kern<<<grid, TB, bytes(TB), c->stream>>>(a);
+    return cudaGetLastError();
+}
+
+// labels_small_kernel where it applies: every cluster's padded parameters in 100 KB
+template <typename T, int DV>
+static cudaError_t labels_small_t(dpmm_ctx* c, uint64_t seed) {
+    const size_t smem = (size_t)c->K_max * (DV * DV + DV + 1) * sizeof(T);
+    const int64_t room = 2048 * (int64_t)c->num_sms;  // resident threads
+    const int L = c->N * 8 <= room ? 8 : c->N * 4 <= room ? 4 : c->N * 2 <= room ? 2 : 1;
+    auto kern = L == 8 ? labels_small_kernel<T, DV, 8> : L == 4 ? labels_small_kernel<T, DV, 4>
+              : L == 2 ? labels_small_kernel<T, DV, 2> : labels_small_kernel<T, DV, 1>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const int64_t blocks = (c->N * L + 255) / 256;
+    kern<<<(int)std::min<int64_t>(blocks, 8 * (int64_t)c->num_sms), 256, smem, c->stream>>>(
+        c->d, c->xs, c->N, (const T*)c->X, pview<T>(c), c->dK, c->diter, seed, c->z);
+    return cudaGetLastError();
+}
+
+static bool labels_small(const dpmm_ctx* c) {
+    const bool f64 = c->prec == DPMM_PREC_FP64_PLAIN;
+    const int DV = c->d <= 2 ? 2 : c->d <= 4 ? 4 : c->d <= 8 ? 8 : 16;
+    return c->kind == DPMM_PRIOR_NIW && c->d <= (f64 ? 8 : 16) && !c->dbg_scores &&
+           (size_t)c->K_max * (DV * DV + DV + 1) * (f64 ? 8 : 4) <= 100 * 1024;
+}
+
 cudaError_t launch_labels_simt_gated(dpmm_ctx* c, uint64_t seed, const int* gate) {
     const char* name = gate ? "labels_simt_overflow" : "labels_simt";
     prof_begin(c, name);
     cudaError_t e;
-    if (c->prec == DPMM_PREC_FP64_PLAIN) e = labels_simt_t<double, double>(c, seed, gate);
+    if (!gate && labels_small(c)) {
+        if (c->prec == DPMM_PREC_FP64_PLAIN)
+            e = c->d <= 2 ? labels_small_t<double, 2>(c, seed) : c->d <= 4 ? labels_small_t<double, 4>(c, seed)
+                                                               : labels_small_t<double, 8>(c, seed);
+        else
+            e = c->d <= 2 ? labels_small_t<float, 2>(c, seed) : c->d <= 4 ? labels_small_t<float, 4>(c, seed)
+              : c->d <= 8 ? labels_small_t<float, 8>(c, seed) : labels_small_t<float, 16>(c, seed);
+    } else if (c->kind == DPMM_PRIOR_NIW && c->prec == DPMM_PREC_FP64_PLAIN && !c->dbg_scores) e = labels_niw64(c, seed, gate);
+    else if (c->prec == DPMM_PREC_FP64_PLAIN) e = labels_simt_t<double, double>(c, seed, gate);
     else if (c->xdt == 2) e = labels_simt_t<float, __nv_bfloat16>(c, seed, gate);
     else e = labels_simt_t<float, float>(c, seed, gate);
     prof_end(c, name);
@@ -1365,6 +2162,7 @@ static cudaError_t sort_impl(dpmm_ctx* c, const int* gate) {
                                                                                gate, c->K_max, c->idx);
     prof_end(c, "sort");
     c->nlaunch += 3;
+    if (!gate) c->sorted = true;
     return cudaGetLastError();
 }
 
@@ -1383,7 +2181,10 @@ static SubCfg sub_cfg(const dpmm_ctx* c) {
     BT = std::min(1024, std::max(256, (BT + 31) / 32 * 32));
     q.P = P;
     q.BT = BT;
-    q.G = std::max(1, BT / L.nblk);
+    // groups of points per register block; every run's end adds the groups up one after
+    // another in FP64 (64 cycles each), so no more than 16 (d = 2: one block, 256 groups,
+    // took 105 us per statistics step at N = 10,000; 16 groups 19 us)
+    q.G = std::max(1, std::min(16, BT / L.nblk));
     size_t head = (size_t)P * L.dp * sizeof(T) + (2 * (size_t)P + 2) * sizeof(int) + P;
     head = (head + 15) / 16 * 16;
     q.smem = head + (size_t)q.G * L.nblk * 32 * sizeof(T);
@@ -1442,6 +2243,42 @@ static cudaError_t substats_t(dpmm_ctx* c, uint64_t seed, int draw, const int* g
         if (ea != cudaSuccess) return ea;
         substats_kernel<T, XT, 1024><<<c->Gr, q.BT, q.smem, c->stream>>>(a);
     }
+    return cudaGetLastError();
+}
+
+static cudaError_t substats_niw64(dpmm_ctx* c, uint64_t seed, int draw, const int* gate) {
+    SubCfg q = sub_cfg<double>(c);
+    Sub64 b;
+    SubArgs<double>& a = b.a;
+    a.kind = c->kind;
+    a.d = c->d;
+    a.xs = c->xs;
+    a.N = c->N;
+    a.X = c->X;
+    a.pv = pview<double>(c);
+    a.shift = c->shift_new;
+    a.z = c->z;
+    a.zbar = c->zbar;
+    a.idx = c->idx;
+    a.dK = c->dK;
+    a.diter = c->diter;
+    a.gate = gate;
+    a.seed = seed;
+    a.draw = draw;
+    a.P = std::min(128, q.P);  // find_runs takes a thread per point; two blocks per SM at d = 32
+    a.G = q.G;
+    a.R = (c->N + c->Gr - 1) / c->Gr;
+    a.L = c->st;
+    a.rec = c->records;
+    b.qW = c->q_W;
+    b.qmu = c->q_mu;
+    b.qn = c->q_b;
+    b.qc = c->q_c;
+    const size_t smem = sub64_head(a.P, a.L.dp) + std::max((size_t)q.G * a.L.nblk * 32 * 8, (size_t)c->d * (a.P + 1) * 4);
+    auto kern = q.BT <= 256 ? substats_niw64_kernel<256> : substats_niw64_kernel<1024>;
+    cudaError_t ea = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (ea != cudaSuccess) return ea;
+    kern<<<c->Gr, q.BT, smem, c->stream>>>(b);
     return cudaGetLastError();
 }
 
@@ -1619,6 +2456,7 @@ static cudaError_t substats_dispatch(dpmm_ctx* c, uint64_t seed, int draw, const
                                    : substats_f32_t<64, float>(c, seed, draw, gate);
     else if (c->prec != DPMM_PREC_FP64_PLAIN && c->kind == DPMM_PRIOR_NIW && c->d <= 128 && c->st.nblk <= WIDE_T)
         e = c->xdt == 2 ? substats_wide_t<__nv_bfloat16>(c, seed, draw, gate) : substats_wide_t<float>(c, seed, draw, gate);
+    else if (c->prec == DPMM_PREC_FP64_PLAIN && c->kind == DPMM_PRIOR_NIW && c->d > 8) e = substats_niw64(c, seed, draw, gate);
     else if (c->prec == DPMM_PREC_FP64_PLAIN) e = substats_t<double, double>(c, seed, draw, gate);
     else if (c->xdt == 2) e = substats_t<float, __nv_bfloat16>(c, seed, draw, gate);
     else e = substats_t<float, float>(c, seed, draw, gate);
