@@ -447,6 +447,10 @@ dpmm_status dpmm_create(const dpmm_prior* prior, double alpha, int d, int K_max,
     }
     A(&c->Ltab, sizeof(double) * (3 * (size_t)K_max + 3 * ((size_t)K_max * (K_max - 1) / 2) + 1 + 6 * (size_t)K_max));
     A(&c->relabel, sizeof(int) * 4 * K_max);
+    if (c->kind == DPMM_PRIOR_NIW) {
+        A(&c->sm_T, sizeof(float) * (size_t)K_max * d * d);
+        A(&c->sm_xbar, sizeof(double) * (size_t)K_max * (d + 1));
+    }
     A(&c->acc, sizeof(int) * ((size_t)K_max + (size_t)K_max * (K_max - 1) / 2 + 1));
     A(&c->center, sizeof(double) * (2 * (size_t)d + (size_t)d * d));
     if (!ok) {
@@ -477,7 +481,7 @@ void dpmm_destroy(dpmm_ctx* c) {
     void* ps[] = {c->dK, c->diter, c->age, c->counters, c->derr, c->stats, c->shift_new, c->shift_stats,
                   c->shift32, c->p_logw, c->p_mu, c->p_W, c->p_logdetW, c->p_c, c->p_logtheta, c->q_mu,
                   c->q_W, c->q_c, c->q_b, c->q_logtheta, c->cweights, c->tot, c->records, c->Ltab,
-                  c->relabel, c->acc, c->center, c->tc_img, c->tcs_img, c->tc_flag, c->dbg_scores, c->eps, c->bart, c->lgs, c->retry, c->x3_fimg,
+                  c->relabel, c->acc, c->sm_T, c->sm_xbar, c->center, c->tc_img, c->tcs_img, c->tc_flag, c->dbg_scores, c->eps, c->bart, c->lgs, c->retry, c->x3_fimg,
                   c->sp_cc, c->sp_ltT, c->sp_ct, c->sp_lgt, c->sp_lgb, c->sp_part, c->shard_scratch, c->p_b, c->mcnt,
                   c->stage};
     if (c->cstream) cudaStreamSynchronize(c->cstream);

@@ -296,7 +296,8 @@ struct dpmm_ctx {
                              // pair lgamma(n) and lgamma(alpha + n) (K_max (K_max - 1))
     int* relabel = nullptr;  // 4 K_max
     int* acc = nullptr;      // K_max + K_max (K_max - 1)/2 accept flags of the split/merge proposals
-    double* canon = nullptr; // canonical (n, xbar, C) per cluster and sub-cluster: 3 K_max x (1 + d + d d)
+    float* sm_T = nullptr;     // NIW: K_max x d x d, Psi0 / 2 + scatter of every cluster (FP32)
+    double* sm_xbar = nullptr; // NIW: K_max x d cluster means, then K_max log determinants of sm_T
 
     // tensor-core path
     int* tc_flag = nullptr;        // device: 1 when K did not fit the tensor-core kernel

@@ -217,9 +217,14 @@ struct NiwPrior {
 // factorisation loses more than 10 bits of a pivot to cancellation (or meets a
 // non-positive one) is flagged in retry[] and redone by the FP64 instantiation
 // (launched with retry set, it takes only the flagged slots).
-// Dynamic shared memory: (E doubles when staged) + (d*ld + 11*d (+ d*d when W fits)) T.
+// Psi_n (lower triangle, with the diagonal) and W (upper triangle, with the diagonal) share one
+// array of rows of ld T: W's entry (r, c) sits at column c + 1, so that W is in shared memory in
+// FP64 too up to d = 156 (d = 128, 192 slots: 1,526 us; 1,725 us with W in global memory).
+// Dynamic shared memory: (E doubles when staged) + (d*ld + 12*d) T.
 __device__ inline float log_t(float x) { return logf(x); }
 __device__ inline double log_t(double x) { return log(x); }
+
+__host__ __device__ inline int niw_ld(int d) { return (d + 1) | 1; }
 
 template <typename T>
 __global__ void niw_params_kernel(StatView sv, const double* shift_stats, NiwPrior pr, const int* dK,
@@ -234,7 +239,7 @@ __global__ void niw_params_kernel(StatView sv, const double* shift_stats, NiwPri
     const bool retry_pass = sizeof(T) == 8 && retry != nullptr;
     if (retry_pass && retry[s] == 0) return;
     const int k = s / 3, h = s % 3 - 1;  // h = -1: the cluster
-    const int ld = d | 1;         // odd row stride: column reads without bank conflicts
+    const int ld = niw_ld(d);     // odd row stride: column reads without bank conflicts
     double* S = smem;             // E: staged statistics
     T* A = (T*)(S + (staged ? E : 0));  // d x ld: Psi_n (lower), then the solve's multipliers
     T* mn = A + d * ld;           // d
@@ -246,7 +251,8 @@ __global__ void niw_params_kernel(StatView sv, const double* shift_stats, NiwPri
     T* piv = rw + d;              // d: pivots
     T* cols = piv + d;            // 4 d: the factorisation's scaled panel columns
     double* Wg = p_W + (size_t)s * d * d;
-    T* W = w_in_smem ? cols + 4 * d : (T*)Wg;  // d x d working copy (global only when T = double)
+    T* W = w_in_smem ? A + 1 : (T*)Wg;  // working copy (global only when T = double), rows of ws
+    const int ws = w_in_smem ? ld : d;
     __shared__ double sh[32];
     __shared__ double s_n, s_rn, s_kn, s_rkn;
     __shared__ int s_fail;
@@ -279,21 +285,25 @@ __global__ void niw_params_kernel(StatView sv, const double* shift_stats, NiwPri
     // xbar - m0 per coordinate (FP64), for the Psi_n build below; in the factorisation's
     // scratch columns, which it overwrites only after that build
     double* dxm = (double*)(((uintptr_t)cols + 7) & ~(uintptr_t)7);
+    double* m1 = dxm + d;  // first moments
     for (int j = tid; j < d; j += nt) {
-        const double xbar = n > 0 ? sh_k[j] + M(j, d) * rn : 0.0;
+        const double mj = M(j, d), xbar = n > 0 ? sh_k[j] + mj * rn : 0.0;
+        m1[j] = mj;
         mn[j] = (T)((pr.kappa0 * pr.m0s[j] + n * xbar) * rkn);
         dxm[j] = xbar - pr.m0s[j];
         Bd[j] = (T)bart[(size_t)s * d + j];
         acc[j] = (T)eps[(size_t)s * d + j];
     }
-    if (w_in_smem)  // the normals above the diagonal (zero below), drawn by variates_kernel
+    if (w_in_smem)  // the normals above the diagonal, drawn by variates_kernel
         for (int e0 = tid; e0 < d * d; e0 += 8 * nt) {  // eight loads in flight per thread
             double v[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) v[u] = e0 + u * nt < d * d ? Wg[e0 + u * nt] : 0.0;
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (e0 + u * nt < d * d) W[e0 + u * nt] = (T)v[u];
+            for (int u = 0; u < 8; ++u) {
+                const int r = (e0 + u * nt) / d, c = (e0 + u * nt) % d;
+                if (r < c && r < d) W[r * ws + c] = (T)v[u];
+            }
         }
     __syncthreads();
     // Psi_n = Psi0 + C + (kappa0 n / kappa_n)(xbar - m0)(xbar - m0)^T, C = S2 - S1 S1^T / n
@@ -301,21 +311,22 @@ __global__ void niw_params_kernel(StatView sv, const double* shift_stats, NiwPri
     // nothing else
     const double f = n > 0 ? pr.kappa0 * n * rkn : 0.0;
     const int ntri = d * (d + 1) / 2;
-    for (int e0 = tid; e0 < ntri; e0 += 4 * nt) {  // the Psi0 entries of four entries loaded first
+    for (int e0 = tid; e0 < ntri; e0 += 4 * nt) {  // the loads of four entries issued first
         int jj[4], ll[4];
-        double p0[4];
+        double p0[4], m2[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int e = min(e0 + u * nt, ntri - 1);
             tri_index(e, jj[u], ll[u]);  // l <= j
             p0[u] = pr.psi0[jj[u] * d + ll[u]];
+            m2[u] = M(ll[u], jj[u]);
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             if (e0 + u * nt >= ntri) break;
             const int j = jj[u], l = ll[u];
             double C = 0.0;
-            if (n > 0) C = M(l, j) - M(l, d) * M(j, d) * rn;
+            if (n > 0) C = m2[u] - m1[l] * m1[j] * rn;
             const T a = (T)(p0[u] + C + f * dxm[j] * dxm[l]);
             A[j * ld + l] = a;
             if (l == j) dg[j] = a;
@@ -340,30 +351,30 @@ __global__ void niw_params_kernel(StatView sv, const double* shift_stats, NiwPri
     }
     // U^T W = B, right-looking: after step r, row r of W (unscaled) is final and the rows
     // above are updated with it; the rows are scaled by 1 / U_rr at the end
-    for (int j = tid; j < d; j += nt) W[j * d + j] = Bd[j];
+    for (int j = tid; j < d; j += nt) W[j * ws + j] = Bd[j];
     __syncthreads();
     for (int r = d - 1; r > 0; --r) {
         const int w = d - r;  // columns c = r .. d-1
-        const T* Wr = W + (size_t)r * d;
+        const T* Wr = W + (size_t)r * ws;
         const T* Vr = A + (size_t)r * ld;
         for (int e0 = tid; e0 < r * w; e0 += 2 * nt) {
             const int e1 = e0 + nt;
             const int i0 = e0 / w, c0 = r + e0 % w;  // row i < r
             const bool two = e1 < r * w;
             const int i1 = two ? e1 / w : i0, c1 = two ? r + e1 % w : c0;
-            const T a0 = W[i0 * d + c0], v0 = Vr[i0], w0 = Wr[c0];
-            const T a1 = W[i1 * d + c1], v1 = Vr[i1], w1 = Wr[c1];
-            W[i0 * d + c0] = fma(-v0, w0, a0);
-            if (two) W[i1 * d + c1] = fma(-v1, w1, a1);
+            const T a0 = W[i0 * ws + c0], v0 = Vr[i0], w0 = Wr[c0];
+            const T a1 = W[i1 * ws + c1], v1 = Vr[i1], w1 = Wr[c1];
+            W[i0 * ws + c0] = fma(-v0, w0, a0);
+            if (two) W[i1 * ws + c1] = fma(-v1, w1, a1);
         }
         __syncthreads();
     }
     for (int e = tid; e < d * d; e += nt) {
         const int r = e / d, c = e % d;
-        if (c >= r) W[e] *= rd[r];
+        if (c >= r) W[r * ws + c] *= rd[r];
     }
     __syncthreads();
-    for (int j = tid; j < d; j += nt) rw[j] = T(1) / W[j * d + j];
+    for (int j = tid; j < d; j += nt) rw[j] = T(1) / W[j * ws + j];
     __syncthreads();
     // W^T v = eps (forward substitution) by warp 0, lane m keeps sum_{j<m} W[j][m] v_j;
     // mu = m_n + v / sqrt(kappa_n)
@@ -387,7 +398,7 @@ __global__ void niw_params_kernel(StatView sv, const double* shift_stats, NiwPri
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const int m = tid + 32 * i;
-                if (i < ns && m > j && m < d) am[i] += W[j * d + m] * vj;
+                if (i < ns && m > j && m < d) am[i] += W[j * ws + m] * vj;
             }
         }
     }
@@ -396,9 +407,12 @@ __global__ void niw_params_kernel(StatView sv, const double* shift_stats, NiwPri
     const T rsk = rsqrt_t((T)kn);
     for (int j = tid; j < d; j += nt) mu[j] = (double)(mn[j] + Bd[j] * rsk);
     if (w_in_smem)
-        for (int e = tid; e < d * d; e += nt) Wg[e] = (double)W[e];
+        for (int e = tid; e < d * d; e += nt) {  // zero below the diagonal already
+            const int r = e / d, c = e % d;
+            if (c >= r) Wg[e] = (double)W[r * ws + c];
+        }
     double lgd = 0.0;
-    for (int j = tid; j < d; j += nt) lgd += (double)log_t(W[j * d + j]);
+    for (int j = tid; j < d; j += nt) lgd += (double)log_t(W[j * ws + j]);
     lgd = block_reduce_sum(lgd, sh);
     if (tid == 0) {
         p_logdetW[s] = lgd;
@@ -589,25 +603,22 @@ cudaError_t launch_weights(dpmm_ctx* c, uint64_t seed) {
 
 cudaError_t launch_params(dpmm_ctx* c, uint64_t seed) {
     if (c->kind == DPMM_PRIOR_NIW) {
-        const size_t dd = (size_t)c->d * c->d, E = (size_t)c->st.E, dl = (size_t)c->d * (c->d | 1);
+        const size_t E = (size_t)c->st.E, dl = (size_t)c->d * niw_ld(c->d);
         NiwPrior pr{c->kappa0, c->nu0, c->center + c->d, c->center + 2 * c->d};
-        // shared memory of the T instantiation: E doubles (staged), then d*ld + 7 d (+ d*d) T
+        // shared memory of the T instantiation: E doubles (staged, while three blocks still fit an
+        // SM), then d * ld + 12 d T
         auto plan = [&](size_t tsz, int& staged, int& w_in_smem) {
-            size_t sm = tsz * (dl + 11 * (size_t)c->d);
-            staged = w_in_smem = 0;
-            if (sm + 8 * E <= 200 * 1024) {
-                sm += 8 * E;
-                staged = 1;
-            }
-            if (sm + tsz * dd <= 200 * 1024) {
-                sm += tsz * dd;
-                w_in_smem = 1;
-            }
-            return sm;
+            size_t sm = tsz * (dl + 12 * (size_t)c->d);
+            w_in_smem = sm <= 200 * 1024;
+            staged = sm + 8 * E <= 72 * 1024;
+            return sm + (staged ? 8 * E : 0);
         };
         int st64, w64, st32, w32;
         const size_t sm64 = plan(8, st64, w64), sm32 = plan(4, st32, w32);
-        const bool fp32 = c->prec != DPMM_PREC_FP64_PLAIN && w32;  // FP32 needs W in shared memory
+        // FP32 up to the d whose matrices and statistics fit 200 KB unpacked (d <= 125), FP64 above
+        const size_t base = 4 * ((size_t)c->d * (c->d | 1) + 11 * (size_t)c->d), sq = 4 * (size_t)c->d * c->d;
+        const bool fp32 = c->prec != DPMM_PREC_FP64_PLAIN && w32 &&
+                          base + (base + 8 * E <= 200 * 1024 ? 8 * E : 0) + sq <= 200 * 1024;
         cudaError_t e = cudaFuncSetAttribute(niw_params_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)sm64);
         if (e == cudaSuccess)

@@ -1,10 +1,12 @@
 // k_splitmerge.cu -- splits and merges (Sec. 4.1, Eqs. sample_splits and
 // sample_merges; Sec. 4.3 "a cluster takes part in at most one merge").
 //
-//   marginal : log f_x(C; lambda) for every cluster, sub-cluster and cluster pair,
+//   marginal : log f_x(C; lambda) for every cluster and sub-cluster (Dirichlet: and pair),
 //              FP64, one CTA per item (NIW: Cholesky log-determinant of Psi_n;
 //              Dirichlet-multinomial: lgamma sums).
-//   decision : one thread walks the proposals in the fixed order (splits by
+//   merge    : every proposal's acceptance (many Gaussian merge pairs: upper bounds of the
+//              ratio first, the pair's marginal only where they leave it open).
+//   decision : walks the proposals in the fixed order (splits by
 //              increasing k, then merge pairs in lexicographic order) with the
 //              Philox uniforms (tag SPLIT, c0 = k; tag MERGE, c0 = k1, block k2,
 //              indices after removing emptied clusters), and writes the relabel map.
@@ -34,7 +36,15 @@ struct SMArgs {
     int stage;                                  // statistics blocks staged in shared memory
     int kind, K_max;
     const int* dK;
+    float* T32;      // NIW: T_k = Psi0 / 2 + C_k of every cluster in FP32 (K_max x d x d, lower triangle)
+    double* xbar;    // K_max x d cluster means
+    double* ldT;     // K_max: log det T_k (NaN: not known)
+    int exact;       // slots and pairs up to this many: every pair is factorised in FP64 at once
 };
+// whether marginal_kernel evaluates the pairs itself (else merge_kernel bounds them)
+__device__ inline bool pairs_at_once(const SMArgs& a, int K) {
+    return a.kind == DPMM_PRIOR_DIRICHLET || 3 * K + K * (K - 1) / 2 <= a.exact;
+}
 
 __device__ inline double smv(const SMArgs& a, int k, int h, int j, int l) {
     int e = a.L.ent(j, l);
@@ -66,13 +76,18 @@ __device__ inline void pair_of(int p, int K, int& k1, int& k2) {
 
 // One item (slot or merge pair) of marginal_kernel.  Dynamic shared memory: d (d | 1) + 10 d
 // doubles (+ 2 E when the statistics are staged).
-__device__ __forceinline__ void marginal_item(const SMArgs& a, double* Ltab, int* derr, int K, int e) {
+// t >= 0: T_t = Psi0 / 2 + C_t of cluster t instead (its entries, the mean and log det T_t).
+__device__ __forceinline__ void marginal_item(const SMArgs& a, double* Ltab, int* derr, int K, int e, int t = -1) {
     extern __shared__ double smem[];
     __shared__ double sh[32];
     __shared__ double s_n, s_n1, s_n2;
     const int d = a.L.d, tid = threadIdx.x, nt = blockDim.x;
     int k1, k2, h;
-    if (e < 3 * K) {
+    if (t >= 0) {
+        k1 = t;
+        k2 = -1;
+        h = -1;
+    } else if (e < 3 * K) {
         k1 = e / 3;
         k2 = -1;
         h = e % 3 - 1;
@@ -81,7 +96,7 @@ __device__ __forceinline__ void marginal_item(const SMArgs& a, double* Ltab, int
         h = -1;
     }
     double* out = Ltab + (e < 3 * K ? e : 3 * a.K_max + (e - 3 * K));
-    if (tid == 32 || tid == 33) {  // the slot's or the pair's lgamma terms for the Hastings ratios
+    if (t < 0 && (tid == 32 || tid == 33)) {  // the slot's or the pair's lgamma terms for the Hastings ratios
         if (e < 3 * K) {
             const double ns = smv(a, k1, h, d, d);
             Ltab[lg_offset(a.K_max) + 2 * e + (tid - 32)] = lgamma(tid == 32 ? ns : 0.5 * a.alpha + ns);
@@ -185,10 +200,35 @@ __device__ __forceinline__ void marginal_item(const SMArgs& a, double* Ltab, int
                 C += M2(l, j) - M2(l, d) * M2(j, d) * r2;
                 if (n1 > 0) C += w12 * (x1[j] - x2[j]) * (x1[l] - x2[l]);
             }
-            A[q] = p0[u] + C + f * dxb[j] * dxb[l];
+            if (t >= 0) {
+                const double v = 0.5 * p0[u] + C;
+                A[q] = v;
+                a.T32[(size_t)t * d * d + j * d + l] = (float)v;
+            } else {
+                A[q] = p0[u] + C + f * dxb[j] * dxb[l];
+            }
         }
     }
+    if (t >= 0)
+        for (int j = tid; j < d; j += nt) a.xbar[(size_t)t * d + j] = xb[j];
     __syncthreads();
+    if (t >= 0) {
+        __shared__ int s_fail;
+        if (tid == 0) s_fail = 0;
+        __syncthreads();
+        chol_ldl_blk<double>(A, d, ld, piv, rs, cols, nullptr, 0.0, &s_fail, nullptr);
+        double part = 0.0;
+        for (int j = tid; j < d; j += nt) part += log(piv[j]);
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        if ((tid & 31) == 0) sh[tid >> 5] = part;
+        __syncthreads();
+        if (tid == 0) {
+            double v = 0.0;
+            for (int w = 0; w < (nt + 31) / 32; ++w) v += sh[w];
+            a.ldT[t] = s_fail ? nan("") : v;  // a factorisation that fails says nothing: the pair is factorised itself
+        }
+        return;
+    }
     chol_ldl(A, d, ld, piv, rs, cols, derr);
     // -(nun/2) log|Psi_n| and the multivariate-lgamma ratio (the prior's part from the
     // host), summed over j by all threads; lane 0 of warp 0 adds log kappa_n
@@ -206,14 +246,17 @@ __device__ __forceinline__ void marginal_item(const SMArgs& a, double* Ltab, int
     }
 }
 
-// Log marginal likelihoods of every slot (cluster and sub-clusters) and merge pair: the
-// resident blocks take the items in turn, so that no block is launched for the slots and
-// pairs beyond the current K.
+// Log marginal likelihoods of every slot (cluster and sub-clusters) and merge pair, or, for
+// Gaussian data with many pairs, T_k of every cluster, from which merge_kernel bounds the
+// pairs.  An item is a chain of FP64 latencies, so pairs that an SM can take beside the slots
+// cost nothing (47 us at d = 32 for 60 slots alone and with 190 pairs).  The resident blocks
+// take the items in turn, so that no block is launched for the slots and pairs beyond K.
 __global__ void marginal_kernel(SMArgs a, double* Ltab, int* derr) {
     const int K = *a.dK;
-    const int total = 3 * K + K * (K - 1) / 2;
+    const bool bound = !pairs_at_once(a, K);
+    const int total = 3 * K + (bound ? K : K * (K - 1) / 2);
     for (int e = blockIdx.x; e < total; e += gridDim.x) {
-        marginal_item(a, Ltab, derr, K, e);
+        marginal_item(a, Ltab, derr, K, e, bound && e >= 3 * K ? e - 3 * K : -1);
         __syncthreads();  // shared memory is reused by the next item
     }
 }
@@ -290,64 +333,7 @@ __global__ void marginal_counts_kernel(SMArgs a, Src cnt, const double* lgt, int
     }
 }
 
-// Every split and merge ratio with its Philox uniform, in parallel: acc[k] for the
-// split of cluster k, acc[K_max + p] for merge pair p; 1 = accepted if proposed.
-// Indices in the Philox counters are those after removing emptied clusters.
-constexpr int DEC_KMAX_SM = 1024;  // K_max <= 1000
-
-// One warp per block: the warp first finds which clusters hold points and their indices
-// after removing the empty ones (a prefix count in shared memory), then each lane takes a
-// proposal.
-__global__ void __launch_bounds__(32) hastings_kernel(SMArgs a, const double* Ltab, const uint32_t* diter, uint64_t seed,
-                                                      int labels_ran, int* acc) {
-    __shared__ int s_live[DEC_KMAX_SM], s_cid[DEC_KMAX_SM];
-    const int K = *a.dK;
-    const int d = a.L.d, lane = threadIdx.x;
-    for (int q0 = 0, base = 0; q0 < K; q0 += 32) {
-        const int q = q0 + lane;
-        const int lv = q < K ? (labels_ran ? (smv(a, q, -1, d, d) > 0 ? 1 : 0) : 1) : 0;
-        const unsigned m = __ballot_sync(0xffffffffu, lv);
-        if (q < K) {
-            s_live[q] = lv;
-            s_cid[q] = base + __popc(m & ((1u << lane) - 1u));
-        }
-        base += __popc(m);
-    }
-    __syncwarp();
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    const int npairs = K * (K - 1) / 2;
-    if (e >= K + npairs) return;
-    Key key{seed, diter[0], diter[1], diter[2]};
-    auto live = [&](int k) { return s_live[k] != 0; };
-    auto cid = [&](int k) { return s_cid[k]; };
-    const double la = a.log_alpha, al = a.alpha;
-    const double* lg = Ltab + lg_offset(a.K_max);
-    if (e < K) {
-        const int k = e;
-        const double nl = smv(a, k, 0, d, d), nr = smv(a, k, 1, d, d);
-        int ok = 0;
-        if (live(k) && nl >= 1 && nr >= 1) {
-            const double lH = la + lg[2 * (3 * k + 1)] + Ltab[3 * k + 1] + lg[2 * (3 * k + 2)] + Ltab[3 * k + 2] -
-                              lg[2 * (3 * k)] - Ltab[3 * k];
-            ok = log(d_uniform(key, (uint32_t)cid(k), TAG_SPLIT, 0)) < lH;
-        }
-        acc[k] = ok;
-    } else {
-        const int p = e - K;
-        int k1, k2;
-        pair_of(p, K, k1, k2);
-        int ok = 0;
-        if (live(k1) && live(k2)) {
-            // lgamma(n_k1 + n_k2) and lgamma(alpha + n_k1 + n_k2), formed by the marginal kernel
-            const double* lgp = Ltab + lg_pair_offset(a.K_max) + 2 * (size_t)p;
-            const double lH = lgp[0] - la - lg[2 * (3 * k1)] - lg[2 * (3 * k2)] + Ltab[3 * a.K_max + p] -
-                              Ltab[3 * k1] - Ltab[3 * k2] + a.lg_alpha - lgp[1] + lg[2 * (3 * k1) + 1] +
-                              lg[2 * (3 * k2) + 1] - 2.0 * a.lg_half_alpha;
-            ok = log(d_uniform(key, (uint32_t)cid(k1), TAG_MERGE, (uint32_t)cid(k2))) < lH;
-        }
-        acc[a.K_max + p] = ok;
-    }
-}
+constexpr int DEC_KMAX = 1024;  // K_max <= 1000
 
 struct DecArgs {
     SMArgs s;
@@ -355,7 +341,7 @@ struct DecArgs {
     const uint32_t* diter;
     uint64_t seed;
     int burn_out, labels_ran, sm_enabled, init_mode;
-    const int* acc;    // hastings_kernel's accept flags
+    const int* acc;    // merge_kernel's accept flags
     int* age;          // K_max
     int* dK;
     int* relabel;      // 3 K_max: map_l, map_r, zmode
@@ -364,8 +350,6 @@ struct DecArgs {
     float* shift32;
     int* derr;
 };
-
-#define DEC_KMAX 1024
 
 // Dynamic shared memory: the accept flags (one byte per proposal) when they fit in
 // dyn_flags bytes, so that the sequential walk reads shared memory only.  The
@@ -568,6 +552,253 @@ __global__ void decision_kernel(DecArgs a, int dyn_flags) {
     if (tid == 0) *a.dK = Kn;
 }
 
+// log H of the split of cluster k (Eq. sample_splits) and of the merge of pair p = (k1, k2)
+// (Eq. sample_merges) from the tables of marginal_kernel.
+__device__ inline double split_ratio(const SMArgs& a, const double* Ltab, int k) {
+    const double* lg = Ltab + lg_offset(a.K_max);
+    return a.log_alpha + lg[2 * (3 * k + 1)] + Ltab[3 * k + 1] + lg[2 * (3 * k + 2)] + Ltab[3 * k + 2] - lg[2 * (3 * k)] -
+           Ltab[3 * k];
+}
+// what the ratio of a merge takes from its two clusters
+__device__ inline double merge_rest(const SMArgs& a, const double* Ltab, int k1, int k2) {
+    const double* lg = Ltab + lg_offset(a.K_max);
+    return -a.log_alpha - lg[2 * (3 * k1)] - lg[2 * (3 * k2)] - Ltab[3 * k1] - Ltab[3 * k2] + a.lg_alpha +
+           lg[2 * (3 * k1) + 1] + lg[2 * (3 * k2) + 1] - 2.0 * a.lg_half_alpha;
+}
+__device__ inline double merge_ratio(const SMArgs& a, const double* Ltab, int p, int k1, int k2) {
+    const double* lgp = Ltab + lg_pair_offset(a.K_max) + 2 * (size_t)p;
+    return lgp[0] + Ltab[3 * a.K_max + p] - lgp[1] + merge_rest(a, Ltab, k1, k2);
+}
+
+// A merge is refused whatever its uniform (log u >= -36.8) when an upper bound of log H says so.
+// log H falls by nu_n / 2 times whatever log|Psi| grows, so a lower bound ld of the pair's log
+// determinant gives one.  In FP64 but for lgammaf and logf; lgm = sum_j lgamma((nu_n - j) / 2).  The
+// margin, 60 + 4e-6 of the magnitudes of the terms, covers the FP32 functions (lgammaf: 6 ulp) and
+// an ld that is off by 8e-6 relative.  False when anything is NaN.
+__device__ inline bool refused_at(const SMArgs& a, const double* Ltab, int k1, int k2, double n1, double n2, double ld,
+                                  float lgm) {
+    const int d = a.L.d;
+    const double n = n1 + n2, nun = a.nu0 + n, kn = a.kappa0 + n;
+    const double lg = (double)lgammaf((float)n) - (double)lgammaf((float)(a.alpha + n));
+    const double L = -0.5 * n * d * 1.1447298858494002 - 0.5 * nun * ld + (double)lgm - (double)(0.5f * d * logf((float)kn)) -
+                     a.lmvg_nu0 + 0.5 * a.nu0 * a.logdet_psi0 + a.half_d_log_kappa0;
+    const double rest = merge_rest(a, Ltab, k1, k2);
+    const double size = 0.6 * n * d + 0.5 * nun * (fabs(ld) + d) + fabs((double)lgm) + 2.0 * fabs((double)lgammaf((float)n)) +
+                        fabs(Ltab[3 * k1]) + fabs(Ltab[3 * k2]) + fabs(rest);
+    return lg + L + rest + 60.0 + 4e-6 * size < -40.0;
+}
+
+__device__ inline float warp_lmvgamma(const SMArgs& a, double n) {  // the sum over j, in every lane
+    float v = 0.f;
+    for (int j = threadIdx.x & 31; j < a.L.d; j += 32) v += lgammaf((float)(0.5 * (a.nu0 + n) - 0.5 * j));
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// First bound, one warp, no factorisation.  With T_k = Psi0 / 2 + C_k, n = n1 + n2, t = n1 / n,
+// delta = xbar1 - xbar2 and w = n1 n2 / n, the pair's scale is Psi = T_1 + T_2 + w delta delta^T + (a
+// square), so
+//   log|Psi| >= log|T_1 + T_2| + log(1 + w delta^T (T_1 + T_2)^-1 delta),
+//   log|T_1 + T_2| >= t log|T_1 / t| + (1 - t) log|T_2 / (1 - t)|   (log det is concave),
+//   delta^T M^-1 delta >= (delta^T u)^2 / (u^T M u) for any u        (Cauchy-Schwarz),
+// taken at u = delta / diag(M).  The quadratic form is raised by 1e-4 of the sum of its magnitudes
+// (at most 800 FP32 terms a lane).  u: d floats of the warp's own.
+__device__ inline bool refused_by_means(const SMArgs& a, const double* Ltab, int k1, int k2, double n1, double n2, float* u) {
+    const int d = a.L.d, lane = threadIdx.x & 31;
+    const float* T1 = a.T32 + (size_t)k1 * d * d;
+    const float* T2 = a.T32 + (size_t)k2 * d * d;
+    float du = 0.f;
+    for (int j = lane; j < d; j += 32) {
+        const float dl = (float)(a.xbar[(size_t)k1 * d + j] - a.xbar[(size_t)k2 * d + j]);
+        const float v = dl / (T1[j * d + j] + T2[j * d + j]);
+        u[j] = v;
+        du = fmaf(dl, v, du);
+    }
+    __syncwarp();
+    float qf = 0.f, qa = 0.f;
+#pragma unroll 4
+    for (int j = 0; j < d; ++j) {
+        const float uj = u[j];
+        for (int l = lane; l <= j; l += 32) {
+            const float m = (l < j ? 2.f : 1.f) * (T1[j * d + l] + T2[j * d + l]) * uj * u[l];
+            qf += m;
+            qa += fabsf(m);
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        du += __shfl_xor_sync(0xffffffffu, du, o);
+        qf += __shfl_xor_sync(0xffffffffu, qf, o);
+        qa += __shfl_xor_sync(0xffffffffu, qa, o);
+    }
+    __syncwarp();
+    const double n = n1 + n2;
+    const float t = (float)(n1 / n), den = qf + 1e-4f * qa;
+    const float q = 0.999f * du * du / den;  // below delta^T M^-1 delta
+    const float ent = -(t * logf(t) + (1.f - t) * log1pf(-t));
+    const double ld = n1 / n * a.ldT[k1] + n2 / n * a.ldT[k2] + (double)(d * ent + log1pf((float)(n1 * n2 / n) * q));
+    return den > 0.f && q >= 0.f && refused_at(a, Ltab, k1, k2, n1, n2, ld, warp_lmvgamma(a, n));
+}
+
+// Second bound, the whole block: log|B| of B = T_1 + T_2 + w delta delta^T by an FP32 LDL
+// factorisation of A = B - theta diag(B).  The computed factors are those of A + E with
+// |E_jl| <= (d + 24) 2^-24 sqrt(b_jj b_ll) (d + 8 roundings of a sum, 4 ulp a reciprocal, the
+// rounding of the entries), so E is at most theta diag(B) for theta = d (d + 24) 2^-24 (1.1 of
+// it is taken), what was factorised is at most B, and the pivots' product at most |B|.
+// Dynamic shared memory: d (d | 1) + 9 d floats.
+__device__ inline bool refused_by_factor(const SMArgs& a, const double* Ltab, int k1, int k2, double n1, double n2, float* sm) {
+    const int d = a.L.d, ld = d | 1, tid = threadIdx.x, nt = blockDim.x;
+    __shared__ int s_fail, s_ref;
+    float* A = sm;
+    float* dl = A + d * ld;
+    float* piv = dl + d;
+    float* rs = piv + d;
+    float* cols = rs + d;  // 4 d
+    const float* T1 = a.T32 + (size_t)k1 * d * d;
+    const float* T2 = a.T32 + (size_t)k2 * d * d;
+    for (int j = tid; j < d; j += nt) dl[j] = (float)(a.xbar[(size_t)k1 * d + j] - a.xbar[(size_t)k2 * d + j]);
+    if (tid == 0) s_fail = 0;
+    __syncthreads();
+    const float w = (float)(n1 * n2 / (n1 + n2)) * 0.9999f;
+    const float keep = 1.f - 1.1f * 5.97e-8f * (float)d * (float)(d + 24);
+    for (int j = tid >> 5; j < d; j += nt >> 5)
+        for (int l = tid & 31; l <= j; l += 32) {
+            const float b = T1[j * d + l] + T2[j * d + l] + w * dl[j] * dl[l];
+            A[j * ld + l] = l == j ? b * keep : b;
+        }
+    __syncthreads();
+    chol_ldl_blk<float>(A, d, ld, piv, rs, cols, nullptr, 0.f, &s_fail, nullptr);
+    if (tid < 32) {
+        float v = 0.f;
+        for (int j = tid; j < d; j += 32) v += logf(piv[j]);
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        const bool r = !s_fail && refused_at(a, Ltab, k1, k2, n1, n2, (double)v, warp_lmvgamma(a, n1 + n2));
+        if (tid == 0) s_ref = r;
+    }
+    __syncthreads();
+    const bool r = s_ref != 0;
+    __syncthreads();  // s_ref and the workspace are written again
+    return r;
+}
+
+// The two bounds of every pair ahead of merge_kernel: acc[K_max + p] = 0 (refused) or 2 (open).  For
+// dimensions whose FP64 factorisation leaves room for one block per SM (d = 128: 142 KB): the
+// FP32 one takes half of that, and three of these blocks run side by side.
+// Dynamic shared memory: refused_by_factor's.
+constexpr int BOUND_W = 4;  // warps
+
+__global__ void __launch_bounds__(32 * BOUND_W) bound_kernel(SMArgs a, const double* Ltab, int labels_ran, int* acc) {
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ int s_open[BOUND_W];
+    const int K = *a.dK, d = a.L.d, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (pairs_at_once(a, K)) return;
+    const int npairs = K * (K - 1) / 2;
+    // a block's warps take pairs far apart: a small cluster's pairs, most likely to be open, are
+    // neighbours and go to different blocks
+    for (int p0 = blockIdx.x; p0 < npairs; p0 += gridDim.x * BOUND_W) {
+        const int p = p0 + warp * gridDim.x;
+        bool open = false;
+        if (p < npairs) {
+            int k1, k2;
+            pair_of(p, K, k1, k2);
+            const double n1 = smv(a, k1, -1, d, d), n2 = smv(a, k2, -1, d, d);
+            open = (n1 > 0 && n2 > 0 && !refused_by_means(a, Ltab, k1, k2, n1, n2, (float*)dyn + warp * d)) ||
+                   (!labels_ran && !(n1 > 0 && n2 > 0));
+            if (!open && lane == 0) acc[a.K_max + p] = 0;
+        }
+        if (lane == 0) s_open[warp] = open;
+        __syncthreads();
+        for (int w = 0; w < BOUND_W; ++w) {
+            if (!s_open[w]) continue;  // uniform
+            int k1, k2;
+            const int q = p0 + w * gridDim.x;
+            pair_of(q, K, k1, k2);
+            const double n1 = smv(a, k1, -1, d, d), n2 = smv(a, k2, -1, d, d);
+            const bool r = refused_by_factor(a, Ltab, k1, k2, n1, n2, (float*)dyn);
+            if (threadIdx.x == 0) acc[a.K_max + q] = r ? 0 : 2;
+        }
+        __syncthreads();  // u and s_open are written again
+    }
+}
+
+// Every split and merge proposal's acceptance, acc[k] for the split of cluster k and acc[K_max
+// + p] for merge pair p (1: accepted if proposed; indices in the Philox counters are those
+// after removing emptied clusters).  bounded: bound_kernel has been there.  Many Gaussian pairs (not pairs_at_once): a warp bounds each pair's ratio from the means, the
+// block factorises in FP32 what that leaves open, and in FP64 what that leaves open; the FP64
+// factorisation of every pair was the step's cost (d = 128, K = 64: 2,016 pairs and 192 slots
+// 6.0 ms; now 0.8 ms for the slots and 1.2 ms for the pairs).
+// Dynamic shared memory: marginal_item's; the bounds' u (a row of d floats per warp) share it.
+constexpr int MERGE_W = 8;  // warps
+
+__global__ void __launch_bounds__(32 * MERGE_W) merge_kernel(SMArgs a, double* Ltab, const uint32_t* diter, uint64_t seed,
+                                                              int labels_ran, int* acc, int* derr, int bounded) {
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ short s_cid[DEC_KMAX];  // index after removing the empty clusters; -1: empty
+    __shared__ int s_open[MERGE_W];
+    const int K = *a.dK, d = a.L.d, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nt = 32 * MERGE_W, npairs = K * (K - 1) / 2;
+    const bool once = pairs_at_once(a, K);
+    // blocks with work (acceptances alone: a proposal per thread); the others leave at once
+    const int nb = once ? min((int)gridDim.x, (max(K, npairs) + nt - 1) / nt) : (int)gridDim.x;
+    if ((int)blockIdx.x >= nb) return;
+    if (warp == 0)
+        for (int q0 = 0, base = 0; q0 < K; q0 += 32) {
+            const int q = q0 + lane;
+            const bool lv = q < K && (!labels_ran || smv(a, q, -1, d, d) > 0);
+            const unsigned m = __ballot_sync(0xffffffffu, lv);
+            if (q < K) s_cid[q] = lv ? (short)(base + __popc(m & ((1u << lane) - 1u))) : (short)-1;
+            base += __popc(m);
+        }
+    __syncthreads();
+    const Key key{seed, diter[0], diter[1], diter[2]};
+    // log u < lH; no logarithm where it cannot change the outcome (-36.8 <= log u < 0)
+    auto accept = [&](double lH, uint32_t c0, uint32_t tag, uint32_t blk) -> int {
+        if (lH >= 0.0) return 1;
+        if (!(lH > -40.0)) return 0;
+        return log(d_uniform(key, c0, tag, blk)) < lH;
+    };
+    for (int k = blockIdx.x * nt + tid; k < K; k += nb * nt)
+        acc[k] = s_cid[k] >= 0 && smv(a, k, 0, d, d) >= 1 && smv(a, k, 1, d, d) >= 1
+                     ? accept(split_ratio(a, Ltab, k), (uint32_t)s_cid[k], TAG_SPLIT, 0) : 0;
+    if (once) {
+        for (int p = blockIdx.x * nt + tid; p < npairs; p += nb * nt) {
+            int k1, k2;
+            pair_of(p, K, k1, k2);
+            acc[a.K_max + p] = s_cid[k1] >= 0 && s_cid[k2] >= 0
+                                   ? accept(merge_ratio(a, Ltab, p, k1, k2), (uint32_t)s_cid[k1], TAG_MERGE, (uint32_t)s_cid[k2]) : 0;
+        }
+    } else {
+        for (int p0 = blockIdx.x; p0 < npairs; p0 += gridDim.x * MERGE_W) {
+            const int p = p0 + warp * gridDim.x;
+            bool open = false;
+            if (p < npairs) {
+                int k1, k2;
+                pair_of(p, K, k1, k2);
+                if (bounded)
+                    open = acc[a.K_max + p] == 2;
+                else if (s_cid[k1] >= 0 && s_cid[k2] >= 0)
+                    open = !refused_by_means(a, Ltab, k1, k2, smv(a, k1, -1, d, d), smv(a, k2, -1, d, d), (float*)dyn + warp * d);
+                if (!open && lane == 0) acc[a.K_max + p] = 0;
+            }
+            if (lane == 0) s_open[warp] = open;
+            __syncthreads();
+            for (int w = 0; w < MERGE_W; ++w) {
+                if (!s_open[w]) continue;  // uniform
+                const int q = p0 + w * gridDim.x;
+                int k1, k2, ok = 0;
+                pair_of(q, K, k1, k2);
+                if (bounded ||
+                    !refused_by_factor(a, Ltab, k1, k2, smv(a, k1, -1, d, d), smv(a, k2, -1, d, d), (float*)dyn)) {
+                    marginal_item(a, Ltab, derr, K, 3 * K + q);
+                    __syncthreads();
+                    ok = accept(merge_ratio(a, Ltab, q, k1, k2), (uint32_t)s_cid[k1], TAG_MERGE, (uint32_t)s_cid[k2]);
+                }
+                if (tid == 0) acc[a.K_max + q] = ok;
+            }
+            __syncthreads();  // u and s_open are written again
+        }
+    }
+}
+
 __global__ void relabel_kernel(int64_t N, const int* relabel, int Kmax, const int* gate, const uint32_t* diter,
                                uint64_t seed, int32_t* z, uint8_t* zbar, int* derr) {
     if (*gate == 0) return;
@@ -621,7 +852,11 @@ static SMArgs sm_args(dpmm_ctx* c) {
         }
         a.lg_sum_beta = std::lgamma(a.sum_beta);
     }
+    a.T32 = c->sm_T;
+    a.xbar = c->sm_xbar;
+    a.ldT = c->sm_xbar ? c->sm_xbar + (size_t)c->K_max * c->d : nullptr;
     a.stage = 0;
+    a.exact = 0;
     a.kind = c->kind;
     a.K_max = c->K_max;
     a.dK = c->dK;
@@ -630,65 +865,79 @@ static SMArgs sm_args(dpmm_ctx* c) {
 
 cudaError_t launch_restats_gated(dpmm_ctx* c, const int* gate);
 
+// the marginals and every proposal's acceptance
+static cudaError_t launch_proposals(dpmm_ctx* c, SMArgs& s, uint64_t seed, int labels_ran) {
+    // the Dirichlet marginal needs no matrix workspace; the NIW one stages the two statistics
+    // blocks it reads when they fit
+    size_t smi = 0;
+    if (c->kind == DPMM_PRIOR_NIW) {
+        smi = sizeof(double) * ((size_t)c->d * (c->d | 1) + 10 * c->d);
+        const size_t st = smi + sizeof(double) * 2 * (size_t)c->st.E;
+        if (st <= 160 * 1024) {
+            smi = st;
+            s.stage = 1;
+        }
+    }
+    if (smi > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(marginal_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smi);
+        if (e != cudaSuccess) return e;
+    }
+    // one wave of resident blocks, each taking items in turn (the items beyond the current K
+    // launch no block)
+    auto waves = [&](const void* fn, int threads, size_t smem, int items) {
+        int per = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads, smem) != cudaSuccess || per < 1) {
+            cudaGetLastError();
+            per = 1;
+        }
+        return (unsigned)std::max<int64_t>(1, std::min<int64_t>(items, (int64_t)per * c->num_sms));
+    };
+    const int pairs = c->K_max * (c->K_max - 1) / 2, all = 3 * c->K_max + pairs;
+    // two items an SM where two fit it side by side (their chains of latencies overlap)
+    s.exact = c->num_sms * (smi <= 100 * 1024 ? 2 : 1);
+    const bool bounds = c->kind == DPMM_PRIOR_NIW && all > s.exact;  // else every pair is evaluated with the slots
+    prof_begin(c, "marginal");
+    if (c->sparse)
+        marginal_counts_kernel<CountsF32>
+            <<<waves((const void*)marginal_counts_kernel<CountsF32>, 256, 0, all), 256, 0, c->stream>>>(
+                s, CountsF32{c->sp_cc, c->d}, c->sp_lgt, c->sp_lgt ? SP_LGT : 0, c->sp_lgb, c->Ltab);
+    else if (c->kind == DPMM_PRIOR_DIRICHLET && c->prec != DPMM_PREC_FP64_PLAIN)  // dense counts
+        marginal_counts_kernel<CountsStats>
+            <<<waves((const void*)marginal_counts_kernel<CountsStats>, 256, 0, all), 256, 0, c->stream>>>(
+                s, CountsStats{c->stats, c->st}, c->sp_lgt, c->sp_lgt ? SP_LGT : 0, c->sp_lgb, c->Ltab);
+    else
+        marginal_kernel<<<waves((const void*)marginal_kernel, 128, smi, bounds ? std::max(4 * c->K_max, s.exact) : all), 128, smi,
+                          c->stream>>>(s, c->Ltab, c->derr);
+    prof_end(c, "marginal");
+    c->nlaunch += 1;
+    prof_begin(c, "hastings");
+    cudaError_t ea = cudaFuncSetAttribute(merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smi);
+    if (ea != cudaSuccess) return ea;
+    const int bounded = bounds && smi > 100 * 1024;
+    if (bounded) {
+        const size_t bs = sizeof(float) * ((size_t)c->d * (c->d | 1) + 9 * c->d);
+        cudaError_t e = cudaFuncSetAttribute(bound_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bs);
+        if (e != cudaSuccess) return e;
+        bound_kernel<<<waves((const void*)bound_kernel, 32 * BOUND_W, bs, (pairs + BOUND_W - 1) / BOUND_W), 32 * BOUND_W, bs,
+                       c->stream>>>(s, c->Ltab, labels_ran, c->acc);
+        c->nlaunch += 1;
+    }
+    const int items = std::max(1, bounds ? (pairs + MERGE_W - 1) / MERGE_W : (pairs + 32 * MERGE_W - 1) / (32 * MERGE_W));
+    merge_kernel<<<waves((const void*)merge_kernel, 32 * MERGE_W, smi, items), 32 * MERGE_W, smi, c->stream>>>(
+        s, c->Ltab, c->diter, seed, labels_ran, c->acc, c->derr, bounded);
+    prof_end(c, "hastings");
+    c->nlaunch += 1;
+    return cudaGetLastError();
+}
+
 cudaError_t launch_splitmerge(dpmm_ctx* c, uint64_t seed, int labels_ran, int sm_enabled) {
     SMArgs s = sm_args(c);
-    if (sm_enabled) {
-        int items = 3 * c->K_max + c->K_max * (c->K_max - 1) / 2;
-        // the Dirichlet marginal needs no matrix workspace; the NIW one stages the two
-        // statistics blocks it reads when they fit
-        size_t sm = 0;
-        if (c->kind == DPMM_PRIOR_NIW) {
-            sm = sizeof(double) * ((size_t)c->d * (c->d | 1) + 10 * c->d);
-            const size_t st = sm + sizeof(double) * 2 * (size_t)c->st.E;
-            if (st <= 160 * 1024) {
-                sm = st;
-                s.stage = 1;
-            }
-        }
-        if (sm > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(marginal_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            if (e != cudaSuccess) return e;
-        }
-        // one wave of resident blocks, each taking items in turn (the items beyond the
-        // current K launch no block)
-        auto waves = [&](const void* fn, int threads, size_t smem) {
-            int per = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads, smem) != cudaSuccess || per < 1) {
-                cudaGetLastError();
-                per = 1;
-            }
-            return (unsigned)std::min<int64_t>(items, (int64_t)per * c->num_sms);
-        };
-        prof_begin(c, "marginal");
-        if (c->sparse)
-            marginal_counts_kernel<CountsF32>
-                <<<waves((const void*)marginal_counts_kernel<CountsF32>, 256, 0), 256, 0, c->stream>>>(
-                    s, CountsF32{c->sp_cc, c->d}, c->sp_lgt, c->sp_lgt ? SP_LGT : 0, c->sp_lgb, c->Ltab);
-        else if (c->kind == DPMM_PRIOR_DIRICHLET && c->prec != DPMM_PREC_FP64_PLAIN)  // dense counts
-            marginal_counts_kernel<CountsStats>
-                <<<waves((const void*)marginal_counts_kernel<CountsStats>, 256, 0), 256, 0, c->stream>>>(
-                    s, CountsStats{c->stats, c->st}, c->sp_lgt, c->sp_lgt ? SP_LGT : 0, c->sp_lgb, c->Ltab);
-        else
-            marginal_kernel<<<waves((const void*)marginal_kernel, 128, sm), 128, sm, c->stream>>>(s, c->Ltab, c->derr);
-        prof_end(c, "marginal");
-        c->nlaunch += 1;
-    }
-    if (sm_enabled) {
-        const int items = c->K_max + c->K_max * (c->K_max - 1) / 2;
-        prof_begin(c, "hastings");
-        hastings_kernel<<<(items + 31) / 32, 32, 0, c->stream>>>(s, c->Ltab, c->diter, seed, labels_ran ? 1 : 0,
-                                                                   c->acc);
-        prof_end(c, "hastings");
-        c->nlaunch += 1;
-    }
     DecArgs a;
-    a.s = s;
     a.acc = c->acc;
     a.Ltab = c->Ltab;
     a.diter = c->diter;
     a.seed = seed;
     a.burn_out = c->burn_out;
-    a.labels_ran = labels_ran;
     a.sm_enabled = sm_enabled;
     a.init_mode = (labels_ran == 2);
     a.labels_ran = labels_ran ? 1 : 0;
@@ -699,6 +948,11 @@ cudaError_t launch_splitmerge(dpmm_ctx* c, uint64_t seed, int labels_ran, int sm
     a.shift_new = c->shift_new;
     a.shift32 = c->shift32;
     a.derr = c->derr;
+    if (sm_enabled) {
+        const cudaError_t e = launch_proposals(c, s, seed, a.labels_ran);
+        if (e != cudaSuccess) return e;
+    }
+    a.s = s;
     prof_begin(c, "decision");
     const int dyn = 32 * 1024;
     cudaError_t ea = cudaFuncSetAttribute(decision_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
