@@ -1417,141 +1417,177 @@ __global__ void __launch_bounds__(256) substats_f32_kernel(SubArgs<float> a) {
     if (cur >= 0) flush(cur);
 }
 
-// FP32 variant for 64 < d <= 128 (Gaussian).  Per batch of WP = 64 points (sorted by
-// cluster): each sub-cluster score is the squared norm of (x - mu_h) W_h
-// = (x - shift) W_h - bh, with bh = (mu_h - shift)^T W_h formed once per cluster run and
-// shift the cluster's statistics centre; both products run at once over the shifted rows
-// (warps 0-7 sub-cluster 0, warps 8-15 sub-cluster 1; each thread owns 8 points x 4
-// columns; per K step two broadcast float4 loads of (x - shift)^T and one float4 of W
-// feed 32 FMAs; W is staged once per cluster run, zero below the diagonal and beyond d,
-// so the loop needs no triangular bound).  Statistics: one 4x4 register block per
-// worker thread (nblk <= 561 workers, so every block has one owner and is written
-// straight to the records) and one accumulator set per sub-cluster (warp-uniform
-// branch on h).  Dynamic shared memory: 2 x 128 x 128 floats (W_l, W_r), 128 x WP
-// (x - mu_h)^T, WP x dp point rows, WP x 2 scores, then ints and bytes.
+// FP32 variant for 64 < d <= 128 (Gaussian), two groups of warps.  The sorted positions of the
+// block's range are cut into batches of at most WP = 64 points of one cluster.  The score
+// group (8 warps) shifts batch i's rows by the cluster's centre, transposes them, and forms both
+// Y_h = (X - shift) W_h - bh (bh = (mu_h - shift)^T W_h once per cluster) as register tiles of 8
+// points x 4 columns, then the scores and z-bar; the statistics group (10 warps) adds batch i - 1
+// to its register blocks (8 x 4 entries per thread and sub-cluster, every entry with one owner,
+// written straight to the records); the rows of batch i + 1 arrive by cp.async meanwhile.
+// What bounds it: shared-memory reads (12 floats a lane for 32 multiply-adds; LSU pipe 66% busy),
+// then the FP32 FMA pipe.  W is upper triangular, so a tile of 16 columns ends at its last
+// column's diagonal (56% of the square; a warp takes tiles i and 7 - i, 144 rows in all), and 14.3
+// thousand FMA issues per scheduler and batch are left of 21.  Skipped products are exact zeros,
+// every sum adds in the order l = 0, 1, ... (points: sorted order), and a score's 32 column
+// groups are added by halves (16, 8, 4, 2, 1 apart).
+// Measured at d = 128, N = 4e6, K = 64: 8.25 ms; 10.9 ms with square products and the two phases
+// in turn over 18 warps.
+// Dynamic shared memory: three row buffers of WP x dp, W_l and W_r as packed column tiles, the
+// transposed rows (128 x TTS), the column groups' sums (2 x 32 x WP), then the small arrays.
 constexpr int WP = 64;
-constexpr int WIDE_T = 576;
+constexpr int WIDE_S = 256;  // threads of the score group
+constexpr int WIDE_T = 576;  // threads in all
+constexpr int TTS = 68;      // row stride of the transposed rows
+constexpr int WTILE = 16 * 16 * 36;  // floats of a packed factor: 8 column tiles of 16 (t + 1) rows
 
-template <typename XT>
-__global__ void __launch_bounds__(WIDE_T, 1) substats_wide_kernel(SubArgs<float> a) {
+static size_t wide_smem_of(int dp) {
+    return ((size_t)3 * WP * dp + 8 + 2 * WTILE + 128 * TTS + 64 * WP + 256 + 128 + 4) * 4 + (3 * WP + 260) * sizeof(int) + 3 * WP;
+}
+
+struct WideArgs {
+    SubArgs<float> a;
+    const int* starts;
+};
+
+__device__ __forceinline__ void wide_bar() { asm volatile("bar.sync 1, 256;" ::: "memory"); }  // the score group's
+
+__global__ void __launch_bounds__(WIDE_T, 1) substats_wide_kernel(WideArgs wa) {
+    const SubArgs<float>& a = wa.a;
     if (a.gate && *a.gate == 0) return;
     extern __shared__ __align__(16) unsigned char smraw[];
-    const int d = a.d, dp = a.L.dp, nblk = a.L.nblk;
-    float* Ws = (float*)smraw;              // 2 x 128 x 128: W_h[l][j]
-    float* Tt = Ws + 2 * 128 * 128;         // 128 x WP: (x_p - shift)_l at Tt[l * WP + p]
-    float* xs = Tt + 128 * WP;              // WP x dp
-    float* qv = xs + WP * dp;               // WP x 2
-    float* mus = qv + 2 * WP;               // 2 x 128
-    float* bh = mus + 256;                  // 2 x 128
-    float* shf = bh + 256;                  // 128
-    float* cc = shf + 128;                  // 2 (+2 pad)
-    int* kq = (int*)(cc + 4);               // WP
-    int* runs = kq + WP;                    // WP + 1
-    int* nruns = runs + WP + 1;             // 1
-    unsigned char* hq = (unsigned char*)(nruns + 1);  // WP
-    __shared__ int staged;
-    __shared__ int wcnt[32];
-
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
-    const int g = blockIdx.x;
+    const int d = a.d, dp = a.L.dp, nb = a.L.nb;
+    float* xs = (float*)smraw;                // 3 x WP x dp (+ 8: the last row's read past its end)
+    float* Wp = xs + 3 * WP * dp + 8;         // 2 x WTILE
+    float* Tt = Wp + 2 * WTILE;               // 128 x TTS
+    float* qp = Tt + 128 * TTS;               // 2 x 32 x WP
+    float* bh = qp + 64 * WP;                 // 2 x 128
+    float* shf = bh + 256;                    // 128
+    float* cc = shf + 128;                    // 2 (+ 2)
+    int* iq = (int*)(cc + 4);                 // 3 x WP points
+    int* st = iq + 3 * WP;                    // the range's clusters' starts
+    unsigned char* hq = (unsigned char*)(st + 260);  // 3 x WP
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int g = blockIdx.x, K = *a.dK;
     const int64_t p0 = (int64_t)g * a.R, p1 = min(a.N, p0 + a.R);
-    Key key{a.seed, a.diter[0], a.diter[1], a.diter[2]};
-    const XT* X = (const XT*)a.X;
-    const bool worker = tid < nblk;
-    int jb = 0, lb = 0;
-    a.L.blk_coords(worker ? tid : 0, jb, lb);
-    float acc0[16], acc1[16];
-#pragma unroll
-    for (int e = 0; e < 16; ++e) acc0[e] = acc1[e] = 0.f;
-    int cur = -1;
-    if (tid == 0) staged = -1;
-
-    auto flush = [&](int k) {  // every block has a single owner: no reduction
-        if (worker) {
-            double* out = a.rec + (size_t)(g + k) * 2 * a.L.E + (size_t)tid * 16;
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                out[e] = (double)acc0[e];
-                out[a.L.E + e] = (double)acc1[e];
-            }
-        }
-#pragma unroll
-        for (int e = 0; e < 16; ++e) acc0[e] = acc1[e] = 0.f;
+    if (p0 >= p1 || K < 1) return;
+    int k0 = 0;  // the cluster of position p0: the last k with starts[k] <= p0
+    for (int lo = 0, hi = K; hi - lo > 1;) {
+        const int mid = (lo + hi) >> 1;
+        if (wa.starts[mid] <= p0) lo = mid;
+        else hi = mid;
+        k0 = lo;
+    }
+    // the batches, walked alike by every thread
+    struct Batch {
+        int64_t pos;
+        int k, np, run;  // np = 0: none left; run: batch number
     };
+    auto first_end = [&](int k) { return min(p1, (int64_t)(k - k0 < 259 ? st[k - k0 + 1] : wa.starts[k + 1])); };
+    for (int e = tid; e < 260; e += WIDE_T) st[e] = k0 + e <= K ? wa.starts[k0 + e] : (int)min(a.N, (int64_t)0x7fffffff);
+    __syncthreads();
+    auto settle = [&](Batch& q) {  // q.pos, q.k -> the batch that begins there
+        while (q.k + 1 < K && first_end(q.k) <= q.pos && q.pos < p1) ++q.k;
+        q.np = q.pos < p1 ? (int)min((int64_t)WP, first_end(q.k) - q.pos) : 0;
+        if (q.np < 0) q.np = 0;  // the starts do not cover the points (never for consistent state)
+    };
+    auto next = [&](Batch& q) {
+        q.pos = q.np > 0 ? q.pos + q.np : p1;
+        q.run += 1;
+        settle(q);
+    };
+    Batch cur{p0, k0, 0, 0};
+    settle(cur);
 
-    for (int64_t base = p0; base < p1; base += WP) {
-        const int np = (int)min((int64_t)WP, p1 - base);
-        __syncthreads();
-        if (tid < np) kq[tid] = a.z[a.idx[base + tid]];
-        // raw rows, one warp per row (d <= 128: one float4 per lane)
-        for (int r = warp; r < np; r += nt / 32) {
-            const int i = a.idx[base + r];
-            float* xr = xs + (size_t)r * dp;
-            if constexpr (sizeof(XT) == 4) {
-                if (lane * 4 < d) *(float4*)(xr + lane * 4) = *(const float4*)(X + (int64_t)i * a.xs + lane * 4);
-            } else {
-                for (int j = lane; j < d; j += 32) xr[j] = ldx<float, XT>(X + (int64_t)i * a.xs + j);
+    if (warp < WIDE_S / 32) {
+        // ------------------------------------------------------------ score group
+        const Key key{a.seed, a.diter[0], a.diter[1], a.diter[2]};
+        const float* X = (const float*)a.X;
+        // rows 8 warp .. 8 warp + 7 of a batch: lane r < 8 holds row r's point
+        auto load_idx = [&](const Batch& q) {
+            const int r = 8 * warp + lane;
+            return lane < 8 && r < q.np ? a.idx[q.pos + r] : 0;
+        };
+        auto fetch = [&](const Batch& q, int pt) {
+            float* to = xs + (size_t)(q.run % 3) * WP * dp;
+            for (int r = 0; r < 8; ++r) {
+                const int i = __shfl_sync(0xffffffffu, pt, r), row = 8 * warp + r;
+                if (row < q.np && lane * 4 < d) mw_cp16(to + row * dp + lane * 4, X + (int64_t)i * a.xs + lane * 4);
             }
-        }
-        __syncthreads();
-        find_runs(kq, np, runs, nruns, wcnt);
-        const int nr = *nruns;
-        for (int r = 0; r < nr; ++r) {
-            const int qs = runs[r], qe = runs[r + 1];
-            const int k = kq[qs];
-            if (k != staged) {  // uniform: stage the cluster's two sub-clusters
-                __syncthreads();
-                for (int e = tid; e < 2 * 128 * 128; e += nt) {
-                    const int h = e >> 14, l = (e >> 7) & 127, j = e & 127;
-                    const int s = 3 * k + 1 + h;
-                    Ws[e] = (j < d && l <= j) ? a.pv.W[((size_t)s * d + l) * d + j] : 0.f;
-                }
-                for (int e = tid; e < 256; e += nt) {
-                    const int h = e >> 7, j = e & 127;
-                    mus[e] = j < d ? a.pv.mu[(size_t)(3 * k + 1 + h) * d + j] : 0.f;
+            if (lane < 8) iq[(q.run % 3) * WP + 8 * warp + lane] = pt;
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        Batch nx = cur;
+        fetch(cur, load_idx(cur));
+        next(nx);
+        int pt = load_idx(nx);
+        int staged = -1;
+        for (; cur.np > 0;) {
+            Batch n2 = nx;
+            if (nx.np > 0) {
+                fetch(nx, pt);
+                next(n2);
+                pt = load_idx(n2);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+            const int np = cur.np, k = cur.k, buf = cur.run % 3;
+            float* xb = xs + (size_t)buf * WP * dp;
+            if (k != staged) {  // the cluster's two sub-clusters (every reader of the last is past a barrier)
+                for (int e = tid; e < 2 * WTILE; e += WIDE_S) {
+                    const int h = e / WTILE, f = e % WTILE, r16 = f >> 4;  // 16-float row r16 of the packed tiles
+                    int t = 0;
+                    while (8 * (t + 1) * (t + 2) <= r16) ++t;
+                    const int l = r16 - 8 * t * (t + 1), j = 16 * t + (f & 15);
+                    Wp[e] = (j < d && l <= j) ? a.pv.W[((size_t)(3 * k + 1 + h) * d + l) * d + j] : 0.f;
                 }
                 if (tid < 2) cc[tid] = a.pv.c[3 * k + 1 + tid];
-                for (int j = tid; j < 128; j += nt) shf[j] = j < d ? a.shift[(size_t)k * d + j] : 0.f;
-                __syncthreads();
-                // bh[h][j] = sum_l (mu_h - shift)_l W_h[l][j]: the products below run on the
-                // shifted rows x - shift, so y_h = (x - shift) W_h - bh
-                for (int e = tid; e < 256; e += nt) {
-                    const int h = e >> 7, j = e & 127;
-                    const float* Wh = Ws + h * 128 * 128;
+                if (tid < 128) shf[tid] = tid < d ? a.shift[(size_t)k * d + tid] : 0.f;
+                wide_bar();
+                {  // bh[h][j] = sum_l (mu_h - shift)_l W_h[l][j]
+                    const int h = tid >> 7, j = tid & 127, t = j >> 4;
+                    const float* mu = a.pv.mu + (size_t)(3 * k + 1 + h) * d;
+                    const float* Wt = Wp + h * WTILE + 128 * t * (t + 1) + (j & 15);
                     float b = 0.f;
-                    for (int l = 0; l < d; ++l) b = fmaf(mus[h * 128 + l] - shf[l], Wh[l * 128 + j], b);
-                    bh[e] = b;
+                    if (j < d)
+                        for (int l = 0; l <= j; ++l) b = fmaf(__ldg(mu + l) - shf[l], Wt[l * 16], b);
+                    bh[tid] = b;
                 }
-                __syncthreads();
-                if (tid == 0) staged = k;
+                staged = k;
             }
-            // the run's rows shifted by the cluster's centre, then 1, then zeros (the
-            // statistics read them too)
-            for (int e = tid; e < (qe - qs) * dp; e += nt) {
-                const int q = qs + e / dp, j = e % dp;
-                float* xr = xs + (size_t)q * dp;
-                xr[j] = j < d ? xr[j] - shf[j] : (j == d ? 1.f : 0.f);
+            wide_bar();  // the rows have landed, the parameters are staged
+            // the rows less the centre, then 1, then zeros; and transposed
+            for (int p = warp; p < WP; p += WIDE_S / 32) {
+                float* xr = xb + p * dp;
+                for (int j = lane; j < max(dp, 128); j += 32) {
+                    float v = 0.f;
+                    if (p < np) v = j < d ? xr[j] - shf[j] : (j == d ? 1.f : 0.f);
+                    if (j < dp) xr[j] = v;
+                    if (j < 128) Tt[j * TTS + p] = j < d ? v : 0.f;
+                }
             }
             if (a.draw) {
-                __syncthreads();
-                for (int e = tid; e < 128 * WP; e += nt) {
-                    const int l = e / WP, p = e % WP;
-                    Tt[e] = (l < d && p >= qs && p < qe) ? xs[(size_t)p * dp + l] : 0.f;
-                }
-                __syncthreads();
-                if (tid < 512) {  // warps 0-7: sub-cluster 0, warps 8-15: sub-cluster 1
-                    const int h = warp >> 3;
-                    const int pg = warp & 7, cg = lane;  // points 8 pg .. 8 pg + 7, columns 4 cg .. 4 cg + 3
+                wide_bar();
+                const int h = warp >> 2, pg = lane & 7, cg = lane >> 3;  // points 8 pg .., columns 16 t + 4 cg ..
+                for (int half = 0; half < 2; ++half) {
+                    const int t = half ? warp & 3 : 7 - (warp & 3);
+                    if (16 * t >= d) {  // no such columns: zero sums, as their products would give
+                        for (int u = 0; u < 8; ++u) qp[(h * 32 + 4 * t + cg) * WP + 8 * pg + u] = 0.f;
+                        continue;
+                    }
                     float y[8][4];
 #pragma unroll
                     for (int u = 0; u < 8; ++u)
 #pragma unroll
                         for (int v = 0; v < 4; ++v) y[u][v] = 0.f;
-                    const float* Wh = Ws + h * 128 * 128;
-                    for (int l = 0; l < d; ++l) {
-                        const float4 t0 = *(const float4*)(Tt + l * WP + pg * 8);
-                        const float4 t1 = *(const float4*)(Tt + l * WP + pg * 8 + 4);
-                        const float4 w0 = *(const float4*)(Wh + l * 128 + cg * 4);
+                    const float* Wt = Wp + h * WTILE + 128 * t * (t + 1) + 4 * cg;
+                    const float* tp = Tt + 8 * pg;
+                    const int le = min(d, 16 * t + 16);
+#pragma unroll 4
+                    for (int l = 0; l < le; ++l) {
+                        const float4 t0 = *(const float4*)(tp + l * TTS);
+                        const float4 t1 = *(const float4*)(tp + l * TTS + 4);
+                        const float4 w0 = *(const float4*)(Wt + l * 16);
                         const float tv[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
                         const float wv[4] = {w0.x, w0.y, w0.z, w0.w};
 #pragma unroll
@@ -1559,75 +1595,116 @@ __global__ void __launch_bounds__(WIDE_T, 1) substats_wide_kernel(SubArgs<float>
 #pragma unroll
                             for (int v = 0; v < 4; ++v) y[u][v] = fmaf(tv[u], wv[v], y[u][v]);
                     }
-                    const float4 b4 = *(const float4*)(bh + h * 128 + cg * 4);
+                    const float4 b4 = *(const float4*)(bh + h * 128 + 16 * t + 4 * cg);
                     const float bv[4] = {b4.x, b4.y, b4.z, b4.w};
-                    float qp[8];
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
                         float s0 = 0.f;
 #pragma unroll
                         for (int v = 0; v < 4; ++v) {
-                            const float t = y[u][v] - bv[v];
-                            s0 = fmaf(t, t, s0);
+                            const float r = y[u][v] - bv[v];
+                            s0 = fmaf(r, r, s0);
                         }
-                        qp[u] = s0;
+                        qp[(h * 32 + 4 * t + cg) * WP + 8 * pg + u] = s0;
                     }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) qp[u] += __shfl_xor_sync(0xffffffffu, qp[u], o);
-                    if (cg == 0)
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) qv[(pg * 8 + u) * 2 + h] = qp[u];
                 }
-                __syncthreads();
+                wide_bar();
             }
-            if (tid >= qs && tid < qe) {
-                const int i = a.idx[base + tid];
+            if (tid < np) {
+                const int i = iq[buf * WP + tid];
                 int h;
                 if (a.draw) {
+                    float q[2];
+#pragma unroll
+                    for (int hh = 0; hh < 2; ++hh) {  // the column groups 16, 8, 4, 2, 1 apart
+                        float v[16];
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) v[c] = qp[(hh * 32 + c) * WP + tid] + qp[(hh * 32 + c + 16) * WP + tid];
+#pragma unroll
+                        for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+                            for (int c = 0; c < o; ++c) v[c] += v[c + o];
+                        q[hh] = v[0];
+                    }
                     uint32_t w[4];
                     key.block((uint32_t)i, TAG_ZBAR, 0, w);
-                    const float vl = cc[0] - 0.5f * qv[tid * 2] + gumbel_of<float>(w[0], w[1]);
-                    const float vr = cc[1] - 0.5f * qv[tid * 2 + 1] + gumbel_of<float>(w[2], w[3]);
+                    const float vl = cc[0] - 0.5f * q[0] + gumbel_of<float>(w[0], w[1]);
+                    const float vr = cc[1] - 0.5f * q[1] + gumbel_of<float>(w[2], w[3]);
                     h = vr > vl ? 1 : 0;
                     a.zbar[i] = (uint8_t)h;
                 } else {
                     h = a.zbar[i];
                 }
-                hq[tid] = (unsigned char)h;
+                hq[buf * WP + tid] = (unsigned char)h;
             }
+            __syncthreads();  // batch cur is ready for the statistics group, batch cur - 1 added up
+            cur = nx;
+            nx = n2;
         }
-        __syncthreads();
-        for (int r = 0; r < nr; ++r) {
-            const int qs = runs[r], qe = runs[r + 1];
-            const int k = kq[qs];
-            if (k != cur) {
-                if (cur >= 0) flush(cur);
-                cur = k;
-            }
+        __syncthreads();  // the last batch added up
+    } else {
+        // ------------------------------------------------------------ statistics group
+        const int t = tid - WIDE_S;
+        int J = 0, lb = t;  // rows 8 J .. 8 J + 7, columns 4 lb .. 4 lb + 3 (blocks 2 J <= lb, 2 J + 1 <= lb)
+        bool worker = true;
+        while (worker && lb >= nb - 2 * J) {
+            lb -= nb - 2 * J;
+            ++J;
+            worker = 2 * J < nb;
+        }
+        lb += 2 * J;
+        float acc0[32], acc1[32];
+#pragma unroll
+        for (int e = 0; e < 32; ++e) acc0[e] = acc1[e] = 0.f;
+        auto flush = [&](int k) {
             if (worker) {
-                for (int q = qs; q < qe; ++q) {
-                    const float* xr = xs + (size_t)q * dp;
-                    const float4 xj = *(const float4*)(xr + jb * 4);
-                    const float4 xl = *(const float4*)(xr + lb * 4);
-                    const float aj[4] = {xj.x, xj.y, xj.z, xj.w}, al[4] = {xl.x, xl.y, xl.z, xl.w};
-                    if (hq[q]) {
+                double* out = a.rec + (size_t)(g + k) * 2 * a.L.E;
 #pragma unroll
-                        for (int u = 0; u < 4; ++u)
+                for (int v = 0; v < 2; ++v) {
+                    const int jb = 2 * J + v;
+                    if (jb > lb || jb >= nb) continue;
+                    double* o = out + (size_t)a.L.blk(jb, lb) * 16;
 #pragma unroll
-                            for (int w2 = 0; w2 < 4; ++w2) acc1[u * 4 + w2] = fmaf(aj[u], al[w2], acc1[u * 4 + w2]);
-                    } else {
-#pragma unroll
-                        for (int u = 0; u < 4; ++u)
-#pragma unroll
-                            for (int w2 = 0; w2 < 4; ++w2) acc0[u * 4 + w2] = fmaf(aj[u], al[w2], acc0[u * 4 + w2]);
+                    for (int e = 0; e < 16; ++e) {
+                        o[e] = (double)acc0[16 * v + e];
+                        o[a.L.E + e] = (double)acc1[16 * v + e];
                     }
                 }
             }
+#pragma unroll
+            for (int e = 0; e < 32; ++e) acc0[e] = acc1[e] = 0.f;
+        };
+        Batch prev = cur;
+        for (bool more = cur.np > 0; more;) {
+            __syncthreads();  // batch prev is ready
+            next(cur);
+            more = cur.np > 0;
+            const float* xb = xs + (size_t)(prev.run % 3) * WP * dp;
+            const unsigned char* hb = hq + (prev.run % 3) * WP;
+            if (worker) {
+                for (int q = 0; q < prev.np; ++q) {
+                    const float* xr = xb + q * dp;
+                    const float4 j0 = *(const float4*)(xr + J * 8), j1 = *(const float4*)(xr + J * 8 + 4);
+                    const float4 xl = *(const float4*)(xr + lb * 4);
+                    const float aj[8] = {j0.x, j0.y, j0.z, j0.w, j1.x, j1.y, j1.z, j1.w}, al[4] = {xl.x, xl.y, xl.z, xl.w};
+                    if (hb[q]) {
+#pragma unroll
+                        for (int u = 0; u < 8; ++u)
+#pragma unroll
+                            for (int v = 0; v < 4; ++v) acc1[u * 4 + v] = fmaf(aj[u], al[v], acc1[u * 4 + v]);
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < 8; ++u)
+#pragma unroll
+                            for (int v = 0; v < 4; ++v) acc0[u * 4 + v] = fmaf(aj[u], al[v], acc0[u * 4 + v]);
+                    }
+                }
+            }
+            if (!more || cur.k != prev.k) flush(prev.k);
+            prev = cur;
         }
+        __syncthreads();
     }
-    if (cur >= 0) flush(cur);
 }
 
 // Multinomial variant (first-moment statistics only): the point's counts become a
@@ -2360,14 +2437,9 @@ static cudaError_t substats_mult_t(dpmm_ctx* c, uint64_t seed, int draw, const i
     return cudaGetLastError();
 }
 
-static size_t wide_smem(const dpmm_ctx* c) {
-    return ((size_t)2 * 128 * 128 + 128 * WP + (size_t)WP * c->st.dp + 2 * WP + 256 + 256 + 128 + 4) * 4 +
-           ((size_t)2 * WP + 2) * sizeof(int) + WP + 16;
-}
-
-template <typename XT>
-static cudaError_t substats_wide_t(dpmm_ctx* c, uint64_t seed, int draw, const int* gate) {
-    SubArgs<float> a;
+static cudaError_t substats_wide(dpmm_ctx* c, uint64_t seed, int draw, const int* gate) {
+    WideArgs w;
+    SubArgs<float>& a = w.a;
     a.kind = c->kind;
     a.d = c->d;
     a.xs = c->xs;
@@ -2388,11 +2460,11 @@ static cudaError_t substats_wide_t(dpmm_ctx* c, uint64_t seed, int draw, const i
     a.R = (c->N + c->Gr - 1) / c->Gr;
     a.L = c->st;
     a.rec = c->records;
-    const size_t smem = wide_smem(c);
-    cudaError_t ea = cudaFuncSetAttribute(substats_wide_kernel<XT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)smem);
+    w.starts = c->tot;
+    const size_t smem = wide_smem_of(c->st.dp);
+    cudaError_t ea = cudaFuncSetAttribute(substats_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (ea != cudaSuccess) return ea;
-    substats_wide_kernel<XT><<<c->Gr, WIDE_T, smem, c->stream>>>(a);
+    substats_wide_kernel<<<c->Gr, WIDE_T, smem, c->stream>>>(w);
     return cudaGetLastError();
 }
 
@@ -2455,7 +2527,7 @@ static cudaError_t substats_dispatch(dpmm_ctx* c, uint64_t seed, int draw, const
     else if (fast) e = c->xdt == 2 ? substats_f32_t<64, __nv_bfloat16>(c, seed, draw, gate)
                                    : substats_f32_t<64, float>(c, seed, draw, gate);
     else if (c->prec != DPMM_PREC_FP64_PLAIN && c->kind == DPMM_PRIOR_NIW && c->d <= 128 && c->st.nblk <= WIDE_T)
-        e = c->xdt == 2 ? substats_wide_t<__nv_bfloat16>(c, seed, draw, gate) : substats_wide_t<float>(c, seed, draw, gate);
+        e = substats_wide(c, seed, draw, gate);
     else if (c->prec == DPMM_PREC_FP64_PLAIN && c->kind == DPMM_PRIOR_NIW && c->d > 8) e = substats_niw64(c, seed, draw, gate);
     else if (c->prec == DPMM_PREC_FP64_PLAIN) e = substats_t<double, double>(c, seed, draw, gate);
     else if (c->xdt == 2) e = substats_t<float, __nv_bfloat16>(c, seed, draw, gate);
