@@ -272,6 +272,10 @@ struct dpmm_ctx {
     size_t tc_img_bytes = 0;
     void* tcs_img = nullptr;  // tensor-core sub-cluster factor images (K_max x 10 KB)
     void* x3_ximg = nullptr;  // split-BF16 point tiles (BF16X3), pre-swizzled
+    void* x3_xn = nullptr;    // screening (BF16X3, large N): per point |x_h|, |x_l|
+    void* x3_list = nullptr;  // the points it leaves open, their gathered tiles,
+    void* x3_cimg = nullptr;
+    void* x3_words = nullptr; // its words, then per cluster |W_h|, |W_l|, |mu|
     void* x3_fimg = nullptr;  // split-BF16 factor image (BF16X3), K_max clusters
     double* cweights = nullptr;  // K_max: pi_k of the last sweep (linear)
     double* eps = nullptr;       // 3 K_max x d: normals of the drawn means

@@ -25,6 +25,10 @@
 // the largest value an FP32 Gumbel can take reaches the best perturbed score so far, so
 // skipped clusters could not have won and the argmax is that of every draw.
 //
+// Large data are screened first (x3_screen_kernel): the single product x_h W_h encloses every
+// score, and the three products are formed only for the points whose label the enclosures
+// leave open, gathered into tiles of their own.
+//
 // CTA roles (320 threads):
 //   warp 0    : producer (bulk copies of the pre-swizzled point tiles and factor stages)
 //   warp 1    : TMEM allocation (512 columns) and the single-thread MMA issue
@@ -74,7 +78,13 @@ struct Args {
     int32_t* z;
     int* derr;
     double* scores;             // optional N x K scores (test hook), else null
+    // after a screening: the points left open (null: all points), their gathered tiles, and
+    // X3_* words
+    const int* list;
+    const unsigned char* cimg;
+    const int* words;
 };
+enum { X3_COUNT = 0, X3_SKIP = 1, X3_FULL = 2 };  // points left open; sweeps not to screen; score all points
 
 __device__ __noinline__ void gumbel_draw(uint64_t seed, uint32_t iter, uint32_t prob, uint32_t i, int k, float sc,
                                          float* best,
@@ -112,7 +122,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) labels_x3_kernel(Args a) {
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int K = *a.dK;
-    const int64_t ntiles = (a.N + BM - 1) / BM;
+    const bool part = a.list && !a.words[X3_FULL];
+    const int64_t N = part ? a.words[X3_COUNT] : a.N;
+    const unsigned char* ximg = part ? a.cimg : a.ximg;
+    if (N == 0) return;
+    const int64_t ntiles = (N + BM - 1) / BM;
     const int64_t npass = (ntiles + MT - 1) / MT;
 
     if (threadIdx.x == 0) {
@@ -160,7 +174,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) labels_x3_kernel(Args a) {
                 if (!tc::mbar_wait(xempty, (uint32_t)((it & 1) ^ 1), abort)) { ok = false; break; }
                 const uint32_t xb = (uint32_t)MT * g.xtile;
                 tc::mbar_expect_tx(xfull, xb);
-                const unsigned char* src = a.ximg + (size_t)t * xb;
+                const unsigned char* src = ximg + (size_t)t * xb;
                 for (uint32_t off = 0; off < xb; off += 32768u)
                     tc::bulk_load(xs + off, src + off, min(32768u, xb - off), xfull);
                 for (int k = 0; k < K && ok; ++k) {
@@ -243,7 +257,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) labels_x3_kernel(Args a) {
         uint32_t cc = 0;
         bool ok = true;
         for (int64_t t = blockIdx.x; t < npass && ok; t += gridDim.x) {
-            const int64_t i = (t * MT + mt) * BM + r;
+            const int64_t pos = (t * MT + mt) * BM + r;
+            const int64_t i = part ? (pos < N ? a.list[pos] : a.N) : pos;
             float best = -INFINITY;
             int zb = 0;
             for (int k = 0; k < K; ++k, ++cc) {
@@ -252,10 +267,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) labels_x3_kernel(Args a) {
                 tc::fence_after();
                 const uint32_t ta = tmem + lane_off + (uint32_t)b * ncols + (uint32_t)(mt * g.dp);
                 float q = 0.f;
-                for (int c0 = 0; c0 < g.dp; c0 += 64) {
-                    float ya[32], yb[32];
-                    tc::tmem_ld32x2(ta + (uint32_t)c0, ta + (uint32_t)(c0 + 32), ya, yb);
-                    q += tc::sqsum32(ya) + tc::sqsum32(yb);
+#pragma unroll 1
+                for (int c0 = 0; c0 < g.dp; c0 += 64) {  // one block's 32 values at a time: no spills
+                    float y[32];
+                    tc::tmem_ld32(ta + (uint32_t)c0, y);
+                    const float qa = tc::sqsum32(y);
+                    tc::tmem_ld32(ta + (uint32_t)(c0 + 32), y);
+                    q += qa + tc::sqsum32(y);
                 }
                 tc::fence_before();
                 tc::mbar_arrive(&tempty[b]);
@@ -280,6 +298,304 @@ __global__ void __launch_bounds__(NTHREADS, 1) labels_x3_kernel(Args a) {
     if (*abort && warp == 1) __nanosleep(1000000);
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+}
+
+// ------------------------------------------------------------------ screening
+// The label step for large data: y' = x_h W_h - b, one product of the three, encloses every
+// score.  With |.| Euclidean (Frobenius) norms, the terms left out are at most
+//   E = |x_l| |W_h| + |x_h| |W_l| + 1e-4 (|x_h| + |mu|) |W_h|
+// in the norm of y: Cauchy-Schwarz, and 1e-4 for the FP32 accumulations of this kernel and of the
+// full one (36 tensor-core steps, each off by at most 2^-21 of the largest partial sum, which is
+// at most (|x| + |mu|) |W|).  So c_k - (|y'| + E)^2 / 2 <= s_ik <= c_k - max(0, |y'| - E)^2 / 2, and
+// a point is decided when the largest upper bound of the others plus the largest Gumbel value
+// is below the best lower bound plus the smallest: its label is that cluster whatever is drawn.
+// The points left open are listed for labels_x3_kernel.
+//
+// What bounds it: the tensor cores' shared-memory reads (M = N = 128: 8 KB for 64 cycles of MMA)
+// and the factors' traffic from L2, so a pass holds MT = 4 point tiles (x_h only) per factor
+// stage, each tile with an accumulator buffer of its own.  Same roles as labels_x3_kernel; an
+// epilogue warp takes tiles g and g + 2 of its TMEM lane quarter.
+// Measured at d = 128, K = 64, N = 4e6: 7.95 ms for the whole label step, 1.2 PFLOP/s (19.9 ms
+// with the three products for every point; 12.7 ms with two blocks of 32 accumulators in
+// registers at once, which spilled).
+constexpr int SMT = 4;
+constexpr int SG = 2;              // epilogue groups of four warps (4: the same time)
+constexpr int STHREADS = 32 * (2 + 4 * SG);
+constexpr int SJ = SMT / SG;       // tiles of a group
+struct ScreenArgs {
+    int64_t N;
+    Geo g;
+    int Kmax, fst;
+    const int* dK;
+    const unsigned char *ximg, *fimg;
+    const float* qc;      // c_k at slot 3k
+    const float4* kn;     // per cluster: |W_h|, |W_l|, |mu|
+    const float2* xn;     // per point: |x_h|, |x_l|
+    int32_t* z;
+    int* list;
+    int* words;
+    int* derr;
+};
+
+__global__ void __launch_bounds__(STHREADS, 1) x3_screen_kernel(ScreenArgs a) {
+    extern __shared__ __align__(1024) unsigned char smraw[];
+    if (a.words[X3_SKIP] > 0) return;
+    unsigned char* base = (unsigned char*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
+    const Geo g = a.g;
+    const uint32_t xhalf = g.xtile / 2;                         // x_h of one tile
+    unsigned char* xs = base;                                   // SMT x xhalf
+    unsigned char* fs = xs + (size_t)SMT * xhalf;               // fst x sbytes
+    __nv_bfloat16* ones = (__nv_bfloat16*)(fs + (size_t)a.fst * g.sbytes);  // BM rows x 16, no swizzle
+    float4* ct = (float4*)(ones + BM * 16);                     // Kmax: c, and E = x |x_l| + y |x_h| + w
+    uint64_t* bars = (uint64_t*)(ct + a.Kmax);
+    uint64_t* xfull = bars;              // 1
+    uint64_t* xempty = xfull + 1;        // 1
+    uint64_t* ffull = xempty + 1;        // fst
+    uint64_t* fempty = ffull + FSTMAX;   // fst
+    uint64_t* tfull = fempty + FSTMAX;   // SMT
+    uint64_t* tempty = tfull + SMT;      // SMT
+    __shared__ uint32_t tmem_base;
+    __shared__ int abort_flag;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int K = *a.dK;
+    const int64_t npass = ((a.N + BM - 1) / BM + SMT - 1) / SMT;
+
+    if (threadIdx.x == 0) {
+        abort_flag = 0;
+        mbar_init(xfull, 1);
+        mbar_init(xempty, 1);
+        for (int s = 0; s < a.fst; ++s) {
+            mbar_init(&ffull[s], 1);
+            mbar_init(&fempty[s], 1);
+        }
+        for (int b = 0; b < SMT; ++b) {
+            mbar_init(&tfull[b], 1);
+            mbar_init(&tempty[b], 4 * 32);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc::saddr(&tmem_base)),
+                     "r"(TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    for (int e = threadIdx.x; e < BM * 16; e += blockDim.x) {  // as in labels_x3_kernel
+        const int m = e >> 4, kk = e & 15;
+        ones[(m >> 3) * 128 + (kk >> 3) * 64 + (m & 7) * 8 + (kk & 7)] = __float2bfloat16_rn(kk < 3 ? 1.f : 0.f);
+    }
+    for (int k = threadIdx.x; k < K; k += blockDim.x) {
+        const float4 n = a.kn[k];
+        ct[k] = make_float4(a.qc[3 * k], n.x, n.y + 1e-4f * n.x, 1e-4f * n.z * n.x);
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    const uint32_t tmem = tmem_base;
+    volatile int* abort = &abort_flag;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int64_t it = 0;
+            uint32_t pc = 0;
+            bool ok = true;
+            for (int64_t t = blockIdx.x; t < npass && ok; t += gridDim.x, ++it) {
+                if (!tc::mbar_wait(xempty, (uint32_t)((it & 1) ^ 1), abort)) { ok = false; break; }
+                tc::mbar_expect_tx(xfull, SMT * xhalf);
+                for (int mt = 0; mt < SMT; ++mt) {
+                    const unsigned char* src = a.ximg + (size_t)(t * SMT + mt) * g.xtile;
+                    for (uint32_t off = 0; off < xhalf; off += 32768u)
+                        tc::bulk_load(xs + (size_t)mt * xhalf + off, src + off, min(32768u, xhalf - off), xfull);
+                }
+                for (int k = 0; k < K; ++k, ++pc) {  // W_h and -b of every cluster
+                    const int s = (int)(pc % (uint32_t)a.fst);
+                    if (!tc::mbar_wait(&fempty[s], ((pc / (uint32_t)a.fst) & 1u) ^ 1u, abort)) { ok = false; break; }
+                    tc::mbar_expect_tx(&ffull[s], g.sbytes);
+                    const unsigned char* src = a.fimg + (size_t)k * g.cbytes;
+                    for (uint32_t off = 0; off < g.sbytes; off += 32768u)
+                        tc::bulk_load(fs + (size_t)s * g.sbytes + off, src + off, min(32768u, g.sbytes - off), &ffull[s]);
+                }
+            }
+            if (!ok) {
+                atomicExch(a.derr, (int)DPMM_ETIMEOUT);
+                *abort = 1;
+            }
+            // own copies must land before the CTA may exit
+            if (it > 0) tc::mbar_wait(xfull, (uint32_t)((it - 1) & 1), abort);
+            const uint32_t f = (uint32_t)a.fst;
+            for (uint32_t j = (pc > f ? pc - f : 0); j < pc; ++j) tc::mbar_wait(&ffull[j % f], (j / f) & 1u, abort);
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            const uint32_t id = tc::idesc(g.dp, 1);
+            int64_t it = 0;
+            uint32_t pc = 0;
+            bool ok = true;
+            for (int64_t t = blockIdx.x; t < npass && ok; t += gridDim.x, ++it) {
+                if (!tc::mbar_wait(xfull, (uint32_t)(it & 1), abort)) { ok = false; break; }
+                tc::fence_after();
+                const uint32_t xa = tc::saddr(xs);
+                for (int k = 0; k < K && ok; ++k, ++pc) {
+                    const int s = (int)(pc % (uint32_t)a.fst);
+                    if (!tc::mbar_wait(&ffull[s], (pc / (uint32_t)a.fst) & 1u, abort)) { ok = false; break; }
+                    const uint32_t fa = tc::saddr(fs + (size_t)s * g.sbytes);
+                    for (int mt = 0; mt < SMT; ++mt) {
+                        if (!tc::mbar_wait(&tempty[mt], (pc & 1u) ^ 1u, abort)) { ok = false; break; }
+                        tc::fence_after();
+                        const uint32_t dt = tmem + (uint32_t)(mt * g.dp), xh = xa + (uint32_t)mt * xhalf;
+                        for (int kb = 0; kb < g.KB; ++kb)
+#pragma unroll
+                            for (int kk = 0; kk < 4; ++kk)
+                                tc::mma<1>(dt, tc::sdesc(xh + kb * XBLK + kk * 32),
+                                           tc::sdesc(fa + (uint32_t)kb * (uint32_t)(g.dp * 128) + kk * 32), id, (kb | kk) != 0);
+                        tc::mma<1>(dt, tc::sdesc_ns(tc::saddr(ones)), tc::sdesc_ns(fa + g.wbytes), id, 1u);
+                        tc::mma_commit(&tfull[mt]);
+                    }
+                    if (!ok) break;
+                    tc::mma_commit(&fempty[s]);
+                }
+                if (!ok) break;
+                tc::mma_commit(xempty);
+            }
+            if (!ok) {
+                atomicExch(a.derr, (int)DPMM_ETIMEOUT);
+                *abort = 1;
+            }
+        }
+        __syncwarp();
+    } else {
+        const int grp = (warp - 2) >> 2, quarter = warp & 3;
+        const int r = quarter * 32 + lane;
+        const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
+        uint32_t pc = 0;
+        bool ok = true;
+        for (int64_t t = blockIdx.x; t < npass && ok; t += gridDim.x) {
+            int64_t i[SJ];
+            float2 xn[SJ];
+            float Lb[SJ], Ub[SJ], U2[SJ];  // best lower bound, its cluster's upper one, the largest of the others
+            int kb[SJ];
+#pragma unroll
+            for (int j = 0; j < SJ; ++j) {
+                i[j] = (t * SMT + grp + SG * j) * BM + r;
+                xn[j] = i[j] < a.N ? a.xn[i[j]] : make_float2(0.f, 0.f);
+                Lb[j] = Ub[j] = U2[j] = -INFINITY;
+                kb[j] = 0;
+            }
+            for (int k = 0; k < K && ok; ++k, ++pc) {
+                const float4 c = ct[k];
+#pragma unroll
+                for (int j = 0; j < SJ; ++j) {
+                    const int mt = grp + SG * j;
+                    ok = __all_sync(0xffffffffu, tc::mbar_wait(&tfull[mt], pc & 1u, abort));
+                    if (!ok) break;
+                    tc::fence_after();
+                    const uint32_t ta = tmem + lane_off + (uint32_t)(mt * g.dp);
+                    float q = 0.f;
+#pragma unroll 1
+                    for (int c0 = 0; c0 < g.dp; c0 += 32) {
+                        float y[32];
+                        tc::tmem_ld32(ta + (uint32_t)c0, y);
+                        q += tc::sqsum32(y);
+                    }
+                    tc::fence_before();
+                    tc::mbar_arrive(&tempty[mt]);
+                    float y;
+                    asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(q));
+                    const float E = fmaf(c.y, xn[j].y, fmaf(c.z, xn[j].x, c.w)) + 2e-5f * y;  // and the sum's rounding
+                    const float lo = fmaxf(y - E, 0.f), hi = y + E, slack = 1e-2f + 1e-6f * (fabsf(c.x) + q);
+                    const float U = c.x - 0.5f * lo * lo + slack, L = c.x - 0.5f * hi * hi - slack;
+                    if (!(c.x > -INFINITY)) continue;  // weight zero: never a label
+                    if (L > Lb[j]) {
+                        U2[j] = fmaxf(U2[j], Ub[j]);
+                        Lb[j] = L;
+                        Ub[j] = U;
+                        kb[j] = k;
+                    } else if (!(U <= U2[j])) {  // a NaN stays and leaves the point open
+                        U2[j] = U;
+                    }
+                }
+            }
+            if (!ok) break;
+#pragma unroll
+            for (int j = 0; j < SJ; ++j) {
+                // FP32 Gumbel values lie in [-2.82, 16.64]
+                const bool open = i[j] < a.N && !(U2[j] + 17.5f < Lb[j] - 3.f);
+                if (i[j] < a.N && !open) a.z[i[j]] = kb[j];
+                const unsigned m = __ballot_sync(0xffffffffu, open);
+                if (m) {
+                    int at = 0;
+                    if (lane == 0) at = atomicAdd(a.words + X3_COUNT, __popc(m));
+                    at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+                    if (open) a.list[at] = (int)i[j];
+                }
+            }
+        }
+        if (!ok) {
+            atomicExch(a.derr, (int)DPMM_ETIMEOUT);
+            *abort = 1;
+        }
+    }
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    if (*abort && warp == 1) __nanosleep(1000000);
+    if (warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+}
+
+// The rows left open, gathered into tiles of their own (rows up to the last pass's end are zero), or,
+// when there are more than cap, the word that has all points scored; the screening is then left
+// out for 15 sweeps (its enclosures are too wide for these clusters), which changes no label.
+__global__ void x3_gather_kernel(Geo g, const unsigned char* ximg, const int* list, int cap, int* words, unsigned char* cimg) {
+    const int skip = words[X3_SKIP], n = words[X3_COUNT];
+    const bool full = skip > 0 || n > cap;
+    __shared__ int s_last;
+    if (!full) {
+        const int64_t rows = (n + MT * BM - 1) / (MT * BM) * (int64_t)(MT * BM);
+        const int nh = 2 * g.KB;  // 64-feature blocks of a row, x_h then x_l
+        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < rows * nh * 8; e += (int64_t)gridDim.x * blockDim.x) {
+            const int c = (int)(e & 7), hb = (int)((e >> 3) % nh);
+            const int64_t q = (e >> 3) / nh;
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (q < n) {
+                const int i = list[q], rs = i % BM;
+                v = *(const uint4*)(ximg + (size_t)(i / BM) * g.xtile + (size_t)hb * XBLK + rs * 128 + ((c ^ (rs & 7)) << 4));
+            }
+            const int rd = (int)(q % BM);
+            *(uint4*)(cimg + (size_t)(q / BM) * g.xtile + (size_t)hb * XBLK + rd * 128 + ((c ^ (rd & 7)) << 4)) = v;
+        }
+    }
+    // the block that is last to get here, when every block has read the words, writes them
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(words + 3, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (s_last && threadIdx.x == 0) {
+        words[3] = 0;
+        words[X3_FULL] = full;
+        words[X3_SKIP] = skip > 0 ? skip - 1 : full ? 15 : 0;
+    }
+}
+
+// |x_h| and |x_l| of every point (rounded up), one warp per row
+__global__ void x3_norm_kernel(const float* X, int64_t N, int d, int xs, float2* xn) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < N; i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        float h2 = 0.f, l2 = 0.f;
+        for (int j = lane; j < d; j += 32) {
+            const float x = X[i * xs + j], h = __bfloat162float(__float2bfloat16_rn(x));
+            const float l = __bfloat162float(__float2bfloat16_rn(x - h));
+            h2 = fmaf(h, h, h2);
+            l2 = fmaf(l, l, l2);
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            h2 += __shfl_xor_sync(0xffffffffu, h2, o);
+            l2 += __shfl_xor_sync(0xffffffffu, l2, o);
+        }
+        if (lane == 0) xn[i] = make_float2(sqrtf(h2) * 1.0001f, sqrtf(l2) * 1.0001f);
+    }
 }
 
 // Point tiles: tile T, half h (0: x_h, 1: x_l), 64-feature block kb, row r, feature
@@ -311,9 +627,38 @@ __global__ void x3_points_kernel(const float* X, int64_t N, int d, int xs, Geo g
 // element (j, kk) at (j / 8) * 256 + (kk / 8) * 128 + (j % 8) * 16 + (kk % 8) * 2) holds the
 // three BF16 parts of -b_j, b_j = sum_m mu_m (W_h + W_l)[m][j] formed in FP64 with the
 // factor as the tensor cores see it.
+// Then the norms |W_h|, |W_l|, |mu| (rounded up) of cluster k into kn[k], where kn is given.
 __global__ void x3_factor_kernel(const int* dK, int Kmax, int d, Geo g, const double* pW, const double* pmu,
-                                 unsigned char* img) {
+                                 unsigned char* img, float4* kn) {
     const int K = min(*dK, Kmax);
+    for (int k = blockIdx.x; kn && k < K; k += gridDim.x) {
+        __shared__ float part[3][8];
+        const double* W = pW + (size_t)3 * k * d * d;
+        float v[3] = {0.f, 0.f, 0.f};
+        for (int e = threadIdx.x; e < d * d; e += blockDim.x) {
+            const double w = W[e];
+            const float h = __bfloat162float(__float2bfloat16_rn((float)w));
+            const float l = __bfloat162float(__float2bfloat16_rn((float)(w - (double)h)));
+            v[0] = fmaf(h, h, v[0]);
+            v[1] = fmaf(l, l, v[1]);
+        }
+        for (int j = threadIdx.x; j < d; j += blockDim.x) {
+            const float m = (float)pmu[(size_t)3 * k * d + j];
+            v[2] = fmaf(m, m, v[2]);
+        }
+        for (int u = 0; u < 3; ++u) {
+            for (int o = 16; o > 0; o >>= 1) v[u] += __shfl_xor_sync(0xffffffffu, v[u], o);
+            if ((threadIdx.x & 31) == 0) part[u][threadIdx.x >> 5] = v[u];
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            float t[3] = {0.f, 0.f, 0.f};
+            for (int u = 0; u < 3; ++u)
+                for (int w = 0; w < 8; ++w) t[u] += part[u][w];
+            kn[k] = make_float4(sqrtf(t[0]) * 1.0001f, sqrtf(t[1]) * 1.0001f, sqrtf(t[2]) * 1.0001f, 0.f);
+        }
+        __syncthreads();
+    }
     const int64_t per_k = (int64_t)2 * g.KB * g.dp * 64 + g.dp;
     const int64_t total = (int64_t)K * per_k;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
@@ -384,8 +729,16 @@ bool x3_supported(const dpmm_ctx* c) {
 
 static int64_t x3_ntile_pad(const dpmm_ctx* c) {
     const int64_t ntiles = (c->N + 127) / 128;
-    return (ntiles + x3::MT - 1) / x3::MT * x3::MT;
+    return (ntiles + x3::SMT - 1) / x3::SMT * x3::SMT;
 }
+
+// Screening pays where the label step is long beside two more launches (from 65,536 points
+// at d > 64, 262,144 below).
+static bool x3_screened(const dpmm_ctx* c) {
+    const int64_t dp = c->d <= 64 ? 64 : 128;
+    return c->N * dp * dp >= (int64_t)1 << 30 && c->N <= 0x7FFFFFFF;
+}
+static int x3_cap(const dpmm_ctx* c) { return (int)(c->N / 8); }  // points that the gathered tiles hold
 
 // after the data are stored (centred FP32): allocate the point and factor images and
 // split the points into their BF16 parts
@@ -404,17 +757,32 @@ cudaError_t x3_prepare_data(dpmm_ctx* c) {
         e = cudaMemsetAsync(c->x3_fimg, 0, (size_t)c->K_max * g.cbytes, c->stream);
         if (e != cudaSuccess) return e;
     }
+    if (x3_screened(c)) {
+        const int64_t ct = (x3_cap(c) + 127) / 128 + x3::MT;
+        cudaError_t e = cudaSuccess;
+        if (!c->x3_xn) {
+            e = cudaMalloc(&c->x3_xn, sizeof(float2) * c->N);
+            if (e == cudaSuccess) e = cudaMalloc(&c->x3_list, sizeof(int) * c->N);
+            if (e == cudaSuccess) e = cudaMalloc(&c->x3_cimg, (size_t)ct * g.xtile);
+        }
+        if (e == cudaSuccess && !c->x3_words) e = cudaMalloc(&c->x3_words, 4 * sizeof(int) + sizeof(float4) * c->K_max);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->x3_words, 0, 4 * sizeof(int) + sizeof(float4) * c->K_max, c->stream);
+        if (e != cudaSuccess) return e;
+        x3::x3_norm_kernel<<<8 * c->num_sms, 256, 0, c->stream>>>((const float*)c->X, c->N, c->d, c->xs, (float2*)c->x3_xn);
+    }
     x3::x3_points_kernel<<<4 * c->num_sms, 256, 0, c->stream>>>((const float*)c->X, c->N, c->d, c->xs, g, nt,
                                                                 (unsigned char*)c->x3_ximg);
     return cudaGetLastError();
 }
+
+static float4* x3_kn(const dpmm_ctx* c) { return c->x3_words && x3_screened(c) ? (float4*)((int*)c->x3_words + 4) : nullptr; }
 
 // per sweep, after the parameters are drawn: the factor image
 cudaError_t x3_prepare(dpmm_ctx* c) {
     if (!c->x3_fimg) return cudaErrorNotSupported;
     const x3::Geo g = x3_geo(c, nullptr);
     x3::x3_factor_kernel<<<2 * c->num_sms, 256, 0, c->stream>>>(c->dK, c->K_max, c->d, g, c->p_W, c->p_mu,
-                                                                (unsigned char*)c->x3_fimg);
+                                                                (unsigned char*)c->x3_fimg, x3_kn(c));
     c->nlaunch += 1;
     return cudaGetLastError();
 }
@@ -440,9 +808,44 @@ cudaError_t launch_labels_x3(dpmm_ctx* c, uint64_t seed) {
     auto kern = a.scores ? x3::labels_x3_kernel<true> : x3::labels_x3_kernel<false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
+    a.list = nullptr;
+    a.cimg = nullptr;
+    a.words = nullptr;
     const int64_t npass = x3_ntile_pad(c) / x3::MT;
     const int grid = (int)std::min<int64_t>(c->num_sms, npass);
     prof_begin(c, "labels_x3");
+    if (!a.scores && c->x3_words && x3_screened(c)) {
+        int* words = (int*)c->x3_words;
+        x3::ScreenArgs b;
+        b.N = c->N;
+        b.g = g;
+        b.Kmax = c->K_max;
+        b.dK = c->dK;
+        b.ximg = a.ximg;
+        b.fimg = a.fimg;
+        b.qc = c->q_c;
+        b.kn = x3_kn(c);
+        b.xn = (const float2*)c->x3_xn;
+        b.z = c->z;
+        b.list = (int*)c->x3_list;
+        b.words = words;
+        b.derr = c->derr;
+        const size_t fixed = 1024 + (size_t)x3::SMT * g.xtile / 2 + (size_t)tc::BM * 16 * 2 + (size_t)c->K_max * 16 +
+                             (size_t)(2 + 2 * x3::FSTMAX + 2 * x3::SMT) * 8;
+        b.fst = (int)std::min<size_t>(x3::FSTMAX, (227 * 1024 - 2048 - fixed) / g.sbytes);
+        if (b.fst < 2) return cudaErrorNotSupported;
+        const size_t sm = fixed + (size_t)b.fst * g.sbytes;
+        e = cudaFuncSetAttribute(x3::x3_screen_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e == cudaSuccess) e = cudaMemsetAsync(words + x3::X3_COUNT, 0, sizeof(int), c->stream);
+        if (e != cudaSuccess) return e;
+        x3::x3_screen_kernel<<<(int)std::min<int64_t>(c->num_sms, x3_ntile_pad(c) / x3::SMT), x3::STHREADS, sm, c->stream>>>(b);
+        x3::x3_gather_kernel<<<2 * c->num_sms, 256, 0, c->stream>>>(g, a.ximg, b.list, x3_cap(c), words,
+                                                                    (unsigned char*)c->x3_cimg);
+        c->nlaunch += 2;
+        a.list = b.list;
+        a.cimg = (const unsigned char*)c->x3_cimg;
+        a.words = words;
+    }
     kern<<<grid, x3::NTHREADS, smem, c->stream>>>(a);
     prof_end(c, "labels_x3");
     c->nlaunch += 1;
