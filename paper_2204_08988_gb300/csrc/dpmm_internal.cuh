@@ -321,6 +321,11 @@ struct dpmm_ctx {
     double* sp_lgb = nullptr;      // lgamma(beta_j)
     void* sp_part = nullptr;       // 3 K_max x ceil(d / 2048) (max, sum exp) of the FP32 theta draws
 
+    // getters: unpacked statistics (device), the chain's words (page-locked host memory)
+    double* unpack = nullptr;
+    size_t unpack_bytes = 0;
+    int* pub = nullptr;
+
     // point-sharded chains: this context's first point in the whole data set
     int64_t poff = 0;
     void* shard_scratch = nullptr; // the summed statistics of a sharded sweep (shard 0)
