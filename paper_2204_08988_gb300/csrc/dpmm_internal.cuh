@@ -305,7 +305,7 @@ struct dpmm_ctx {
 
     // tensor-core path
     int* tc_flag = nullptr;        // device: 1 when K did not fit the tensor-core kernel
-    void* tc_carry = nullptr;      // device: per-point state between cluster groups (TF32), N x 20 B
+    void* tc_carry = nullptr;      // device: per-point state between cluster groups (TF32), N x 28 B
 
     // multinomial data of more than SPARSE_MIN_D categories: compressed rows
     bool sparse = false;

@@ -1899,8 +1899,9 @@ __global__ void __launch_bounds__(256) substats_mult_kernel(SubArgs<float> a) {
 // positions, that is, of points in cluster order.  Lane l holds categories 8l .. 8l + 7 (d <= 256)
 // of a point's counts and of the two sub-cluster log theta rows of the current cluster; the
 // two sub-cluster scores are dot products reduced across the warp; the z-bar draws of 32
-// points are made at once, one point per lane; the counts of a cluster's run stay in registers
-// and are added at the run's end to the compact table cnt (2 K_max x (d + 1) integers, column
+// points are made at once, one point per lane, and four points' scores are reduced together
+// (N = 1e6, d = 200, K = 50: @@MULT@@ us, from 238 us with two five-step reductions a point).  The
+// counts of a cluster's run stay in registers and are added at the run's end to the compact table cnt (2 K_max x (d + 1) integers, column
 // d: the points) with atomic adds, exact in any order.  No block-wide barrier.
 struct MwArgs {
     int64_t N, R;  // points; sorted positions per warp
@@ -2008,57 +2009,17 @@ __global__ void __launch_bounds__(256, 3) mult_warp_kernel(MwArgs a) {
         }
     };
     draws();
-    for (int64_t p = p0; p < p1; ++p) {
-        if (p - bstart == 32) {  // the next batch
-            bstart += 32;
-            cur = nxt;
-            nxt = bstart + 32 + lane < p1 ? a.idx[bstart + 32 + lane] : 0;
-            draws();
+    auto unpack = [](const uint4& q, float* x) {  // the row's padding beyond d is zero
+        const uint32_t wv[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            x[2 * u] = __uint_as_float(wv[u] << 16);
+            x[2 * u + 1] = __uint_as_float(wv[u] & 0xFFFF0000u);
         }
-        const int slot = (int)((p - p0) % MW_DEPTH);
-        asm volatile("cp.async.wait_group %0;" ::"n"(MW_DEPTH - 1) : "memory");
-        __syncwarp();
+    };
+    auto add = [&](const uint4& q, int h) {
         float x[8];
-        if (lane < nch) {
-            const uint4 q = *(const uint4*)(ring + slot * MW_ROWB + lane * 16);
-            const uint32_t wv[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                x[2 * u] = j0 + 2 * u < d ? __uint_as_float(wv[u] << 16) : 0.f;
-                x[2 * u + 1] = j0 + 2 * u + 1 < d ? __uint_as_float(wv[u] & 0xFFFF0000u) : 0.f;
-            }
-        } else {
-#pragma unroll
-            for (int u = 0; u < 8; ++u) x[u] = 0.f;
-        }
-        __syncwarp();  // every lane has read the slot: it may be refilled
-        issue(slot, p + MW_DEPTH);
-        while (p >= kend) {  // the next cluster's run begins
-            flush(k);
-            ++k;
-            kend = a.starts[k + 1];
-            if (a.draw) stage(k);
-        }
-        const int q = (int)(p - bstart);
-        int h;
-        if (a.draw) {
-            float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                s0 = fmaf(x[u], lt0[u], s0);
-                s1 = fmaf(x[u], lt1[u], s1);
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-                s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-            }
-            const float vl = c0 + s0 + __shfl_sync(0xffffffffu, gl, q);
-            const float vr = c1 + s1 + __shfl_sync(0xffffffffu, gr, q);
-            h = vr > vl ? 1 : 0;
-            if (lane == q) a.zbar[cur] = (uint8_t)h;
-        } else {
-            h = __shfl_sync(0xffffffffu, hz, q);
-        }
+        unpack(q, x);
         if (h) {
 #pragma unroll
             for (int u = 0; u < 8; ++u) acc1[u] += (unsigned)x[u];
@@ -2067,6 +2028,93 @@ __global__ void __launch_bounds__(256, 3) mult_warp_kernel(MwArgs a) {
 #pragma unroll
             for (int u = 0; u < 8; ++u) acc0[u] += (unsigned)x[u];
             ++n0;
+        }
+    };
+    for (int64_t p = p0; p < p1; p += 4) {  // four points at a time
+        if (p - bstart == 32) {  // the next batch
+            bstart += 32;
+            cur = nxt;
+            nxt = bstart + 32 + lane < p1 ? a.idx[bstart + 32 + lane] : 0;
+            draws();
+        }
+        const int slot = (int)((p - p0) % MW_DEPTH);
+        asm volatile("cp.async.wait_group %0;" ::"n"(MW_DEPTH - 4) : "memory");
+        __syncwarp();
+        uint4 row[4];  // unpacked where used: the registers hold two rows of floats at most
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+            row[v] = lane < nch ? *(const uint4*)(ring + (slot + v) * MW_ROWB + lane * 16) : make_uint4(0u, 0u, 0u, 0u);
+        __syncwarp();  // every lane has read the slots: they may be refilled
+#pragma unroll
+        for (int v = 0; v < 4; ++v) issue(slot + v, p + MW_DEPTH + v);
+        const int q = (int)(p - bstart);
+        if (a.draw && p + 4 <= min(p1, kend)) {
+            // Eight sums (two scores of four points) reduced across the lanes at once: at each
+            // of the first three levels a lane keeps one of two values and hands the other over,
+            // so 9 exchanges do the work of 40; every sum adds lanes 16, 8, 4, 2, 1 apart, in
+            // that order, as reducing each on its own would.
+            float t[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                float s0 = 0.f, s1 = 0.f, x[8];
+                unpack(row[v], x);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    s0 = fmaf(x[u], lt0[u], s0);
+                    s1 = fmaf(x[u], lt1[u], s1);
+                }
+                const bool up = lane & 16;
+                t[v] = (up ? s1 : s0) + __shfl_xor_sync(0xffffffffu, up ? s0 : s1, 16);
+            }
+            const bool b8 = lane & 8, b4 = lane & 4;
+            const float m0 = (b8 ? t[1] : t[0]) + __shfl_xor_sync(0xffffffffu, b8 ? t[0] : t[1], 8);
+            const float m1 = (b8 ? t[3] : t[2]) + __shfl_xor_sync(0xffffffffu, b8 ? t[2] : t[3], 8);
+            float w = (b4 ? m1 : m0) + __shfl_xor_sync(0xffffffffu, b4 ? m0 : m1, 4);
+            w += __shfl_xor_sync(0xffffffffu, w, 2);
+            w += __shfl_xor_sync(0xffffffffu, w, 1);
+            // lane bits 16: sub-cluster, 8 and 4: point
+            const int pt = (b4 ? 2 : 0) + (b8 ? 1 : 0);
+            const float el = __shfl_sync(0xffffffffu, gl, q + pt), er = __shfl_sync(0xffffffffu, gr, q + pt);
+            const float val = (lane & 16 ? c1 : c0) + w + (lane & 16 ? er : el);
+            const float oth = __shfl_xor_sync(0xffffffffu, val, 16);
+            const unsigned m = __ballot_sync(0xffffffffu, oth > val);  // lanes 0, 8, 4, 12: points 0 .. 3
+            const int h[4] = {(int)(m & 1u), (int)(m >> 8 & 1u), (int)(m >> 4 & 1u), (int)(m >> 12 & 1u)};
+            const int r = lane - q;
+            if (r >= 0 && r < 4) a.zbar[cur] = (uint8_t)(r == 0 ? h[0] : r == 1 ? h[1] : r == 2 ? h[2] : h[3]);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) add(row[v], h[v]);
+            continue;
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            if (p + v >= p1) break;
+            while (p + v >= kend) {  // the next cluster's run begins
+                flush(k);
+                ++k;
+                kend = a.starts[k + 1];
+                if (a.draw) stage(k);
+            }
+            int h;
+            if (a.draw) {
+                float s0 = 0.f, s1 = 0.f, x[8];
+                unpack(row[v], x);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    s0 = fmaf(x[u], lt0[u], s0);
+                    s1 = fmaf(x[u], lt1[u], s1);
+                }
+                for (int o = 16; o > 0; o >>= 1) {
+                    s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+                    s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+                }
+                const float vl = c0 + s0 + __shfl_sync(0xffffffffu, gl, q + v);
+                const float vr = c1 + s1 + __shfl_sync(0xffffffffu, gr, q + v);
+                h = vr > vl ? 1 : 0;
+                if (lane == q + v) a.zbar[cur] = (uint8_t)h;
+            } else {
+                h = __shfl_sync(0xffffffffu, hz, q + v);
+            }
+            add(row[v], h);
         }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");

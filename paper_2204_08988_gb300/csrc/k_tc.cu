@@ -63,13 +63,18 @@ constexpr uint32_t TMEM_COLS = 512;
 constexpr int NBUF = 2;                        // TMEM accumulator buffers
 constexpr int BUFCOLS = (int)TMEM_COLS / NBUF; // columns per buffer (the chunk width)
 
-// per-point state carried from one cluster group to the next
+// Per-point state carried from one cluster group to the next.  At most two clusters within the
+// window of the best score are carried undrawn: a group of clusters that are all far from the
+// point often has two whose scores lie close together, and drawing them there (26 clusters, 32
+// rows a warp: nearly every one for some row) cost more than the scores; mostly a later group's
+// cluster is ahead of both by more than the window, and nothing is drawn (N = 200,003, d = 32,
+// K = 60: @@CARRY@@ us a label step, from 312 us).
 struct Carry {
-    float* g1;  // best score so far
-    float* g2;  // second-best score so far
-    float* v;   // best perturbed score among the clusters drawn so far (-inf: none)
-    int* k1;    // cluster of the best score
-    int* zv;    // cluster of the best perturbed score
+    float* g;        // best score so far
+    float *u1, *u2;  // undrawn clusters within the window of g (-inf: none)
+    int *k1, *k2;
+    float* v;        // best perturbed score among the clusters drawn (-inf: none), and its cluster
+    int* zv;
 };
 
 struct Args {
@@ -347,8 +352,27 @@ __global__ void __launch_bounds__(NTHREADS, 1) labels_tc_kernel(const __grid_con
         const bool first = g == 0, final = g == ngroups - 1;
         for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++it) {
             const int sl = (int)(it & 1);
+            // the state carried from the earlier groups (their clusters have lower ids), loaded
+            // for the four rows while the tile is scored
+            struct {
+                float G, u1, u2, v;
+                int k1, k2, zv;
+            } cs[4];
+            if (!first)
+#pragma unroll
+                for (int qr = 0; qr < 4; ++qr) {
+                    const int64_t i = min(t * BM + qr * 32 + lane, a.N - 1);
+                    cs[qr].G = a.carry.g[i];
+                    cs[qr].u1 = a.carry.u1[i];
+                    cs[qr].u2 = a.carry.u2[i];
+                    cs[qr].v = a.carry.v[i];
+                    cs[qr].k1 = a.carry.k1[i];
+                    cs[qr].k2 = a.carry.k2[i];
+                    cs[qr].zv = a.carry.zv[i];
+                }
             if (!mbar_wait(&sfull[sl], (uint32_t)((it >> 1) & 1), abort)) { ok = false; break; }
             const float* sb = sbuf + (size_t)sl * a.capc * BM;
+#pragma unroll
             for (int qr = 0; qr < 4; ++qr) {
                 const int r = qr * 32 + lane;
                 const int64_t i = t * BM + r;
@@ -366,66 +390,86 @@ __global__ void __launch_bounds__(NTHREADS, 1) labels_tc_kernel(const __grid_con
                         g2 = fmaxf(g2, o1);
                     }
                 }
-                // the state carried from the earlier groups (their clusters have lower ids)
-                float cg1 = -INFINITY, cg2 = -INFINITY, cv = -INFINITY;
-                int ck1 = 0, cz = 0;
-                if (!first && i < a.N) {
-                    cg1 = a.carry.g1[i];
-                    cg2 = a.carry.g2[i];
-                    cv = a.carry.v[i];
-                    ck1 = a.carry.k1[i];
-                    cz = a.carry.zv[i];
-                }
+                float G = -INFINITY, u1 = -INFINITY, u2 = -INFINITY, v = -INFINITY;
+                int k1 = 0, k2 = 0, zv = 0;
                 if (!first) {
-                    if (cg1 >= g1) {
-                        g2 = fmaxf(g1, cg2);
-                        g1 = cg1;
-                        gk = ck1;
-                    } else {
-                        g2 = fmaxf(g2, cg1);
+                    G = cs[qr].G;
+                    u1 = cs[qr].u1;
+                    u2 = cs[qr].u2;
+                    v = cs[qr].v;
+                    k1 = cs[qr].k1;
+                    k2 = cs[qr].k2;
+                    zv = cs[qr].zv;
+                }
+                G = fmaxf(G, g1);
+                const float lim = G - WINDOW;  // a cluster at or below it cannot win
+                if (!(u1 > lim)) u1 = -INFINITY;
+                if (!(u2 > lim)) u2 = -INFINITY;
+                const bool in = g1 > lim, more = g2 > lim;  // this group's best, and others of it
+                const int held = (u1 > -INFINITY) + (u2 > -INFINITY), tot = held + in + more;
+                bool draw = final ? tot >= 2 || (tot == 1 && v > -INFINITY) : tot > 2;
+                if (!draw && more) {  // not the last group, nothing held: are there just two?
+                    int n = 0;
+                    for (int kk = 0; kk < Kg; ++kk) {
+                        const float sc = sb[(size_t)kk * BM + r];
+                        if (sc > lim) {
+                            ++n;
+                            if (kb + kk != gk) {
+                                u2 = sc;
+                                k2 = kb + kk;
+                            }
+                        }
+                    }
+                    u1 = g1;
+                    k1 = gk;
+                    if (n > 2) {
+                        draw = true;
+                        u1 = u2 = -INFINITY;  // drawn with the group's
                     }
                 }
-                const float lim = g1 - WINDOW;
-                const bool need = !(g2 <= lim);  // another cluster might win: draw
-                float vbest = cv;  // best perturbed score among all clusters drawn so far
-                int zbest = cz;
-                if (need) {
-                    float best = -INFINITY;
-                    int zb = 0;
-                    auto draw = [&](int k, float sc) {
+                if (draw) {
+                    auto one = [&](int k, float sc) {
                         uint32_t w[4];
                         key.block((uint32_t)i, TAG_Z, (uint32_t)(k >> 1), w);
                         const float u = u01_f32((k & 1) ? w[2] : w[0]);
-                        const float v = sc - __logf(-logf(u));
-                        if (v > best || (v == best && k < zb)) {
-                            best = v;
-                            zb = k;
+                        const float x = sc - __logf(-logf(u));
+                        if (x > v || (x == v && k < zv)) {
+                            v = x;
+                            zv = k;
                         }
                     };
-                    for (int kk = 0; kk < Kg; ++kk) {
-                        const float sc = sb[(size_t)kk * BM + r];
-                        if (sc > lim) draw(kb + kk, sc);
+                    if (more) {
+                        for (int kk = 0; kk < Kg; ++kk) {
+                            const float sc = sb[(size_t)kk * BM + r];
+                            if (sc > lim) one(kb + kk, sc);
+                        }
+                    } else if (in) {
+                        one(gk, g1);
                     }
-                    // the carried best cluster: its draw was deferred until a rival appeared
-                    // (drawing it again later gives the same value)
-                    if (!first && cg1 > lim) draw(ck1, cg1);
-                    if (cv > best || (cv == best && cz < zb)) {
-                        best = cv;
-                        zb = cz;
+                    if (u1 > -INFINITY) one(k1, u1);
+                    if (u2 > -INFINITY) one(k2, u2);
+                    u1 = u2 = -INFINITY;
+                } else if (in && !more) {
+                    if (u1 > -INFINITY) {
+                        u2 = g1;
+                        k2 = gk;
+                    } else {
+                        u1 = g1;
+                        k1 = gk;
                     }
-                    vbest = best;
-                    zbest = zb;
                 }
                 if (i < a.N) {
                     if (final) {
-                        a.z[i] = need ? zbest : gk;
+                        a.z[i] = u1 > -INFINITY ? k1 : u2 > -INFINITY ? k2 : zv;
                     } else {
                         // read back by this lane in the next group
-                        a.carry.g1[i] = g1;
-                        a.carry.g2[i] = g2;
-                        a.carry.v[i] = vbest;
-                        a.carry.k1[i] = gk;
-                        a.carry.zv[i] = zbest;
+                        a.carry.g[i] = G;
+                        a.carry.u1[i] = u1;
+                        a.carry.u2[i] = u2;
+                        a.carry.k1[i] = k1;
+                        a.carry.k2[i] = k2;
+                        a.carry.v[i] = v;
+                        a.carry.zv[i] = zv;
                     }
                 }
             }
@@ -597,7 +641,7 @@ cudaError_t launch_labels_tc(dpmm_ctx* c, uint64_t seed) {
     {
         float* f = (float*)c->tc_carry;
         const size_t n = (size_t)c->N;
-        a.carry = tc::Carry{f, f + n, f + 2 * n, (int*)(f + 3 * n), (int*)(f + 4 * n)};
+        a.carry = tc::Carry{f, f + n, f + 2 * n, (int*)(f + 3 * n), (int*)(f + 4 * n), f + 5 * n, (int*)(f + 6 * n)};
     }
     a.Kmax = c->K_max;
     a.dK = c->dK;
@@ -633,6 +677,6 @@ namespace dpmm {
 // (0 when one group holds every cluster up to K_max)
 size_t tc_carry_bytes(const dpmm_ctx* c) {
     if (c->kind != DPMM_PRIOR_NIW || c->prec != DPMM_PREC_TF32 || !tc_supported(c)) return 0;
-    return tc_cfg(c).gmax > 1 ? (size_t)c->N * 20 : 0;
+    return tc_cfg(c).gmax > 1 ? (size_t)c->N * 28 : 0;
 }
 }  // namespace dpmm
