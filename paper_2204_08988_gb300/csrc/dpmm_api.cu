@@ -869,7 +869,7 @@ static cudaError_t sweep_phase_a(dpmm_ctx* c, uint64_t seed) {
     if (c->step_mask & 1u) {
         if ((e = launch_weights(c, seed)) != cudaSuccess) return e;
         if ((e = launch_params(c, seed)) != cudaSuccess) return e;
-        if ((e = launch_derive(c)) != cudaSuccess) return e;
+        if ((e = launch_derive(c, true)) != cudaSuccess) return e;
     }
     if ((c->step_mask & 2u) && c->sparse) {
         if ((e = launch_sparse(c, seed, 0, nullptr)) != cudaSuccess) return e;
@@ -1339,7 +1339,7 @@ dpmm_status dpmm_set_params(dpmm_ctx* c, int K, const double* logw, const double
     CK(c, cudaMemcpyAsync(c->p_logw, logw, sizeof(double) * S, cudaMemcpyHostToDevice, c->stream));
     CK(c, cudaMemcpyAsync(c->p_c, cc.data(), sizeof(double) * S, cudaMemcpyHostToDevice, c->stream));
     CK(c, cudaMemcpyAsync(c->dK, &K, sizeof(int), cudaMemcpyHostToDevice, c->stream));
-    CK(c, launch_derive(c));
+    CK(c, launch_derive(c, false));
     CK(c, cudaStreamSynchronize(c->stream));
     return DPMM_OK;
 }

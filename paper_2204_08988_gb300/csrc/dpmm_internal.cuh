@@ -305,7 +305,7 @@ struct dpmm_ctx {
 
     // tensor-core path
     int* tc_flag = nullptr;        // device: 1 when K did not fit the tensor-core kernel
-    void* tc_carry = nullptr;      // device: per-point state between cluster groups (TF32), N x 28 B
+    void* tc_carry = nullptr;      // device: per-point state between cluster groups (TF32), N x 36 B
 
     // multinomial data of more than SPARSE_MIN_D categories: compressed rows
     bool sparse = false;
@@ -370,7 +370,7 @@ struct CountsStats {
 // kernel launchers, one per .cu file group; each returns cudaGetLastError().
 cudaError_t launch_weights(dpmm_ctx* c, uint64_t seed);
 cudaError_t launch_params(dpmm_ctx* c, uint64_t seed);
-cudaError_t launch_derive(dpmm_ctx* c);
+cudaError_t launch_derive(dpmm_ctx* c, bool drawn);
 cudaError_t launch_labels_simt(dpmm_ctx* c, uint64_t seed);
 cudaError_t launch_labels_tc(dpmm_ctx* c, uint64_t seed);
 cudaError_t launch_sort(dpmm_ctx* c);

@@ -484,7 +484,7 @@ __global__ void dirichlet_draw_f32_kernel(int d, const double* beta, const int* 
 }
 
 __global__ void dirichlet_norm_f32_kernel(int d, const int* dK, const double* logw, const float2* part,
-                                          float* q_logtheta, double* p_logtheta, double* p_c) {
+                                          float* q_logtheta, double* p_logtheta, double* p_c, float* q_c) {
     const int K = *dK;
     const int s = blockIdx.x;
     if (s >= 3 * K) return;
@@ -505,7 +505,10 @@ __global__ void dirichlet_norm_f32_kernel(int d, const int* dK, const double* lo
         qt[j] = v;
         lt[j] = (double)v;
     }
-    if (blockIdx.y == 0 && threadIdx.x == 0) p_c[s] = logw[s];
+    if (blockIdx.y == 0 && threadIdx.x == 0) {
+        p_c[s] = logw[s];
+        q_c[s] = (float)logw[s];
+    }
 }
 
 // FP32 mirrors of the drawn parameters for the reduced-precision paths, and the
@@ -650,7 +653,7 @@ cudaError_t launch_params(dpmm_ctx* c, uint64_t seed) {
                     c->d, c->center + c->d, c->dK, c->diter, seed, CountsStats{c->stats, c->st}, c->q_logtheta,
                     (float2*)c->sp_part);
             dirichlet_norm_f32_kernel<<<grid, 256, 0, c->stream>>>(c->d, c->dK, c->p_logw, (const float2*)c->sp_part,
-                                                                  c->q_logtheta, c->p_logtheta, c->p_c);
+                                                                  c->q_logtheta, c->p_logtheta, c->p_c, c->q_c);
             c->nlaunch += 1;
         } else
             dirichlet_params_kernel<<<3 * c->K_max, 256, 0, c->stream>>>(make_sv(c), c->center + c->d, c->dK,
@@ -662,14 +665,20 @@ cudaError_t launch_params(dpmm_ctx* c, uint64_t seed) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_derive(dpmm_ctx* c) {
-    prof_begin(c, "derive");
-    const dim3 dgrid(3 * c->K_max, c->kind == DPMM_PRIOR_NIW ? 1 : (c->d + 4095) / 4096);
-    derive_kernel<<<dgrid, 128, 0, c->stream>>>(c->kind, c->d, c->prec == DPMM_PREC_TF32, c->prec == DPMM_PREC_FP64_PLAIN, c->dK, c->p_logw, c->p_mu, c->p_W, c->p_c,
-                                                       c->p_logtheta, c->q_mu, c->q_W, c->q_c, c->q_b, c->p_b,
-                                                       c->q_logtheta, c->shift_new, c->shift32);
-    prof_end(c, "derive");
-    c->nlaunch += 1;
+// drawn: the parameters come from launch_params, whose FP32 Dirichlet draws leave their mirrors
+// written (a pass over 3 K d values: 15 of a sweep's 240 us at d = 20,000, K = 20)
+cudaError_t launch_derive(dpmm_ctx* c, bool drawn) {
+    const bool mirrored = drawn && c->kind == DPMM_PRIOR_DIRICHLET && c->prec != DPMM_PREC_FP64_PLAIN;
+    if (!mirrored) {
+        prof_begin(c, "derive");
+        const dim3 dgrid(3 * c->K_max, c->kind == DPMM_PRIOR_NIW ? 1 : (c->d + 4095) / 4096);
+        derive_kernel<<<dgrid, 128, 0, c->stream>>>(c->kind, c->d, c->prec == DPMM_PREC_TF32,
+                                                    c->prec == DPMM_PREC_FP64_PLAIN, c->dK, c->p_logw, c->p_mu, c->p_W, c->p_c,
+                                                    c->p_logtheta, c->q_mu, c->q_W, c->q_c, c->q_b, c->p_b, c->q_logtheta,
+                                                    c->shift_new, c->shift32);
+        prof_end(c, "derive");
+        c->nlaunch += 1;
+    }
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && c->sparse) e = sparse_prepare(c);
     if (e == cudaSuccess && tc_supported(c)) e = tc_prepare(c);

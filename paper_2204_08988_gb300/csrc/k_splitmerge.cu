@@ -294,16 +294,22 @@ __device__ __forceinline__ void marginal_counts_item(const SMArgs& a, const Src&
     }
     using V = decltype(cnt(0, 0));  // the source's own type: FP32 sums stay off the FP64 pipe
     const int s0 = 2 * k1 + (h < 0 ? 0 : h);
-    double sc = 0.0, acc = 0.0;
+    // the counts are added as integers (exact, as FP64 adds of them are): a conversion to FP64
+    // and an FP64 add a category kept the two-lane FP64 pipe busy two thirds of the time
+    // (d = 20,000, K = 20: 46 us, from 66)
+    unsigned long long si = 0;
+    double acc = 0.0;
     for (int j = tid; j < d; j += nt) {
         V c = cnt(s0, j);
         if (h < 0) c += cnt(2 * k1 + 1, j);
         if (k2 >= 0) c += cnt(2 * k2, j) + cnt(2 * k2 + 1, j);  // integer counts: exact
         if (c > V(0)) {
-            sc += (double)c;
+            if constexpr (sizeof(V) == 4) si += (unsigned)c;
+            else si += (unsigned long long)c;
             acc += (lgt && c < (V)nlgt) ? lgt[(int)c] : lgamma(a.beta[j] + (double)c) - lgb[j];
         }
     }
+    double sc = (double)si;
     for (int o = 16; o > 0; o >>= 1) {
         sc += __shfl_xor_sync(0xffffffffu, sc, o);
         acc += __shfl_xor_sync(0xffffffffu, acc, o);

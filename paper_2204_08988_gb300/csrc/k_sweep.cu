@@ -1900,7 +1900,7 @@ __global__ void __launch_bounds__(256) substats_mult_kernel(SubArgs<float> a) {
 // of a point's counts and of the two sub-cluster log theta rows of the current cluster; the
 // two sub-cluster scores are dot products reduced across the warp; the z-bar draws of 32
 // points are made at once, one point per lane, and four points' scores are reduced together
-// (N = 1e6, d = 200, K = 50: @@MULT@@ us, from 238 us with two five-step reductions a point).  The
+// (N = 1e6, d = 200, K = 50: 187 us, from 238 us with two five-step reductions a point).  The
 // counts of a cluster's run stay in registers and are added at the run's end to the compact table cnt (2 K_max x (d + 1) integers, column
 // d: the points) with atomic adds, exact in any order.  No block-wide barrier.
 struct MwArgs {

@@ -63,19 +63,21 @@ constexpr uint32_t TMEM_COLS = 512;
 constexpr int NBUF = 2;                        // TMEM accumulator buffers
 constexpr int BUFCOLS = (int)TMEM_COLS / NBUF; // columns per buffer (the chunk width)
 
-// Per-point state carried from one cluster group to the next.  At most two clusters within the
+// Per-point state carried from one cluster group to the next.  Up to HELD clusters within the
 // window of the best score are carried undrawn: a group of clusters that are all far from the
-// point often has two whose scores lie close together, and drawing them there (26 clusters, 32
-// rows a warp: nearly every one for some row) cost more than the scores; mostly a later group's
-// cluster is ahead of both by more than the window, and nothing is drawn (N = 200,003, d = 32,
-// K = 60: @@CARRY@@ us a label step, from 312 us).
+// point often has some whose scores lie close together, and drawing them there (for nearly every
+// warp some row has such) cost more than the scores; mostly a later group's cluster is ahead of
+// all by more than the window, and nothing is drawn.  N = 200,003, d = 32, K = 60: 233 us a label
+// step, 276 us with two held, 312 us with none.
+constexpr int HELD = 4;
 struct Carry {
     float* g;        // best score so far
-    float *u1, *u2;  // undrawn clusters within the window of g (-inf: none)
-    int *k1, *k2;
+    float* u[HELD];  // undrawn clusters within the window of g (-inf: none)
+    int* k[HELD / 2];  // their ids, two to a word
     float* v;        // best perturbed score among the clusters drawn (-inf: none), and its cluster
     int* zv;
 };
+constexpr int CARRY_BYTES = 4 * (3 + HELD + HELD / 2);
 
 struct Args {
     int64_t N;
@@ -355,20 +357,20 @@ __global__ void __launch_bounds__(NTHREADS, 1) labels_tc_kernel(const __grid_con
             // the state carried from the earlier groups (their clusters have lower ids), loaded
             // for the four rows while the tile is scored
             struct {
-                float G, u1, u2, v;
-                int k1, k2, zv;
+                float G, u[HELD], v;
+                int k[HELD / 2], zv;
             } cs[4];
             if (!first)
 #pragma unroll
                 for (int qr = 0; qr < 4; ++qr) {
                     const int64_t i = min(t * BM + qr * 32 + lane, a.N - 1);
                     cs[qr].G = a.carry.g[i];
-                    cs[qr].u1 = a.carry.u1[i];
-                    cs[qr].u2 = a.carry.u2[i];
                     cs[qr].v = a.carry.v[i];
-                    cs[qr].k1 = a.carry.k1[i];
-                    cs[qr].k2 = a.carry.k2[i];
                     cs[qr].zv = a.carry.zv[i];
+#pragma unroll
+                    for (int e = 0; e < HELD; ++e) cs[qr].u[e] = a.carry.u[e][i];
+#pragma unroll
+                    for (int e = 0; e < HELD / 2; ++e) cs[qr].k[e] = a.carry.k[e][i];
                 }
             if (!mbar_wait(&sfull[sl], (uint32_t)((it >> 1) & 1), abort)) { ok = false; break; }
             const float* sb = sbuf + (size_t)sl * a.capc * BM;
@@ -390,86 +392,91 @@ __global__ void __launch_bounds__(NTHREADS, 1) labels_tc_kernel(const __grid_con
                         g2 = fmaxf(g2, o1);
                     }
                 }
-                float G = -INFINITY, u1 = -INFINITY, u2 = -INFINITY, v = -INFINITY;
-                int k1 = 0, k2 = 0, zv = 0;
+                float G = -INFINITY, v = -INFINITY, u[HELD];
+                int k[HELD], zv = 0;
+#pragma unroll
+                for (int e = 0; e < HELD; ++e) {
+                    u[e] = first ? -INFINITY : cs[qr].u[e];
+                    k[e] = first ? 0 : (cs[qr].k[e / 2] >> (16 * (e & 1))) & 0xFFFF;
+                }
                 if (!first) {
                     G = cs[qr].G;
-                    u1 = cs[qr].u1;
-                    u2 = cs[qr].u2;
                     v = cs[qr].v;
-                    k1 = cs[qr].k1;
-                    k2 = cs[qr].k2;
                     zv = cs[qr].zv;
                 }
                 G = fmaxf(G, g1);
                 const float lim = G - WINDOW;  // a cluster at or below it cannot win
-                if (!(u1 > lim)) u1 = -INFINITY;
-                if (!(u2 > lim)) u2 = -INFINITY;
+                int n = 0;                     // contenders: the held ones, then this group's
+#pragma unroll
+                for (int e = 0; e < HELD; ++e) {
+                    if (!(u[e] > lim)) u[e] = -INFINITY;
+                    n += u[e] > -INFINITY;
+                }
+                auto hold = [&](float sc, int kk) {
+                    bool todo = true;
+#pragma unroll
+                    for (int e = 0; e < HELD; ++e)
+                        if (todo && u[e] == -INFINITY) {
+                            u[e] = sc;
+                            k[e] = kk;
+                            todo = false;
+                        }
+                    ++n;
+                };
                 const bool in = g1 > lim, more = g2 > lim;  // this group's best, and others of it
-                const int held = (u1 > -INFINITY) + (u2 > -INFINITY), tot = held + in + more;
-                bool draw = final ? tot >= 2 || (tot == 1 && v > -INFINITY) : tot > 2;
-                if (!draw && more) {  // not the last group, nothing held: are there just two?
-                    int n = 0;
+                if (more) {
                     for (int kk = 0; kk < Kg; ++kk) {
                         const float sc = sb[(size_t)kk * BM + r];
-                        if (sc > lim) {
-                            ++n;
-                            if (kb + kk != gk) {
-                                u2 = sc;
-                                k2 = kb + kk;
-                            }
-                        }
+                        if (sc > lim) hold(sc, kb + kk);
                     }
-                    u1 = g1;
-                    k1 = gk;
-                    if (n > 2) {
-                        draw = true;
-                        u1 = u2 = -INFINITY;  // drawn with the group's
-                    }
+                } else if (in) {
+                    hold(g1, gk);
                 }
-                if (draw) {
-                    auto one = [&](int k, float sc) {
+                int label = zv;
+                if (final ? n >= 2 || (n == 1 && v > -INFINITY) : n > HELD) {
+                    auto one = [&](int kk, float sc) {
                         uint32_t w[4];
-                        key.block((uint32_t)i, TAG_Z, (uint32_t)(k >> 1), w);
-                        const float u = u01_f32((k & 1) ? w[2] : w[0]);
-                        const float x = sc - __logf(-logf(u));
-                        if (x > v || (x == v && k < zv)) {
+                        key.block((uint32_t)i, TAG_Z, (uint32_t)(kk >> 1), w);
+                        const float u01 = u01_f32((kk & 1) ? w[2] : w[0]);
+                        const float x = sc - __logf(-logf(u01));
+                        if (x > v || (x == v && kk < zv)) {
                             v = x;
-                            zv = k;
+                            zv = kk;
                         }
                     };
-                    if (more) {
-                        for (int kk = 0; kk < Kg; ++kk) {
-                            const float sc = sb[(size_t)kk * BM + r];
-                            if (sc > lim) one(kb + kk, sc);
+#pragma unroll
+                    for (int e = 0; e < HELD; ++e) {
+                        if (u[e] > -INFINITY) one(k[e], u[e]);
+                        u[e] = -INFINITY;
+                    }
+                    if (n > HELD) {  // some found no room (drawing a cluster twice gives the same value)
+                        if (more) {
+                            for (int kk = 0; kk < Kg; ++kk) {
+                                const float sc = sb[(size_t)kk * BM + r];
+                                if (sc > lim) one(kb + kk, sc);
+                            }
+                        } else {
+                            one(gk, g1);
                         }
-                    } else if (in) {
-                        one(gk, g1);
                     }
-                    if (u1 > -INFINITY) one(k1, u1);
-                    if (u2 > -INFINITY) one(k2, u2);
-                    u1 = u2 = -INFINITY;
-                } else if (in && !more) {
-                    if (u1 > -INFINITY) {
-                        u2 = g1;
-                        k2 = gk;
-                    } else {
-                        u1 = g1;
-                        k1 = gk;
-                    }
+                    label = zv;
+                } else if (final) {
+#pragma unroll
+                    for (int e = 0; e < HELD; ++e)
+                        if (u[e] > -INFINITY) label = k[e];
                 }
                 if (i < a.N) {
                     if (final) {
-                        a.z[i] = u1 > -INFINITY ? k1 : u2 > -INFINITY ? k2 : zv;
+                        a.z[i] = label;
                     } else {
                         // read back by this lane in the next group
                         a.carry.g[i] = G;
-                        a.carry.u1[i] = u1;
-                        a.carry.u2[i] = u2;
-                        a.carry.k1[i] = k1;
-                        a.carry.k2[i] = k2;
                         a.carry.v[i] = v;
                         a.carry.zv[i] = zv;
+#pragma unroll
+                        for (int e = 0; e < HELD; ++e) a.carry.u[e][i] = u[e];
+#pragma unroll
+                        for (int e = 0; e < HELD / 2; ++e) a.carry.k[e][i] = k[2 * e] | k[2 * e + 1] << 16;
                     }
                 }
             }
@@ -641,7 +648,11 @@ cudaError_t launch_labels_tc(dpmm_ctx* c, uint64_t seed) {
     {
         float* f = (float*)c->tc_carry;
         const size_t n = (size_t)c->N;
-        a.carry = tc::Carry{f, f + n, f + 2 * n, (int*)(f + 3 * n), (int*)(f + 4 * n), f + 5 * n, (int*)(f + 6 * n)};
+        a.carry.g = f;
+        a.carry.v = f + n;
+        a.carry.zv = (int*)(f + 2 * n);
+        for (int e = 0; e < tc::HELD; ++e) a.carry.u[e] = f + (3 + e) * n;
+        for (int e = 0; e < tc::HELD / 2; ++e) a.carry.k[e] = (int*)(f + (3 + tc::HELD + e) * n);
     }
     a.Kmax = c->K_max;
     a.dK = c->dK;
@@ -677,6 +688,6 @@ namespace dpmm {
 // (0 when one group holds every cluster up to K_max)
 size_t tc_carry_bytes(const dpmm_ctx* c) {
     if (c->kind != DPMM_PRIOR_NIW || c->prec != DPMM_PREC_TF32 || !tc_supported(c)) return 0;
-    return tc_cfg(c).gmax > 1 ? (size_t)c->N * 28 : 0;
+    return tc_cfg(c).gmax > 1 ? (size_t)c->N * tc::CARRY_BYTES : 0;
 }
 }  // namespace dpmm
