@@ -630,7 +630,7 @@ dpmm_status dpmm_set_data(dpmm_ctx* c, const void* X, int64_t N, dpmm_dtype dt, 
     A(&c->zbar, N);
     A(&c->idx, sizeof(int) * N);
     A(&c->hist, sizeof(int) * (size_t)c->K_max * c->T_tiles);
-    if (const size_t cb = tc_carry_bytes(c)) A(&c->tc_carry, cb);
+    ok = ok && tc_carry_alloc(c) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();  // the failed allocation's error is not left for a later call to report
         free_data(c);

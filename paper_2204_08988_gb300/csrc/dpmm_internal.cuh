@@ -305,7 +305,8 @@ struct dpmm_ctx {
 
     // tensor-core path
     int* tc_flag = nullptr;        // device: 1 when K did not fit the tensor-core kernel
-    void* tc_carry = nullptr;      // device: per-point state between cluster groups (TF32), N x 36 B
+    void* tc_carry = nullptr;      // device: per-point state between cluster groups (TF32), N x 36 or 20 B
+    int tc_held = 0;               // undrawn clusters that it holds per point
 
     // multinomial data of more than SPARSE_MIN_D categories: compressed rows
     bool sparse = false;
@@ -382,7 +383,13 @@ cudaError_t launch_splitmerge(dpmm_ctx* c, uint64_t seed, int labels_ran, int sm
 cudaError_t launch_relabel(dpmm_ctx* c, uint64_t seed);
 cudaError_t launch_advance(dpmm_ctx* c);
 bool tc_supported(const dpmm_ctx* c);
-size_t tc_carry_bytes(const dpmm_ctx* c);
+cudaError_t tc_carry_alloc(dpmm_ctx* c);
+// whether the device has room for an optional buffer, for what is known to be allocated after it
+// and for 1 GiB besides (graphs, factor images, the caller's own tensors)
+inline bool roomy(size_t bytes, size_t later) {
+    size_t free = 0, total = 0;
+    return cudaMemGetInfo(&free, &total) == cudaSuccess && free >= bytes + later + ((size_t)1 << 30);
+}
 cudaError_t tc_prepare(dpmm_ctx* c);
 bool substats_tc_supported(const dpmm_ctx* c);
 cudaError_t substats_tc_prepare(dpmm_ctx* c);

@@ -77,7 +77,8 @@ struct Carry {
     float* v;        // best perturbed score among the clusters drawn (-inf: none), and its cluster
     int* zv;
 };
-constexpr int CARRY_BYTES = 4 * (3 + HELD + HELD / 2);
+// On a nearly full device one is held (20 bytes a point, not 36).
+constexpr int carry_bytes(int held) { return 4 * (3 + held + (held + 1) / 2); }
 
 struct Args {
     int64_t N;
@@ -86,6 +87,7 @@ struct Args {
     int cap_rows;     // factor rows that fit in shared memory
     int capc;         // clusters per group (cap_rows / dn)
     int gmax;         // most cluster groups (more clusters: the CUDA-core kernel)
+    int held;         // undrawn clusters carried over the groups: HELD or 1
     int img_rows;     // rows of the factor image in global memory (all K_max clusters)
     Carry carry;
     int Kmax;
@@ -368,9 +370,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) labels_tc_kernel(const __grid_con
                     cs[qr].v = a.carry.v[i];
                     cs[qr].zv = a.carry.zv[i];
 #pragma unroll
-                    for (int e = 0; e < HELD; ++e) cs[qr].u[e] = a.carry.u[e][i];
+                    for (int e = 0; e < HELD; ++e) cs[qr].u[e] = e < a.held ? a.carry.u[e][i] : -INFINITY;
 #pragma unroll
-                    for (int e = 0; e < HELD / 2; ++e) cs[qr].k[e] = a.carry.k[e][i];
+                    for (int e = 0; e < HELD / 2; ++e) cs[qr].k[e] = 2 * e < a.held ? a.carry.k[e][i] : 0;
                 }
             if (!mbar_wait(&sfull[sl], (uint32_t)((it >> 1) & 1), abort)) { ok = false; break; }
             const float* sb = sbuf + (size_t)sl * a.capc * BM;
@@ -416,7 +418,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) labels_tc_kernel(const __grid_con
                     bool todo = true;
 #pragma unroll
                     for (int e = 0; e < HELD; ++e)
-                        if (todo && u[e] == -INFINITY) {
+                        if (todo && e < a.held && u[e] == -INFINITY) {
                             u[e] = sc;
                             k[e] = kk;
                             todo = false;
@@ -433,7 +435,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) labels_tc_kernel(const __grid_con
                     hold(g1, gk);
                 }
                 int label = zv;
-                if (final ? n >= 2 || (n == 1 && v > -INFINITY) : n > HELD) {
+                if (final ? n >= 2 || (n == 1 && v > -INFINITY) : n > a.held) {
                     auto one = [&](int kk, float sc) {
                         uint32_t w[4];
                         key.block((uint32_t)i, TAG_Z, (uint32_t)(kk >> 1), w);
@@ -449,7 +451,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) labels_tc_kernel(const __grid_con
                         if (u[e] > -INFINITY) one(k[e], u[e]);
                         u[e] = -INFINITY;
                     }
-                    if (n > HELD) {  // some found no room (drawing a cluster twice gives the same value)
+                    if (n > a.held) {  // some found no room (drawing a cluster twice gives the same value)
                         if (more) {
                             for (int kk = 0; kk < Kg; ++kk) {
                                 const float sc = sb[(size_t)kk * BM + r];
@@ -474,9 +476,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) labels_tc_kernel(const __grid_con
                         a.carry.v[i] = v;
                         a.carry.zv[i] = zv;
 #pragma unroll
-                        for (int e = 0; e < HELD; ++e) a.carry.u[e][i] = u[e];
+                        for (int e = 0; e < HELD; ++e)
+                            if (e < a.held) a.carry.u[e][i] = u[e];
 #pragma unroll
-                        for (int e = 0; e < HELD / 2; ++e) a.carry.k[e][i] = k[2 * e] | k[2 * e + 1] << 16;
+                        for (int e = 0; e < HELD / 2; ++e)
+                            if (2 * e < a.held) a.carry.k[e][i] = k[2 * e] | k[2 * e + 1] << 16;
                     }
                 }
             }
@@ -651,8 +655,10 @@ cudaError_t launch_labels_tc(dpmm_ctx* c, uint64_t seed) {
         a.carry.g = f;
         a.carry.v = f + n;
         a.carry.zv = (int*)(f + 2 * n);
-        for (int e = 0; e < tc::HELD; ++e) a.carry.u[e] = f + (3 + e) * n;
-        for (int e = 0; e < tc::HELD / 2; ++e) a.carry.k[e] = (int*)(f + (3 + tc::HELD + e) * n);
+        a.held = c->tc_held;
+        for (int e = 0; e < tc::HELD; ++e) a.carry.u[e] = e < a.held ? f + (3 + e) * n : nullptr;
+        for (int e = 0; e < tc::HELD / 2; ++e)
+            a.carry.k[e] = 2 * e < a.held ? (int*)(f + (3 + a.held + e) * n) : nullptr;
     }
     a.Kmax = c->K_max;
     a.dK = c->dK;
@@ -684,10 +690,14 @@ cudaError_t launch_labels_tc(dpmm_ctx* c, uint64_t seed) {
 }  // namespace dpmm
 
 namespace dpmm {
-// bytes of the per-point state carried between cluster groups of the TF32 label step
-// (0 when one group holds every cluster up to K_max)
-size_t tc_carry_bytes(const dpmm_ctx* c) {
-    if (c->kind != DPMM_PRIOR_NIW || c->prec != DPMM_PREC_TF32 || !tc_supported(c)) return 0;
-    return tc_cfg(c).gmax > 1 ? (size_t)c->N * tc::CARRY_BYTES : 0;
+// the per-point state carried between cluster groups of the TF32 label step (none where one
+// group holds every cluster up to K_max)
+cudaError_t tc_carry_alloc(dpmm_ctx* c) {
+    if (c->kind != DPMM_PRIOR_NIW || c->prec != DPMM_PREC_TF32 || !tc_supported(c) || tc_cfg(c).gmax <= 1) return cudaSuccess;
+    const size_t full = (size_t)c->N * tc::carry_bytes(tc::HELD);
+    c->tc_held = roomy(full, (size_t)c->N * c->d * 8) ? tc::HELD : 1;  // a copy of the input (FP64 at most) follows
+    cudaError_t e = cudaMalloc(&c->tc_carry, (size_t)c->N * tc::carry_bytes(c->tc_held));
+    if (e != cudaSuccess) c->tc_carry = nullptr;
+    return e;
 }
 }  // namespace dpmm

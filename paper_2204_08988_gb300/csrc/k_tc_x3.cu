@@ -740,6 +740,26 @@ static bool x3_screened(const dpmm_ctx* c) {
 }
 static int x3_cap(const dpmm_ctx* c) { return (int)(c->N / 8); }  // points that the gathered tiles hold
 
+// The screening's buffers (44 to 76 bytes a point).  On a nearly full device they are left out, and
+// every point gets the three products: data that fit without them stay accepted.
+static bool x3_screen_alloc(dpmm_ctx* c) {
+    if (!x3_screened(c)) return false;
+    if (c->x3_cimg) return true;
+    const int64_t ct = (x3_cap(c) + 127) / 128 + x3::MT;
+    const size_t cbytes = (size_t)ct * x3_geo(c, nullptr).xtile;
+    if (!roomy((sizeof(float2) + sizeof(int)) * c->N + cbytes, 0)) return false;
+    cudaError_t e = cudaMalloc(&c->x3_xn, sizeof(float2) * c->N);
+    if (e == cudaSuccess) e = cudaMalloc(&c->x3_list, sizeof(int) * c->N);
+    if (e == cudaSuccess && !c->x3_words) e = cudaMalloc(&c->x3_words, 4 * sizeof(int) + sizeof(float4) * c->K_max);
+    if (e == cudaSuccess) e = cudaMalloc(&c->x3_cimg, cbytes);
+    if (e == cudaSuccess) return true;
+    cudaGetLastError();
+    cudaFree(c->x3_xn);
+    cudaFree(c->x3_list);
+    c->x3_xn = c->x3_list = c->x3_cimg = nullptr;
+    return false;
+}
+
 // after the data are stored (centred FP32): allocate the point and factor images and
 // split the points into their BF16 parts
 cudaError_t x3_prepare_data(dpmm_ctx* c) {
@@ -757,16 +777,8 @@ cudaError_t x3_prepare_data(dpmm_ctx* c) {
         e = cudaMemsetAsync(c->x3_fimg, 0, (size_t)c->K_max * g.cbytes, c->stream);
         if (e != cudaSuccess) return e;
     }
-    if (x3_screened(c)) {
-        const int64_t ct = (x3_cap(c) + 127) / 128 + x3::MT;
-        cudaError_t e = cudaSuccess;
-        if (!c->x3_xn) {
-            e = cudaMalloc(&c->x3_xn, sizeof(float2) * c->N);
-            if (e == cudaSuccess) e = cudaMalloc(&c->x3_list, sizeof(int) * c->N);
-            if (e == cudaSuccess) e = cudaMalloc(&c->x3_cimg, (size_t)ct * g.xtile);
-        }
-        if (e == cudaSuccess && !c->x3_words) e = cudaMalloc(&c->x3_words, 4 * sizeof(int) + sizeof(float4) * c->K_max);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->x3_words, 0, 4 * sizeof(int) + sizeof(float4) * c->K_max, c->stream);
+    if (x3_screen_alloc(c)) {
+        cudaError_t e = cudaMemsetAsync(c->x3_words, 0, 4 * sizeof(int) + sizeof(float4) * c->K_max, c->stream);
         if (e != cudaSuccess) return e;
         x3::x3_norm_kernel<<<8 * c->num_sms, 256, 0, c->stream>>>((const float*)c->X, c->N, c->d, c->xs, (float2*)c->x3_xn);
     }
@@ -775,7 +787,7 @@ cudaError_t x3_prepare_data(dpmm_ctx* c) {
     return cudaGetLastError();
 }
 
-static float4* x3_kn(const dpmm_ctx* c) { return c->x3_words && x3_screened(c) ? (float4*)((int*)c->x3_words + 4) : nullptr; }
+static float4* x3_kn(const dpmm_ctx* c) { return c->x3_cimg ? (float4*)((int*)c->x3_words + 4) : nullptr; }
 
 // per sweep, after the parameters are drawn: the factor image
 cudaError_t x3_prepare(dpmm_ctx* c) {
@@ -814,7 +826,7 @@ cudaError_t launch_labels_x3(dpmm_ctx* c, uint64_t seed) {
     const int64_t npass = x3_ntile_pad(c) / x3::MT;
     const int grid = (int)std::min<int64_t>(c->num_sms, npass);
     prof_begin(c, "labels_x3");
-    if (!a.scores && c->x3_words && x3_screened(c)) {
+    if (!a.scores && c->x3_cimg) {
         int* words = (int*)c->x3_words;
         x3::ScreenArgs b;
         b.N = c->N;
