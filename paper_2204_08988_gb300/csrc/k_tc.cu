@@ -394,6 +394,27 @@ __global__ void __launch_bounds__(NTHREADS, 1) labels_tc_kernel(const __grid_con
                         g2 = fmaxf(g2, o1);
                     }
                 }
+                if (first && final) {  // one group: nothing is carried
+                    const float lim = g1 - WINDOW;
+                    int label = gk;
+                    if (!(g2 <= lim)) {  // another cluster might win
+                        float v = -INFINITY;
+                        label = 0;
+                        for (int kk = 0; kk < Kg; ++kk) {
+                            const float sc = sb[(size_t)kk * BM + r];
+                            if (!(sc > lim)) continue;
+                            uint32_t w[4];
+                            key.block((uint32_t)i, TAG_Z, (uint32_t)(kk >> 1), w);
+                            const float x = sc - __logf(-logf(u01_f32((kk & 1) ? w[2] : w[0])));
+                            if (x > v || (x == v && kk < label)) {
+                                v = x;
+                                label = kk;
+                            }
+                        }
+                    }
+                    if (i < a.N) a.z[i] = label;
+                    continue;
+                }
                 float G = -INFINITY, v = -INFINITY, u[HELD];
                 int k[HELD], zv = 0;
 #pragma unroll
@@ -655,7 +676,7 @@ cudaError_t launch_labels_tc(dpmm_ctx* c, uint64_t seed) {
         a.carry.g = f;
         a.carry.v = f + n;
         a.carry.zv = (int*)(f + 2 * n);
-        a.held = c->tc_held;
+        a.held = std::max(1, c->tc_held);
         for (int e = 0; e < tc::HELD; ++e) a.carry.u[e] = e < a.held ? f + (3 + e) * n : nullptr;
         for (int e = 0; e < tc::HELD / 2; ++e)
             a.carry.k[e] = 2 * e < a.held ? (int*)(f + (3 + a.held + e) * n) : nullptr;
