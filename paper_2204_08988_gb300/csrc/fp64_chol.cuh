@@ -1,8 +1,8 @@
 // fp64_chol.cuh -- FP64 building blocks of the parameter and split/merge steps: staging a
 // (sub-)cluster's statistics block in shared memory and a right-looking Cholesky (LDL)
 // factorisation written for GB300's FP64 pipe (about two operations per clock per SM,
-// 64-cycle dependent latency): the only serial work per pivot is one reciprocal square
-// root, and the block meets its barriers once per panel of four pivots.
+// 64-cycle dependent latency): the only serial work per pivot is one reciprocal, and the
+// block meets one barrier per panel of four pivots.
 #pragma once
 #include "dpmm_internal.cuh"
 
@@ -40,83 +40,151 @@ __device__ inline void tri_index(int e, int& i0, int& l0) {
 __device__ inline float rsqrt_t(float x) { return rsqrtf(x); }
 __device__ inline double rsqrt_t(double x) { return rsqrt(x); }
 
+// 1 / v of a positive v in [2^-1000, 2^1000): the FP32 reciprocal of the mantissa, refined by one
+// third-order (Householder) step r (1 + e + e^2), e = 1 - v r, so that three dependent FP64
+// operations remain (a dependent one takes 64 cycles).  The division is kept out of line: beside
+// this, inlined, it was executed for every pivot and its result dropped.
+__device__ inline bool recip_range(double v) {  // false for NaN and what is not positive too
+    return (unsigned)(__double2hiint(v) - (23 << 20)) < (unsigned)(2000 << 20);
+}
+__device__ inline double recip_fast(double v) {
+    const int hi = __double2hiint(v), lo = __double2loint(v);
+    const int e = (hi >> 20) - 1023;
+    const float m = __int_as_float(0x3f800000 | (hi & 0xfffff) << 3 | (int)((unsigned)lo >> 29));
+    const int rb = __float_as_int(__fdividef(1.f, m));  // in [1/2, 1]
+    const double r = __hiloint2double((rb >> 3) + ((1023 - 127 - e) << 20), rb << 29);
+    const double err = fma(-v, r, 1.0);
+    return fma(r, fma(err, err, err), r);
+}
+static __device__ __noinline__ double recip_any(double v) { return 1.0 / v; }
+
 // In-place factorisation of the symmetric matrix whose lower triangle is in A (d x d,
 // row-major with row stride ld, shared memory; an odd ld keeps the column reads free of
 // bank conflicts), in working type T.  Pivot j is v_j = the (j, j) entry of the Schur
 // complement; the update is A_il -= (A_ij / v_j) A_lj for j < l <= i, so column j keeps its
-// unscaled values.  On return piv[j] = v_j and rs[j] = 1 / sqrt(v_j): Psi = U U^T with
-// U_jj = sqrt(v_j), U_ij = A_ij rs[j] (i > j), and log|Psi| = sum_j log v_j.
+// unscaled values.  On return piv[j] = v_j: Psi = U U^T with U_jj = sqrt(v_j),
+// U_ij = A_ij / sqrt(v_j) (i > j), and log|Psi| = sum_j log v_j.
 //
-// Blocked by panels of four pivots, so that the block meets two barriers per panel
-// instead of two per pivot: warp 0 forms a panel's pivots, its scaled columns
-// cols[q][i] = A_i,j0+q / v_j0+q and the updates inside the panel's columns; then every
-// thread applies the panel's four rank-one updates to the rest of the lower triangle, in
-// pivot order.  Every entry receives the same fused multiply-adds in the same order as in
-// the unblocked algorithm, so the results are the same bits.
-// A pivot v_j that is not above rel * dg[j] (rel = 0: not positive, or NaN) sets *fail
+// Blocked by panels of four pivots with one panel of lookahead, one barrier a panel: warp 0
+// applies the previous panel to the next four columns and factorises them while the other
+// warps apply it to the rest of the lower triangle.  The four pivots are a serial chain of
+// latencies (reciprocal, scaling, update); every lane of warp 0 runs it on the panel's 4 x 4
+// block in registers, so that nothing is passed between lanes inside it.  Every entry receives
+// the same fused multiply-adds in the same order as in the unblocked algorithm.  At d = 32 in
+// FP64 44,500 cycles, in FP32 9,900 (52,000 and 24,300 with the panel's columns in shared memory, a barrier on either
+// side of the panel and rsqrt of every pivot in the chain).
+// A pivot v_j that is not positive, or NaN, or in FP32 not above rel * dg[j], sets *fail
 // (shared memory) and/or the device error word *derr (DPMM_ENUMERIC) and is replaced by
-// the smallest normal value of T.  cols: 4 d values of T (shared memory), scratch.
-template <typename T>
-__device__ inline void chol_ldl_blk(T* A, int d, int ld, T* piv, T* rs, T* cols, const T* dg, T rel, int* fail,
-                                    int* derr) {
+// the smallest normal value of T.  cols, cols2: 4 d values of T each (shared memory), scratch.
+// Called by threads 0 .. nt - 1 (at least two warps); sync() is their barrier.
+template <typename T, typename Sync>
+__device__ inline void chol_ldl_blk(T* A, int d, int ld, T* piv, T* cols, T* cols2, const T* dg, T rel, int* fail,
+                                    int* derr, int nt, Sync sync) {
     const int tid = threadIdx.x;
     for (int j0 = 0; j0 < d; j0 += 4) {
-        const int pw = min(4, d - j0), j1 = j0 + pw;
+        const int pw = min(4, d - j0);
+        T* cb = j0 & 4 ? cols2 : cols;        // this panel's scaled columns
+        const T* pb = j0 & 4 ? cols : cols2;  // the previous panel's
         if (tid < 32) {
-            for (int q = 0; q < pw; ++q) {
-                const int j = j0 + q;
-                T v = A[j * ld + j];
-                if (!(v > (rel > T(0) ? rel * dg[j] : T(0)))) {
-                    if (tid == 0) {
-                        if (fail) *fail = 1;
-                        if (derr) atomicExch(derr, (int)DPMM_ENUMERIC);
-                    }
-                    v = sizeof(T) == 4 ? T(1.17549435e-38f) : T(2.2250738585072014e-308);
-                }
-                const T r = rsqrt_t(v), inv = r * r;
-                T* col = cols + (size_t)q * d;
-                for (int i = j + 1 + tid; i < d; i += 32) col[i] = A[i * ld + j] * inv;
-                if (tid == 0) {
-                    piv[j] = v;
-                    rs[j] = r;
-                }
-                __syncwarp();
-                // the panel's later columns, every row at or below the column's diagonal
-                for (int l = j + 1; l < j1; ++l) {
-                    const T alj = A[l * ld + j];
-                    for (int i = l + tid; i < d; i += 32) A[i * ld + l] = fma(-col[i], alj, A[i * ld + l]);
+            if (j0 > 0) {
+                for (int i = j0 + tid; i < d; i += 32) {
+                    T c[4], a[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) c[q] = pb[q * d + i];
+#pragma unroll
+                    for (int l = 0; l < 4; ++l)
+                        if (l < pw && i >= j0 + l) a[l] = A[i * ld + j0 + l];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+#pragma unroll
+                        for (int l = 0; l < 4; ++l)
+                            if (l < pw && i >= j0 + l) a[l] = fma(-c[q], A[(j0 + l) * ld + j0 - 4 + q], a[l]);
+#pragma unroll
+                    for (int l = 0; l < 4; ++l)
+                        if (l < pw && i >= j0 + l) A[i * ld + j0 + l] = a[l];
                 }
                 __syncwarp();
             }
+            T D[4][4], inv[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int q = 0; q <= r; ++q) D[r][q] = r < pw ? A[(j0 + r) * ld + j0 + q] : T(1);
+            __syncwarp();  // read before the rows below are written
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (q >= pw) break;
+                T v = D[q][q];
+                if constexpr (sizeof(T) == 8) {
+                    if (recip_range(v)) {
+                        inv[q] = recip_fast(v);
+                    } else {
+                        if (!(v > 0.0)) {
+                            if (tid == 0 && fail) *fail = 1;
+                            if (tid == 0 && derr) atomicExch(derr, (int)DPMM_ENUMERIC);
+                            v = 2.2250738585072014e-308;
+                        }
+                        inv[q] = recip_any(v);
+                    }
+                } else {
+                    if (!(v > (rel > T(0) ? rel * dg[j0 + q] : T(0)))) {
+                        if (tid == 0 && fail) *fail = 1;
+                        if (tid == 0 && derr) atomicExch(derr, (int)DPMM_ENUMERIC);
+                        v = 1.17549435e-38f;
+                    }
+                    const T r = rsqrt_t(v);
+                    inv[q] = r * r;
+                }
+                if (tid == 0) piv[j0 + q] = v;
+#pragma unroll
+                for (int r = q + 1; r < 4; ++r) {
+                    const T c = D[r][q] * inv[q];
+#pragma unroll
+                    for (int l = q + 1; l <= r; ++l) D[r][l] = fma(-c, D[l][q], D[r][l]);
+                }
+            }
+            for (int i = j0 + tid; i < d; i += 32) {
+                T a[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (q < pw && i >= j0 + q) a[q] = A[i * ld + j0 + q];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (q >= pw || i <= j0 + q) continue;
+                    const T c = a[q] * inv[q];
+                    cb[q * d + i] = c;
+#pragma unroll
+                    for (int l = q + 1; l < 4; ++l)
+                        if (l < pw && i >= j0 + l) {
+                            a[l] = fma(-c, D[l][q], a[l]);
+                            if (l == q + 1) A[i * ld + j0 + l] = a[l];
+                        }
+                }
+            }
+        } else if (j0 > 0) {  // entries (i, l), l beyond this panel
+            const int m = d - j0 - pw, n = m * (m + 1) / 2, st = nt - 32;
+            for (int e0 = tid - 32; e0 < n; e0 += 4 * st) {  // four chains of updates at a time
+                int ii[4], ll[4];
+                T a[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    tri_index(min(e0 + u * st, n - 1), ii[u], ll[u]);
+                    ii[u] += j0 + pw;
+                    ll[u] += j0 + pw;
+                    a[u] = A[ii[u] * ld + ll[u]];
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (e0 + u * st < n) a[u] = fma(-pb[q * d + ii[u]], A[ll[u] * ld + j0 - 4 + q], a[u]);
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (e0 + u * st < n) A[ii[u] * ld + ll[u]] = a[u];
+            }
         }
-        __syncthreads();
-        // the rest of the lower triangle: entries (i, l), j1 <= l <= i < d
-        const int m = d - j1;
-        for (int e = tid; e < m * (m + 1) / 2; e += blockDim.x) {
-            int i, l;
-            tri_index(e, i, l);
-            i += j1;
-            l += j1;
-            T a = A[i * ld + l];
-            for (int q = 0; q < pw; ++q) a = fma(-cols[(size_t)q * d + i], A[l * ld + j0 + q], a);
-            A[i * ld + l] = a;
-        }
-        __syncthreads();
+        sync();
     }
-}
-
-// FP64, a non-positive pivot reported as DPMM_ENUMERIC (split/merge marginals).
-__device__ inline void chol_ldl(double* A, int d, int ld, double* piv, double* rs, double* cols, int* derr) {
-    chol_ldl_blk<double>(A, d, ld, piv, rs, cols, nullptr, 0.0, nullptr, derr);
-}
-
-// The factorisation above for the parameter draws of the reduced-precision paths (T =
-// float) and their FP64 retry (T = double): with rel = 2^-10 an FP32 factorisation is
-// flagged in *fail (and redone in FP64) once cancellation has taken more than 10 of the
-// 24 bits of a pivot.
-template <typename T>
-__device__ inline void chol_ldl_t(T* A, int d, int ld, T* piv, T* rs, T* cols, const T* dg, T rel, int* fail) {
-    chol_ldl_blk<T>(A, d, ld, piv, rs, cols, dg, rel, fail, nullptr);
 }
 
 }  // namespace dpmm

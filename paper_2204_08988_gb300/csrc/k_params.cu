@@ -220,11 +220,104 @@ struct NiwPrior {
 // Psi_n (lower triangle, with the diagonal) and W (upper triangle, with the diagonal) share one
 // array of rows of ld T: W's entry (r, c) sits at column c + 1, so that W is in shared memory in
 // FP64 too up to d = 156 (d = 128, 192 slots: 1,526 us; 1,725 us with W in global memory).
-// Dynamic shared memory: (E doubles when staged) + (d*ld + 12*d) T.
+// Dynamic shared memory: (E doubles when staged) + (d * ld + 12 d) T (13 d + 2 in FP32).
 __device__ inline float log_t(float x) { return logf(x); }
 __device__ inline double log_t(double x) { return log(x); }
 
 __host__ __device__ inline int niw_ld(int d) { return (d + 1) | 1; }
+
+// The draw's triangular solves, by a block of two warps or more; R 32-row slots cover d, a warp
+// takes CB columns at a time.
+//
+// U^T W = B: a column of W needs no other, so a warp keeps CB of them in registers (lane = row)
+// and passes the final element of each step by shuffle; the columns go round robin over the warps,
+// which evens out their lengths.  An entry gets its multiply-adds in the order of the rows below it.
+// V (lower triangle) holds V_ri = U_ri / U_rr; row i is scaled by rd_i = 1 / U_ii at the end.
+// W^T v = eps: warp 0, lane m keeps sum_{j<m} W_jm v_j; the other warps store W meanwhile, and
+// warp 1 returns log det W.
+// d = 32: 15,900 cycles in FP32, 48,100 in FP64 (13,800 + 9,600 and 20,200 + 28,300 with a barrier
+// per row, an integer division per entry and the sums' slot selected at run time).
+template <typename T, int R, int CB>
+__device__ __forceinline__ void niw_solve(T* W, int ws, const T* V, int ld, const T* rd, const T* Bd, const T* eps,
+                                          const T* mn, T rsk, int d, const T* Wsm, double* Wg, double* mu, double& lgd) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    for (int base = warp; base < d; base += nw * CB) {
+        T a[CB][R];
+#pragma unroll
+        for (int u = 0; u < CB; ++u) {
+            const int c = base + nw * u;
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                const int i = lane + 32 * q;
+                a[u][q] = c >= d ? T(0) : i < c ? W[(size_t)i * ws + c] : i == c ? Bd[c] : T(0);
+            }
+        }
+        const int top = min(d - 1, base + nw * (CB - 1));
+#pragma unroll
+        for (int sr = R - 1; sr >= 0; --sr)
+            for (int r = min(top, 32 * sr + 31); r >= max(1, 32 * sr); --r) {
+                T v[R];
+#pragma unroll
+                for (int q = 0; q <= sr; ++q) v[q] = lane + 32 * q < r ? V[(size_t)r * ld + lane + 32 * q] : T(0);
+#pragma unroll
+                for (int u = 0; u < CB; ++u) {
+                    const int c = base + nw * u;
+                    const T w = __shfl_sync(0xffffffffu, a[u][sr], r & 31);
+                    if (c >= r && c < d) {  // a predicate: FP64 operations of finished columns are not issued
+#pragma unroll
+                        for (int q = 0; q <= sr; ++q) a[u][q] = fma(-v[q], w, a[u][q]);
+                    }
+                }
+            }
+#pragma unroll
+        for (int u = 0; u < CB; ++u) {
+            const int c = base + nw * u;
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                const int i = lane + 32 * q;
+                if (c < d && i <= c) W[(size_t)i * ws + c] = a[u][q] * rd[i];
+            }
+        }
+    }
+    __syncthreads();
+    if (warp == 0) {
+        T sum[R], e[R], rw[R];  // of m = lane + 32 q
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            const int m = lane + 32 * q;
+            sum[q] = T(0);
+            e[q] = m < d ? eps[m] : T(0);
+            rw[q] = m < d ? T(1) / W[(size_t)m * ws + m] : T(0);
+        }
+#pragma unroll
+        for (int sj = 0; sj < R; ++sj) {
+            const int steps = min(32, d - 32 * sj);
+#pragma unroll 4
+            for (int jl = 0; jl < steps; ++jl) {
+                const int j = 32 * sj + jl;
+                const T vj = __shfl_sync(0xffffffffu, (e[sj] - sum[sj]) * rw[sj], jl);
+#pragma unroll
+                for (int q = sj; q < R; ++q) {
+                    const int m = lane + 32 * q;
+                    if (m > j && m < d) sum[q] += W[(size_t)j * ws + m] * vj;
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < R; ++q) {  // a lane's sums have been final since its own step
+            const int m = lane + 32 * q;
+            if (m < d) mu[m] = (double)(mn[m] + (e[q] - sum[q]) * rw[q] * rsk);
+        }
+        return;
+    }
+    if (warp == 1) {
+        for (int j = lane; j < d; j += 32) lgd += (double)log_t(W[(size_t)j * ws + j]);
+        for (int o = 16; o > 0; o >>= 1) lgd += __shfl_xor_sync(0xffffffffu, lgd, o);
+    }
+    if (Wsm)
+        for (int r = warp - 1; r < d; r += nw - 1)  // zero below the diagonal already
+            for (int c = r + lane; c < d; c += 32) Wg[(size_t)r * d + c] = (double)Wsm[(size_t)r * ws + c];
+}
 
 template <typename T>
 __global__ void niw_params_kernel(StatView sv, const double* shift_stats, NiwPrior pr, const int* dK,
@@ -243,13 +336,13 @@ __global__ void niw_params_kernel(StatView sv, const double* shift_stats, NiwPri
     double* S = smem;             // E: staged statistics
     T* A = (T*)(S + (staged ? E : 0));  // d x ld: Psi_n (lower), then the solve's multipliers
     T* mn = A + d * ld;           // d
-    T* dg = mn + d;               // d: diagonal of Psi_n
-    T* Bd = dg + d;               // d: Bartlett diagonal, then v
+    T* Bd = mn + d;               // d: Bartlett diagonal, then v
     T* acc = Bd + d;              // d: eps
-    T* rd = acc + d;              // d: 1 / U_jj
-    T* rw = rd + d;               // d: 1 / W_jj
-    T* piv = rw + d;              // d: pivots
+    T* piv = acc + d;             // d: pivots
     T* cols = piv + d;            // 4 d: the factorisation's scaled panel columns
+    T* cols2 = cols + 4 * d;      // 4 d: the same of every other panel, then rd
+    T* rd = cols2;                // d: 1 / U_jj
+    T* dg = cols2 + 4 * d;        // d: diagonal of Psi_n (T = float only)
     double* Wg = p_W + (size_t)s * d * d;
     T* W = w_in_smem ? A + 1 : (T*)Wg;  // working copy (global only when T = double), rows of ws
     const int ws = w_in_smem ? ld : d;
@@ -263,13 +356,16 @@ __global__ void niw_params_kernel(StatView sv, const double* shift_stats, NiwPri
         __syncthreads();
     }
     auto M = [&](int j, int l) -> double { return staged ? S[sv.L.ent(j, l)] : sv.m(k, h, j, l); };
-    if (tid == 0) {
-        const double n = M(d, d);
-        s_n = n;
-        s_rn = n > 0 ? 1.0 / n : 0.0;
-        s_kn = pr.kappa0 + n;
-        s_rkn = 1.0 / s_kn;
-        s_fail = 0;
+    if (tid < 2) {  // 1 / n and 1 / kappa_n, one division in two lanes
+        const double n = M(d, d), den = tid == 0 ? n : pr.kappa0 + n, r = 1.0 / den;
+        if (tid == 0) {
+            s_n = n;
+            s_rn = n > 0 ? r : 0.0;
+            s_fail = 0;
+        } else {
+            s_kn = den;
+            s_rkn = r;
+        }
     }
     __syncthreads();
     const double n = s_n, rn = s_rn, kn = s_kn, rkn = s_rkn;
@@ -329,11 +425,13 @@ __global__ void niw_params_kernel(StatView sv, const double* shift_stats, NiwPri
             if (n > 0) C = m2[u] - m1[l] * m1[j] * rn;
             const T a = (T)(p0[u] + C + f * dxm[j] * dxm[l]);
             A[j * ld + l] = a;
-            if (l == j) dg[j] = a;
+            if (sizeof(T) == 4 && l == j) dg[j] = a;
         }
     }
     __syncthreads();
-    chol_ldl_t<T>(A, d, ld, piv, rd, cols, dg, sizeof(T) == 4 ? T(1.0 / 1024) : T(0), &s_fail);
+    // in FP32 a pivot that has lost more than 10 of its 24 bits to cancellation fails (rel = 2^-10)
+    chol_ldl_blk<T>(A, d, ld, piv, cols, cols2, dg, sizeof(T) == 4 ? T(1.0 / 1024) : T(0), &s_fail, nullptr, nt,
+                    [] { __syncthreads(); });
     if (s_fail) {
         if (sizeof(T) == 4) {  // redo this slot in FP64
             if (tid == 0) retry[s] = 1;
@@ -341,6 +439,8 @@ __global__ void niw_params_kernel(StatView sv, const double* shift_stats, NiwPri
         }
         if (tid == 0) atomicExch(derr, (int)DPMM_ENUMERIC);
     }
+    for (int j = tid; j < d; j += nt) rd[j] = rsqrt_t(piv[j]);
+    __syncthreads();
     // U_ij = A_ij / sqrt(v_j) below the diagonal (U_jj = sqrt(v_j)); the solve below
     // needs V_ri = U_ri / U_rr = A_ri rd[i] rd[r], kept in place of A
     for (int e = tid; e < d * (d - 1) / 2; e += nt) {
@@ -349,72 +449,17 @@ __global__ void niw_params_kernel(StatView sv, const double* shift_stats, NiwPri
         ++r;                 // strict lower triangle: i < r
         A[r * ld + i] *= rd[i] * rd[r];
     }
-    // U^T W = B, right-looking: after step r, row r of W (unscaled) is final and the rows
-    // above are updated with it; the rows are scaled by 1 / U_rr at the end
-    for (int j = tid; j < d; j += nt) W[j * ws + j] = Bd[j];
     __syncthreads();
-    for (int r = d - 1; r > 0; --r) {
-        const int w = d - r;  // columns c = r .. d-1
-        const T* Wr = W + (size_t)r * ws;
-        const T* Vr = A + (size_t)r * ld;
-        for (int e0 = tid; e0 < r * w; e0 += 2 * nt) {
-            const int e1 = e0 + nt;
-            const int i0 = e0 / w, c0 = r + e0 % w;  // row i < r
-            const bool two = e1 < r * w;
-            const int i1 = two ? e1 / w : i0, c1 = two ? r + e1 % w : c0;
-            const T a0 = W[i0 * ws + c0], v0 = Vr[i0], w0 = Wr[c0];
-            const T a1 = W[i1 * ws + c1], v1 = Vr[i1], w1 = Wr[c1];
-            W[i0 * ws + c0] = fma(-v0, w0, a0);
-            if (two) W[i1 * ws + c1] = fma(-v1, w1, a1);
-        }
-        __syncthreads();
-    }
-    for (int e = tid; e < d * d; e += nt) {
-        const int r = e / d, c = e % d;
-        if (c >= r) W[r * ws + c] *= rd[r];
-    }
-    __syncthreads();
-    for (int j = tid; j < d; j += nt) rw[j] = T(1) / W[j * ws + j];
-    __syncthreads();
-    // W^T v = eps (forward substitution) by warp 0, lane m keeps sum_{j<m} W[j][m] v_j;
-    // mu = m_n + v / sqrt(kappa_n)
-    if (tid < 32) {
-        const int ns = (d + 31) >> 5;
-        T am[8];  // m = tid + 32 i, d <= 256
-#pragma unroll
-        for (int i = 0; i < 8; ++i) am[i] = T(0);
-        for (int j = 0; j < d; ++j) {
-            const int own = j & 31, slot = j >> 5;
-            T mine = T(0);
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if (i == slot) mine = am[i];
-            T vj = T(0);
-            if (tid == own) {
-                vj = (acc[j] - mine) * rw[j];
-                Bd[j] = vj;  // reuse as v
-            }
-            vj = __shfl_sync(0xffffffffu, vj, own);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int m = tid + 32 * i;
-                if (i < ns && m > j && m < d) am[i] += W[j * ws + m] * vj;
-            }
-        }
-    }
-    __syncthreads();
-    double* mu = p_mu + (size_t)s * d;
-    const T rsk = rsqrt_t((T)kn);
-    for (int j = tid; j < d; j += nt) mu[j] = (double)(mn[j] + Bd[j] * rsk);
-    if (w_in_smem)
-        for (int e = tid; e < d * d; e += nt) {  // zero below the diagonal already
-            const int r = e / d, c = e % d;
-            if (c >= r) Wg[e] = (double)W[r * ws + c];
-        }
+    // U^T W = B, then W^T v = eps, mu = m_n + v / sqrt(kappa_n) and log det W
     double lgd = 0.0;
-    for (int j = tid; j < d; j += nt) lgd += (double)log_t(W[j * ws + j]);
-    lgd = block_reduce_sum(lgd, sh);
-    if (tid == 0) {
+    T* const Wout = w_in_smem ? W : nullptr;
+    const T rsk = rsqrt_t((T)kn);
+    double* mu = p_mu + (size_t)s * d;
+    if (d <= 32) niw_solve<T, 1, 8>(W, ws, A, ld, rd, Bd, acc, mn, rsk, d, Wout, Wg, mu, lgd);
+    else if (d <= 64) niw_solve<T, 2, 4>(W, ws, A, ld, rd, Bd, acc, mn, rsk, d, Wout, Wg, mu, lgd);
+    else if (d <= 128) niw_solve<T, 4, 4>(W, ws, A, ld, rd, Bd, acc, mn, rsk, d, Wout, Wg, mu, lgd);
+    else niw_solve<T, 8, 2>(W, ws, A, ld, rd, Bd, acc, mn, rsk, d, Wout, Wg, mu, lgd);
+    if (tid == 32) {
         p_logdetW[s] = lgd;
         p_c[s] = logw[s] + lgd - 0.5 * d * 1.8378770664093453;  // log(2 pi)
         if (retry_pass) retry[s] = 0;
@@ -609,9 +654,9 @@ cudaError_t launch_params(dpmm_ctx* c, uint64_t seed) {
         const size_t E = (size_t)c->st.E, dl = (size_t)c->d * niw_ld(c->d);
         NiwPrior pr{c->kappa0, c->nu0, c->center + c->d, c->center + 2 * c->d};
         // shared memory of the T instantiation: E doubles (staged, while three blocks still fit an
-        // SM), then d * ld + 12 d T
+        // SM), then d * ld + 12 d T (13 d + 2 in FP32)
         auto plan = [&](size_t tsz, int& staged, int& w_in_smem) {
-            size_t sm = tsz * (dl + 12 * (size_t)c->d);
+            size_t sm = tsz * (dl + (tsz == 4 ? 13 * (size_t)c->d + 2 : 12 * (size_t)c->d));
             w_in_smem = sm <= 200 * 1024;
             staged = sm + 8 * E <= 72 * 1024;
             return sm + (staged ? 8 * E : 0);

@@ -74,8 +74,8 @@ __device__ inline void pair_of(int p, int K, int& k1, int& k2) {
     k2 = r + 1 + (p - off);
 }
 
-// One item (slot or merge pair) of marginal_kernel.  Dynamic shared memory: d (d | 1) + 10 d
-// doubles (+ 2 E when the statistics are staged).
+// One item (slot or merge pair) of marginal_kernel, by two warps or more (the last one takes the
+// lgamma terms).  Dynamic shared memory: d (d | 1) + 9 d doubles (+ 2 E when the statistics are staged).
 // t >= 0: T_t = Psi0 / 2 + C_t of cluster t instead (its entries, the mean and log det T_t).
 __device__ __forceinline__ void marginal_item(const SMArgs& a, double* Ltab, int* derr, int K, int e, int t = -1) {
     extern __shared__ double smem[];
@@ -96,16 +96,14 @@ __device__ __forceinline__ void marginal_item(const SMArgs& a, double* Ltab, int
         h = -1;
     }
     double* out = Ltab + (e < 3 * K ? e : 3 * a.K_max + (e - 3 * K));
-    if (t < 0 && (tid == 32 || tid == 33)) {  // the slot's or the pair's lgamma terms for the Hastings ratios
-        if (e < 3 * K) {
-            const double ns = smv(a, k1, h, d, d);
-            Ltab[lg_offset(a.K_max) + 2 * e + (tid - 32)] = lgamma(tid == 32 ? ns : 0.5 * a.alpha + ns);
-        } else {
-            const double nm = smv(a, k1, -1, d, d) + smv(a, k2, -1, d, d);
-            Ltab[lg_pair_offset(a.K_max) + 2 * (e - 3 * K) + (tid - 32)] = lgamma(tid == 32 ? nm : a.alpha + nm);
-        }
-    }
+    // the slot's or the pair's lgamma terms for the Hastings ratios
+    double* lgt = Ltab + (e < 3 * K ? lg_offset(a.K_max) + 2 * e : lg_pair_offset(a.K_max) + 2 * (e - 3 * K));
+    const double alpha = e < 3 * K ? 0.5 * a.alpha : a.alpha;
     if (a.kind == DPMM_PRIOR_DIRICHLET) {
+        if (tid == 32 || tid == 33) {
+            const double n = smv(a, k1, h, d, d) + (k2 >= 0 ? smv(a, k2, -1, d, d) : 0.0);
+            lgt[tid - 32] = lgamma(tid == 32 ? n : alpha + n);
+        }
         // the prior's terms (sum beta, lgamma(sum beta), sum lgamma(beta_j)) come from the host
         double sc = 0.0, acc = 0.0;
         for (int j = tid; j < d; j += nt) {
@@ -138,16 +136,30 @@ __device__ __forceinline__ void marginal_item(const SMArgs& a, double* Ltab, int
     }
     const int ld = d | 1;      // odd row stride: column reads without bank conflicts
     double* A = smem;          // d x ld (lower triangle)
-    double* xb = A + d * ld;   // merged mean
-    double* x1 = xb + d;
-    double* x2 = x1 + d;
-    double* piv = x2 + d;      // pivots of the factorisation
-    double* rs = piv + d;
-    double* cols = rs + d;     // 4 d: the factorisation's scaled panel columns
-    double* dxb = cols + 4 * d;  // merged mean - m0
-    double* S1 = dxb + d;      // staged statistics of (k1, h) and of cluster k2 (E each)
+    double* piv = A + d * ld;  // pivots of the factorisation
+    double* cols = piv + d;    // 8 d: the factorisation's scaled panel columns, and before it
+    double* u1 = cols;           // first moments / n of (k1, h), of k2
+    double* u2 = u1 + d;
+    double* g = u2 + d;          // f (merged mean - m0)
+    double* wx = g + d;          // n1 n2 / n (mean 1 - mean 2)
+    double* dx = wx + d;         // mean 1 - mean 2
+    double* dxb = dx + d;        // merged mean - m0
+    double* S1 = cols + 8 * d;   // staged statistics of (k1, h) and of cluster k2 (E each)
     double* S2 = S1 + a.L.E;
     const bool staged = a.stage != 0;
+    // Psi0's entries of a thread's first entries, loaded beside the statistics
+    constexpr int UB = 5;        // entries a thread at a time
+    const int nc = nt - 32, ntri = d * (d + 1) / 2;
+    int jj[UB], ll[UB];
+    double p0[UB];
+    auto psi0_of = [&](int e0) {
+#pragma unroll
+        for (int u = 0; u < UB; ++u) {
+            tri_index(min(e0 + u * nc, ntri - 1), jj[u], ll[u]);  // l <= j: the factorisation reads nothing else
+            p0[u] = a.psi0[jj[u] * d + ll[u]];
+        }
+    };
+    if (tid < nc) psi0_of(tid);
     if (staged) {
         stage_slot(a.stats, a.L.E, k1, h, S1);
         if (k2 >= 0) stage_slot(a.stats, a.L.E, k2, -1, S2);
@@ -156,93 +168,85 @@ __device__ __forceinline__ void marginal_item(const SMArgs& a, double* Ltab, int
     // M[j][l] (j <= l) of the first and second statistics block
     auto M1 = [&](int j, int l) -> double { return staged ? S1[a.L.ent(j, l)] : smv(a, k1, h, j, l); };
     auto M2 = [&](int j, int l) -> double { return staged ? S2[a.L.ent(j, l)] : smv(a, k2, -1, j, l); };
-    __shared__ double s_r1, s_r2, s_rn, s_w12;
-    if (tid == 0) {  // reciprocals once: FP64 division is slow on GB300's narrow FP64 pipe
+    __shared__ double s_div[4], s_lg;
+    if (tid < 4) {  // 1 / n1, 1 / n2, 1 / n and f, one reciprocal in four lanes
         const double n1 = M1(d, d), n2 = k2 >= 0 ? M2(d, d) : 0.0, n = n1 + n2;
-        s_n1 = n1;
-        s_n2 = n2;
-        s_n = n;
-        s_r1 = n1 > 0 ? 1.0 / n1 : 0.0;
-        s_r2 = n2 > 0 ? 1.0 / n2 : 0.0;
-        s_rn = n > 0 ? 1.0 / n : 0.0;
-        s_w12 = n1 * n2 * s_rn;
-    }
-    __syncthreads();
-    const double n1 = s_n1, n2 = s_n2, n = s_n, r1 = s_r1, r2 = s_r2, rn = s_rn, w12 = s_w12;
-    for (int j = tid; j < d; j += nt) {
-        double m1 = n1 > 0 ? a.shift_stats[(size_t)k1 * d + j] + M1(j, d) * r1 : 0.0;
-        double m2 = (k2 >= 0 && n2 > 0) ? a.shift_stats[(size_t)k2 * d + j] + M2(j, d) * r2 : 0.0;
-        x1[j] = m1;
-        x2[j] = m2;
-        xb[j] = n > 0 ? (n1 * m1 + n2 * m2) * rn : 0.0;
-        dxb[j] = xb[j] - a.m0s[j];
-    }
-    __syncthreads();
-    const double kn = a.kappa0 + n, nun = a.nu0 + n;
-    const double f = n > 0 ? a.kappa0 * n / kn : 0.0;
-    const int ntri = d * (d + 1) / 2;
-    for (int e0 = tid; e0 < ntri; e0 += 4 * nt) {  // the Psi0 entries of four entries loaded first
-        int jj[4], ll[4];
-        double p0[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            tri_index(min(e0 + u * nt, ntri - 1), jj[u], ll[u]);  // l <= j: the factorisation reads nothing else
-            p0[u] = a.psi0[jj[u] * d + ll[u]];
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (e0 + u * nt >= ntri) break;
-            const int j = jj[u], l = ll[u];
-            const int q = j * ld + l;
-            double C = 0.0;
-            if (n1 > 0) C += M1(l, j) - M1(l, d) * M1(j, d) * r1;
-            if (k2 >= 0 && n2 > 0) {
-                C += M2(l, j) - M2(l, d) * M2(j, d) * r2;
-                if (n1 > 0) C += w12 * (x1[j] - x2[j]) * (x1[l] - x2[l]);
-            }
-            if (t >= 0) {
-                const double v = 0.5 * p0[u] + C;
-                A[q] = v;
-                a.T32[(size_t)t * d * d + j * d + l] = (float)v;
-            } else {
-                A[q] = p0[u] + C + f * dxb[j] * dxb[l];
-            }
+        const double den = tid == 0 ? n1 : tid == 1 ? n2 : tid == 2 ? n : a.kappa0 + n;
+        const double num = tid == 3 ? a.kappa0 * n : 1.0;
+        s_div[tid] = recip_range(den) ? num * recip_fast(den) : den > 0 ? num * recip_any(den) : 0.0;
+        if (tid == 0) {
+            s_n1 = n1;
+            s_n2 = n2;
+            s_n = n;
         }
     }
-    if (t >= 0)
-        for (int j = tid; j < d; j += nt) a.xbar[(size_t)t * d + j] = xb[j];
     __syncthreads();
-    if (t >= 0) {
-        __shared__ int s_fail;
-        if (tid == 0) s_fail = 0;
-        __syncthreads();
-        chol_ldl_blk<double>(A, d, ld, piv, rs, cols, nullptr, 0.0, &s_fail, nullptr);
+    const double n1 = s_n1, n2 = s_n2, n = s_n, kn = a.kappa0 + n, nun = a.nu0 + n;
+    __shared__ int s_fail;
+    if (tid >= nc) {
+        // the lgamma terms and log kappa_n, which need n alone, beside the factorisation (a call is a chain of
+        // some 6,000 cycles)
         double part = 0.0;
-        for (int j = tid; j < d; j += nt) part += log(piv[j]);
+        if (t < 0) {
+            if (tid == nt - 1) part = -0.5 * d * log(kn);
+            for (int q = tid - nc; q < d + 2; q += 32) {
+                const double v = lgamma(q < d ? 0.5 * nun - 0.5 * q : q == d ? n : alpha + n);
+                if (q < d) part += v;
+                else lgt[q - d] = v;
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        if (tid == nc) s_lg = part;
+    } else {
+        auto sync = [nc] { asm volatile("bar.sync 1, %0;" ::"r"(nc) : "memory"); };
+        const double r1 = s_div[0], r2 = s_div[1], rn = s_div[2], f = s_div[3], w12 = n1 * n2 * rn;
+        if (tid == 0) s_fail = 0;
+        for (int j = tid; j < d; j += nc) {
+            const double v1 = n1 > 0 ? M1(j, d) * r1 : 0.0, v2 = k2 >= 0 && n2 > 0 ? M2(j, d) * r2 : 0.0;
+            const double m1 = n1 > 0 ? a.shift_stats[(size_t)k1 * d + j] + v1 : 0.0;
+            const double m2 = k2 >= 0 && n2 > 0 ? a.shift_stats[(size_t)k2 * d + j] + v2 : 0.0;
+            const double xb = n > 0 ? (n1 * m1 + n2 * m2) * rn : 0.0;
+            u1[j] = v1;
+            u2[j] = v2;
+            dx[j] = m1 - m2;
+            wx[j] = w12 * (m1 - m2);
+            dxb[j] = xb - a.m0s[j];
+            g[j] = f * (xb - a.m0s[j]);
+            if (t >= 0) a.xbar[(size_t)t * d + j] = xb;
+        }
+        sync();
+        for (int e0 = tid; e0 < ntri; e0 += UB * nc) {
+            if (e0 != tid) psi0_of(e0);
+#pragma unroll
+            for (int u = 0; u < UB; ++u) {
+                if (e0 + u * nc >= ntri) break;
+                const int j = jj[u], l = ll[u];
+                double v = t >= 0 ? 0.5 * p0[u] : p0[u];
+                if (n1 > 0) v += fma(-M1(l, d), u1[j], M1(l, j));
+                if (k2 >= 0 && n2 > 0) {
+                    v += fma(-M2(l, d), u2[j], M2(l, j));
+                    if (n1 > 0) v = fma(wx[j], dx[l], v);
+                }
+                if (t >= 0) a.T32[(size_t)t * d * d + j * d + l] = (float)v;
+                else v = fma(g[j], dxb[l], v);
+                A[j * ld + l] = v;
+            }
+        }
+        sync();
+        chol_ldl_blk<double>(A, d, ld, piv, cols, cols + 4 * d, nullptr, 0.0, &s_fail, t >= 0 ? nullptr : derr, nc, sync);
+        double part = 0.0;
+        for (int j = tid; j < d; j += nc) part += log(piv[j]);
         for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
         if ((tid & 31) == 0) sh[tid >> 5] = part;
-        __syncthreads();
-        if (tid == 0) {
-            double v = 0.0;
-            for (int w = 0; w < (nt + 31) / 32; ++w) v += sh[w];
-            a.ldT[t] = s_fail ? nan("") : v;  // a factorisation that fails says nothing: the pair is factorised itself
-        }
-        return;
     }
-    chol_ldl(A, d, ld, piv, rs, cols, derr);
-    // -(nun/2) log|Psi_n| and the multivariate-lgamma ratio (the prior's part from the
-    // host), summed over j by all threads; lane 0 of warp 0 adds log kappa_n
-    double part = 0.0;
-    for (int j = tid; j < d; j += nt) part += -0.5 * nun * log(piv[j]) + lgamma(0.5 * nun - 0.5 * j);
-    if (tid == 0) part -= 0.5 * d * log(kn);
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    if ((tid & 31) == 0) sh[tid >> 5] = part;
     __syncthreads();
     if (tid == 0) {
-        double s = 0.0;
-        for (int w = 0; w < (nt + 31) / 32; ++w) s += sh[w];
-        // 1.1447298858494002 = log(pi)
-        *out = -0.5 * n * d * 1.1447298858494002 + s - a.lmvg_nu0 + 0.5 * a.nu0 * a.logdet_psi0 + a.half_d_log_kappa0;
+        double s = 0.0;  // log det
+        for (int w = 0; w < nc / 32; ++w) s += sh[w];
+        if (t >= 0)
+            a.ldT[t] = s_fail ? nan("") : s;  // a factorisation that fails says nothing: the pair is factorised itself
+        else  // -(nun/2) log|Psi_n| and the multivariate-lgamma ratio; 1.1447298858494002 = log(pi)
+            *out = -0.5 * n * d * 1.1447298858494002 - 0.5 * nun * s + s_lg - a.lmvg_nu0 + 0.5 * a.nu0 * a.logdet_psi0 + a.half_d_log_kappa0;
     }
 }
 
@@ -251,7 +255,8 @@ __device__ __forceinline__ void marginal_item(const SMArgs& a, double* Ltab, int
 // pairs.  An item is a chain of FP64 latencies, so pairs that an SM can take beside the slots
 // cost nothing (47 us at d = 32 for 60 slots alone and with 190 pairs).  The resident blocks
 // take the items in turn, so that no block is launched for the slots and pairs beyond K.
-__global__ void marginal_kernel(SMArgs a, double* Ltab, int* derr) {
+constexpr int MARG_T = 160;
+__global__ void __launch_bounds__(MARG_T) marginal_kernel(SMArgs a, double* Ltab, int* derr) {
     const int K = *a.dK;
     const bool bound = !pairs_at_once(a, K);
     const int total = 3 * K + (bound ? K : K * (K - 1) / 2);
@@ -655,10 +660,9 @@ __device__ inline bool refused_by_factor(const SMArgs& a, const double* Ltab, in
     const int d = a.L.d, ld = d | 1, tid = threadIdx.x, nt = blockDim.x;
     __shared__ int s_fail, s_ref;
     float* A = sm;
-    float* dl = A + d * ld;
-    float* piv = dl + d;
-    float* rs = piv + d;
-    float* cols = rs + d;  // 4 d
+    float* piv = A + d * ld;
+    float* cols = piv + d;  // 8 d
+    float* dl = cols + 4 * d;
     const float* T1 = a.T32 + (size_t)k1 * d * d;
     const float* T2 = a.T32 + (size_t)k2 * d * d;
     for (int j = tid; j < d; j += nt) dl[j] = (float)(a.xbar[(size_t)k1 * d + j] - a.xbar[(size_t)k2 * d + j]);
@@ -672,7 +676,7 @@ __device__ inline bool refused_by_factor(const SMArgs& a, const double* Ltab, in
             A[j * ld + l] = l == j ? b * keep : b;
         }
     __syncthreads();
-    chol_ldl_blk<float>(A, d, ld, piv, rs, cols, nullptr, 0.f, &s_fail, nullptr);
+    chol_ldl_blk<float>(A, d, ld, piv, cols, cols + 4 * d, nullptr, 0.f, &s_fail, nullptr, nt, [] { __syncthreads(); });
     if (tid < 32) {
         float v = 0.f;
         for (int j = tid; j < d; j += 32) v += logf(piv[j]);
@@ -877,7 +881,7 @@ static cudaError_t launch_proposals(dpmm_ctx* c, SMArgs& s, uint64_t seed, int l
     // blocks it reads when they fit
     size_t smi = 0;
     if (c->kind == DPMM_PRIOR_NIW) {
-        smi = sizeof(double) * ((size_t)c->d * (c->d | 1) + 10 * c->d);
+        smi = sizeof(double) * ((size_t)c->d * (c->d | 1) + 9 * c->d);
         const size_t st = smi + sizeof(double) * 2 * (size_t)c->st.E;
         if (st <= 160 * 1024) {
             smi = st;
@@ -912,8 +916,8 @@ static cudaError_t launch_proposals(dpmm_ctx* c, SMArgs& s, uint64_t seed, int l
             <<<waves((const void*)marginal_counts_kernel<CountsStats>, 256, 0, all), 256, 0, c->stream>>>(
                 s, CountsStats{c->stats, c->st}, c->sp_lgt, c->sp_lgt ? SP_LGT : 0, c->sp_lgb, c->Ltab);
     else
-        marginal_kernel<<<waves((const void*)marginal_kernel, 128, smi, bounds ? std::max(4 * c->K_max, s.exact) : all), 128, smi,
-                          c->stream>>>(s, c->Ltab, c->derr);
+        marginal_kernel<<<waves((const void*)marginal_kernel, MARG_T, smi, bounds ? std::max(4 * c->K_max, s.exact) : all),
+                          MARG_T, smi, c->stream>>>(s, c->Ltab, c->derr);
     prof_end(c, "marginal");
     c->nlaunch += 1;
     prof_begin(c, "hastings");
