@@ -68,10 +68,10 @@ static __device__ __noinline__ double recip_any(double v) { return 1.0 / v; }
 // Blocked by panels of four pivots with one panel of lookahead, one barrier a panel: warp 0
 // applies the previous panel to the next four columns and factorises them while the other
 // warps apply it to the rest of the lower triangle.  The four pivots are a serial chain of
-// latencies (reciprocal, scaling, update); every lane of warp 0 runs it on the panel's 4 x 4
-// block in registers, so that nothing is passed between lanes inside it.  Every entry receives
+// latencies (reciprocal, scaling, update) in registers, lane = row; the panel's 4 x 4 block passes by
+// shuffle (in every lane redundantly it costs 16 FP64 instructions a panel, at 19 cycles of the pipe).  Every entry receives
 // the same fused multiply-adds in the same order as in the unblocked algorithm.  At d = 32 in
-// FP64 44,500 cycles, in FP32 9,900 (52,000 and 24,300 with the panel's columns in shared memory, a barrier on either
+// FP64 33,800 cycles, in FP32 8,000 (52,000 and 24,300 with the panel's columns in shared memory, a barrier on either
 // side of the panel and rsqrt of every pivot in the chain).
 // A pivot v_j that is not positive, or NaN, or in FP32 not above rel * dg[j], sets *fail
 // (shared memory) and/or the device error word *derr (DPMM_ENUMERIC) and is replaced by
@@ -105,16 +105,18 @@ __device__ inline void chol_ldl_blk(T* A, int d, int ld, T* piv, T* cols, T* col
                 }
                 __syncwarp();
             }
-            T D[4][4], inv[4];
+            // the panel's first 32 rows with the pivots: lane = row; what the lanes need of the 4 x 4
+            // block comes by shuffle (D_lq = A_l,j0+q)
+            const int i0 = j0 + tid;
+            T a[4], D[4][4], inv[4];
 #pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int q = 0; q <= r; ++q) D[r][q] = r < pw ? A[(j0 + r) * ld + j0 + q] : T(1);
-            __syncwarp();  // read before the rows below are written
+            for (int q = 0; q < 4; ++q) a[q] = i0 < d && tid >= q && q < pw ? A[i0 * ld + j0 + q] : T(0);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 if (q >= pw) break;
-                T v = D[q][q];
+                T v = __shfl_sync(0xffffffffu, a[q], q);
+#pragma unroll
+                for (int l = q + 1; l < 4; ++l) D[l][q] = __shfl_sync(0xffffffffu, a[q], l);
                 if constexpr (sizeof(T) == 8) {
                     if (recip_range(v)) {
                         inv[q] = recip_fast(v);
@@ -136,30 +138,31 @@ __device__ inline void chol_ldl_blk(T* A, int d, int ld, T* piv, T* cols, T* col
                     inv[q] = r * r;
                 }
                 if (tid == 0) piv[j0 + q] = v;
+                const T c = a[q] * inv[q];
 #pragma unroll
-                for (int r = q + 1; r < 4; ++r) {
-                    const T c = D[r][q] * inv[q];
-#pragma unroll
-                    for (int l = q + 1; l <= r; ++l) D[r][l] = fma(-c, D[l][q], D[r][l]);
-                }
+                for (int l = q + 1; l < 4; ++l) a[l] = fma(-c, D[l][q], a[l]);  // kept where l <= row
+                if (i0 < d && tid > q) cb[q * d + i0] = c;
             }
-            for (int i = j0 + tid; i < d; i += 32) {
-                T a[4];
+#pragma unroll
+            for (int q = 1; q < 4; ++q)
+                if (q < pw && i0 < d && tid >= q) A[i0 * ld + j0 + q] = a[q];
+            for (int i = i0 + 32; i < d; i += 32) {  // the rows below
+                T b[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
-                    if (q < pw && i >= j0 + q) a[q] = A[i * ld + j0 + q];
+                    if (q < pw) b[q] = A[i * ld + j0 + q];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    if (q >= pw || i <= j0 + q) continue;
-                    const T c = a[q] * inv[q];
+                    if (q >= pw) break;
+                    const T c = b[q] * inv[q];
                     cb[q * d + i] = c;
 #pragma unroll
                     for (int l = q + 1; l < 4; ++l)
-                        if (l < pw && i >= j0 + l) {
-                            a[l] = fma(-c, D[l][q], a[l]);
-                            if (l == q + 1) A[i * ld + j0 + l] = a[l];
-                        }
+                        if (l < pw) b[l] = fma(-c, D[l][q], b[l]);
                 }
+#pragma unroll
+                for (int q = 1; q < 4; ++q)
+                    if (q < pw) A[i * ld + j0 + q] = b[q];
             }
         } else if (j0 > 0) {  // entries (i, l), l beyond this panel
             const int m = d - j0 - pw, n = m * (m + 1) / 2, st = nt - 32;

@@ -219,7 +219,7 @@ struct NiwPrior {
 // (launched with retry set, it takes only the flagged slots).
 // Psi_n (lower triangle, with the diagonal) and W (upper triangle, with the diagonal) share one
 // array of rows of ld T: W's entry (r, c) sits at column c + 1, so that W is in shared memory in
-// FP64 too up to d = 156 (d = 128, 192 slots: 1,526 us; 1,725 us with W in global memory).
+// FP64 too up to d = 156 (d = 128, 192 slots: 970 us).
 // Dynamic shared memory: (E doubles when staged) + (d * ld + 12 d) T (13 d + 2 in FP32).
 __device__ inline float log_t(float x) { return logf(x); }
 __device__ inline double log_t(double x) { return log(x); }
@@ -235,7 +235,7 @@ __host__ __device__ inline int niw_ld(int d) { return (d + 1) | 1; }
 // V (lower triangle) holds V_ri = U_ri / U_rr; row i is scaled by rd_i = 1 / U_ii at the end.
 // W^T v = eps: warp 0, lane m keeps sum_{j<m} W_jm v_j; the other warps store W meanwhile, and
 // warp 1 returns log det W.
-// d = 32: 15,900 cycles in FP32, 48,100 in FP64 (13,800 + 9,600 and 20,200 + 28,300 with a barrier
+// d = 32: 9,400 cycles in FP32, 33,300 in FP64 (13,800 + 9,600 and 20,200 + 28,300 with a barrier
 // per row, an integer division per entry and the sums' slot selected at run time).
 template <typename T, int R, int CB>
 __device__ __forceinline__ void niw_solve(T* W, int ws, const T* V, int ld, const T* rd, const T* Bd, const T* eps,
@@ -262,11 +262,12 @@ __device__ __forceinline__ void niw_solve(T* W, int ws, const T* V, int ld, cons
 #pragma unroll
                 for (int u = 0; u < CB; ++u) {
                     const int c = base + nw * u;
+                    // a column above r has only zeros from row r on: FP64 leaves it out (uniform), FP32
+                    // adds zeros, which is cheaper than the branch
+                    if (sizeof(T) == 8 && (c < r || c >= d)) continue;
                     const T w = __shfl_sync(0xffffffffu, a[u][sr], r & 31);
-                    if (c >= r && c < d) {  // a predicate: FP64 operations of finished columns are not issued
 #pragma unroll
-                        for (int q = 0; q <= sr; ++q) a[u][q] = fma(-v[q], w, a[u][q]);
-                    }
+                    for (int q = 0; q <= sr; ++q) a[u][q] = fma(-v[q], w, a[u][q]);
                 }
             }
 #pragma unroll

@@ -253,7 +253,7 @@ __device__ __forceinline__ void marginal_item(const SMArgs& a, double* Ltab, int
 // Log marginal likelihoods of every slot (cluster and sub-clusters) and merge pair, or, for
 // Gaussian data with many pairs, T_k of every cluster, from which merge_kernel bounds the
 // pairs.  An item is a chain of FP64 latencies, so pairs that an SM can take beside the slots
-// cost nothing (47 us at d = 32 for 60 slots alone and with 190 pairs).  The resident blocks
+// cost little (d = 32, 60 slots and 190 pairs: 38 us; 50 us before the lookahead factorisation).  The resident blocks
 // take the items in turn, so that no block is launched for the slots and pairs beyond K.
 constexpr int MARG_T = 160;
 __global__ void __launch_bounds__(MARG_T) marginal_kernel(SMArgs a, double* Ltab, int* derr) {
@@ -735,7 +735,7 @@ __global__ void __launch_bounds__(32 * BOUND_W) bound_kernel(SMArgs a, const dou
 // after removing emptied clusters).  bounded: bound_kernel has been there.  Many Gaussian pairs (not pairs_at_once): a warp bounds each pair's ratio from the means, the
 // block factorises in FP32 what that leaves open, and in FP64 what that leaves open; the FP64
 // factorisation of every pair was the step's cost (d = 128, K = 64: 2,016 pairs and 192 slots
-// 6.0 ms; now 0.8 ms for the slots and 1.2 ms for the pairs).
+// 6.0 ms; now 0.6 ms for the slots and 0.8 ms for the pairs).
 // Dynamic shared memory: marginal_item's; the bounds' u (a row of d floats per warp) share it.
 constexpr int MERGE_W = 8;  // warps
 
