@@ -40,9 +40,10 @@ METRIC = "point-sweeps/s (N*iters/s) d=32 N=1e6, BF16/TF32-TC vs FP64-plain, one
 TRAFFIC_BYTES = {
     # 2 M points, K = 20: 256.227840 MB read + 8.569088 MB written
     ("labels_tc", "gauss_d32"): ((256.227840e6 + 8.569088e6) / 2e6, 0.0),
-    # 262,144 points, K = 56: 143.424256 MB read + written, of which the 56 factor images
-    # (69,632 B each, read once from DRAM, then from L2) are the cluster part
-    ("labels_x3", "gauss_d128"): ((143.424256e6 - 56 * 69632) / 262144, 69632.0),
+    # the three launches of a screened label step, 262,144 points, K = 56: 72.67 MB (screen) + 12.40
+    # (gather) + 16.56 (the open points), of which the 56 factor images (69,632 B each, read once
+    # from DRAM, then from L2) are the cluster part
+    ("labels_x3", "gauss_d128"): ((101.63e6 - 56 * 69632) / 262144, 69632.0),
     # 1 M points: 406.888161 MB read + written (the log theta image is a few KB)
     ("labels_tc_mult", "multinomial"): (406.888161e6 / 1e6, 0.0),
     # the newsgroups shape itself (11,314 documents, K = 20): 23.561 MB read + written per
