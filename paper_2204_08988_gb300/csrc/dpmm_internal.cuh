@@ -275,8 +275,9 @@ struct dpmm_ctx {
     void* x3_xn = nullptr;    // screening (BF16X3, large N): per point |x_h|, |x_l|
     void* x3_list = nullptr;  // the points it leaves open, their gathered tiles,
     void* x3_cimg = nullptr;
-    void* x3_words = nullptr; // its words, then per cluster |W_h|, |W_l|, |mu|
+    void* x3_words = nullptr; // its words
     void* x3_fimg = nullptr;  // split-BF16 factor image (BF16X3), K_max clusters
+    void* x3_kn = nullptr;    // per cluster |W_h|, |W_l|, |mu| of the factors in x3_fimg
     double* cweights = nullptr;  // K_max: pi_k of the last sweep (linear)
     double* eps = nullptr;       // 3 K_max x d: normals of the drawn means
     double* bart = nullptr;      // 3 K_max x d: Bartlett diagonal (chi-square roots)

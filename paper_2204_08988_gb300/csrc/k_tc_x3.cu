@@ -627,11 +627,11 @@ __global__ void x3_points_kernel(const float* X, int64_t N, int d, int xs, Geo g
 // element (j, kk) at (j / 8) * 256 + (kk / 8) * 128 + (j % 8) * 16 + (kk % 8) * 2) holds the
 // three BF16 parts of -b_j, b_j = sum_m mu_m (W_h + W_l)[m][j] formed in FP64 with the
 // factor as the tensor cores see it.
-// Then the norms |W_h|, |W_l|, |mu| (rounded up) of cluster k into kn[k], where kn is given.
+// Then the norms |W_h|, |W_l|, |mu| (rounded up) of cluster k into kn[k].
 __global__ void x3_factor_kernel(const int* dK, int Kmax, int d, Geo g, const double* pW, const double* pmu,
                                  unsigned char* img, float4* kn) {
     const int K = min(*dK, Kmax);
-    for (int k = blockIdx.x; kn && k < K; k += gridDim.x) {
+    for (int k = blockIdx.x; k < K; k += gridDim.x) {
         __shared__ float part[3][8];
         const double* W = pW + (size_t)3 * k * d * d;
         float v[3] = {0.f, 0.f, 0.f};
@@ -750,7 +750,7 @@ static bool x3_screen_alloc(dpmm_ctx* c) {
     if (!roomy((sizeof(float2) + sizeof(int)) * c->N + cbytes, 0)) return false;
     cudaError_t e = cudaMalloc(&c->x3_xn, sizeof(float2) * c->N);
     if (e == cudaSuccess) e = cudaMalloc(&c->x3_list, sizeof(int) * c->N);
-    if (e == cudaSuccess && !c->x3_words) e = cudaMalloc(&c->x3_words, 4 * sizeof(int) + sizeof(float4) * c->K_max);
+    if (e == cudaSuccess && !c->x3_words) e = cudaMalloc(&c->x3_words, 4 * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&c->x3_cimg, cbytes);
     if (e == cudaSuccess) return true;
     cudaGetLastError();
@@ -777,8 +777,14 @@ cudaError_t x3_prepare_data(dpmm_ctx* c) {
         e = cudaMemsetAsync(c->x3_fimg, 0, (size_t)c->K_max * g.cbytes, c->stream);
         if (e != cudaSuccess) return e;
     }
+    if (!c->x3_kn) {  // the factors' norms outlast the data as the factors do: new data may be screened by them
+        cudaError_t e = cudaMalloc(&c->x3_kn, sizeof(float4) * c->K_max);
+        if (e != cudaSuccess) return e;
+        e = cudaMemsetAsync(c->x3_kn, 0, sizeof(float4) * c->K_max, c->stream);
+        if (e != cudaSuccess) return e;
+    }
     if (x3_screen_alloc(c)) {
-        cudaError_t e = cudaMemsetAsync(c->x3_words, 0, 4 * sizeof(int) + sizeof(float4) * c->K_max, c->stream);
+        cudaError_t e = cudaMemsetAsync(c->x3_words, 0, 4 * sizeof(int), c->stream);
         if (e != cudaSuccess) return e;
         x3::x3_norm_kernel<<<8 * c->num_sms, 256, 0, c->stream>>>((const float*)c->X, c->N, c->d, c->xs, (float2*)c->x3_xn);
     }
@@ -787,14 +793,12 @@ cudaError_t x3_prepare_data(dpmm_ctx* c) {
     return cudaGetLastError();
 }
 
-static float4* x3_kn(const dpmm_ctx* c) { return c->x3_cimg ? (float4*)((int*)c->x3_words + 4) : nullptr; }
-
 // per sweep, after the parameters are drawn: the factor image
 cudaError_t x3_prepare(dpmm_ctx* c) {
     if (!c->x3_fimg) return cudaErrorNotSupported;
     const x3::Geo g = x3_geo(c, nullptr);
     x3::x3_factor_kernel<<<2 * c->num_sms, 256, 0, c->stream>>>(c->dK, c->K_max, c->d, g, c->p_W, c->p_mu,
-                                                                (unsigned char*)c->x3_fimg, x3_kn(c));
+                                                                (unsigned char*)c->x3_fimg, (float4*)c->x3_kn);
     c->nlaunch += 1;
     return cudaGetLastError();
 }
@@ -836,7 +840,7 @@ cudaError_t launch_labels_x3(dpmm_ctx* c, uint64_t seed) {
         b.ximg = a.ximg;
         b.fimg = a.fimg;
         b.qc = c->q_c;
-        b.kn = x3_kn(c);
+        b.kn = (const float4*)c->x3_kn;
         b.xn = (const float2*)c->x3_xn;
         b.z = c->z;
         b.list = (int*)c->x3_list;
