@@ -500,9 +500,13 @@ __global__ void __launch_bounds__(128) labels_niw64_kernel(Niw64 a) {
         };
         auto admit = [&](int k, float c, float qlo, float qhi) {
             const float slack = 1e-3f + 1e-6f * fabsf(c);
-            const float U = c - 0.5f * (qlo * 0.99998f) + slack;
+            float U = c - 0.5f * (qlo * 0.99998f) + slack;
             float L = c - 0.5f * (qhi * 1.00002f) - slack;
-            if (!(U > -INFINITY) || U + 37.5f < low) return;
+            if (!(fabsf(U) < INFINITY)) {  // c or a square left FP32's range
+                if (!(__ldg(a.c + 3 * k) > -INFINITY)) return;  // weight zero, or NaN
+                U = INFINITY;
+            }
+            if (U + 37.5f < low) return;
             if (!(fabsf(L) < INFINITY)) {  // nothing known: FP64 decides
                 L = -INFINITY;
                 sure = false;
@@ -557,7 +561,7 @@ __global__ void __launch_bounds__(128) labels_niw64_kernel(Niw64 a) {
 #pragma unroll
                 for (int u = 0; u < NIW_B; ++u)
                     if (j0 + u < d) square(y[u], ga * __ldg(qn + j0 + u), qlo, qhi);
-                if (qlo > thr) return;
+                if (qlo > thr && qlo < INFINITY) return;  // a sum that overflowed bounds nothing
             }
             admit(k, c, qlo, qhi);
         };
@@ -612,7 +616,7 @@ __global__ void __launch_bounds__(128) labels_niw64_kernel(Niw64 a) {
 #pragma unroll
             for (int u = 0; u < NIW_B; ++u)
                 if (u < wl) square(y[u], ga * en[u], qlo, qhi);
-            if (k != hint && !(qlo > bound(c))) pend[np++ * nt] = (short)k;
+            if (k != hint && !(qlo > bound(c) && qlo < INFINITY)) pend[np++ * nt] = (short)k;
             __syncwarp();  // the stage is filled again
         }
         purge();
