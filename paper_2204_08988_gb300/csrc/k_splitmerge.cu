@@ -15,6 +15,7 @@
 #include <math.h>
 
 #include <cmath>
+#include <type_traits>
 
 #include "dpmm_internal.cuh"
 #include "fp64_chol.cuh"
@@ -299,18 +300,18 @@ __device__ __forceinline__ void marginal_counts_item(const SMArgs& a, const Src&
     }
     using V = decltype(cnt(0, 0));  // the source's own type: FP32 sums stay off the FP64 pipe
     const int s0 = 2 * k1 + (h < 0 ? 0 : h);
-    // the counts are added as integers (exact, as FP64 adds of them are): a conversion to FP64
-    // and an FP64 add a category kept the two-lane FP64 pipe busy two thirds of the time
-    // (d = 20,000, K = 20: 46 us, from 66)
-    unsigned long long si = 0;
+    // compressed rows hold whole counts, which are added as integers (exact, as FP64 adds of them
+    // are): a conversion to FP64 and an FP64 add a category kept the two-lane FP64 pipe busy two
+    // thirds of the time (d = 20,000, K = 20: 46 us, from 66).  Dense data may hold fractions.
+    std::conditional_t<sizeof(V) == 4, unsigned long long, double> si = 0;
     double acc = 0.0;
     for (int j = tid; j < d; j += nt) {
         V c = cnt(s0, j);
         if (h < 0) c += cnt(2 * k1 + 1, j);
-        if (k2 >= 0) c += cnt(2 * k2, j) + cnt(2 * k2 + 1, j);  // integer counts: exact
+        if (k2 >= 0) c += cnt(2 * k2, j) + cnt(2 * k2 + 1, j);  // whole counts: exact
         if (c > V(0)) {
             if constexpr (sizeof(V) == 4) si += (unsigned)c;
-            else si += (unsigned long long)c;
+            else si += c;
             acc += (lgt && c < (V)nlgt) ? lgt[(int)c] : lgamma(a.beta[j] + (double)c) - lgb[j];
         }
     }
