@@ -582,6 +582,11 @@ __device__ inline double merge_ratio(const SMArgs& a, const double* Ltab, int p,
     return lgp[0] + Ltab[3 * a.K_max + p] - lgp[1] + merge_rest(a, Ltab, k1, k2);
 }
 
+// The FP32 bounds' errors are relative, so a pair that has a diagonal entry of T_1 + T_2 below
+// this stays open: denormal numbers lose bits (entries beside such a diagonal lose 2^-149, which
+// is 2^-50 of it).
+constexpr float MERGE_MIN = 1e-30f;
+
 // A merge is refused whatever its uniform (log u >= -36.8) when an upper bound of log H says so.
 // log H falls by nu_n / 2 times whatever log|Psi| grows, so a lower bound ld of the pair's log
 // determinant gives one.  In FP64 but for lgammaf and logf; lgm = sum_j lgamma((nu_n - j) / 2).  The
@@ -620,13 +625,16 @@ __device__ inline bool refused_by_means(const SMArgs& a, const double* Ltab, int
     const float* T1 = a.T32 + (size_t)k1 * d * d;
     const float* T2 = a.T32 + (size_t)k2 * d * d;
     float du = 0.f;
+    bool in_range = true;
     for (int j = lane; j < d; j += 32) {
         const float dl = (float)(a.xbar[(size_t)k1 * d + j] - a.xbar[(size_t)k2 * d + j]);
-        const float v = dl / (T1[j * d + j] + T2[j * d + j]);
+        const float m = T1[j * d + j] + T2[j * d + j], v = dl / m;
+        in_range = in_range && m >= MERGE_MIN;
         u[j] = v;
         du = fmaf(dl, v, du);
     }
     __syncwarp();
+    if (!__all_sync(0xffffffffu, in_range)) return false;
     float qf = 0.f, qa = 0.f;
 #pragma unroll 4
     for (int j = 0; j < d; ++j) {
@@ -675,6 +683,7 @@ __device__ inline bool refused_by_factor(const SMArgs& a, const double* Ltab, in
         for (int l = tid & 31; l <= j; l += 32) {
             const float b = T1[j * d + l] + T2[j * d + l] + w * dl[j] * dl[l];
             A[j * ld + l] = l == j ? b * keep : b;
+            if (l == j && !(b >= MERGE_MIN)) s_fail = 1;
         }
     __syncthreads();
     chol_ldl_blk<float>(A, d, ld, piv, cols, cols + 4 * d, nullptr, 0.f, &s_fail, nullptr, nt, [] { __syncthreads(); });
