@@ -591,7 +591,7 @@ constexpr float MERGE_MIN = 1e-30f;
 // log H falls by nu_n / 2 times whatever log|Psi| grows, so a lower bound ld of the pair's log
 // determinant gives one.  In FP64 but for lgammaf and logf; lgm = sum_j lgamma((nu_n - j) / 2).  The
 // margin, 60 + 4e-6 of the magnitudes of the terms, covers the FP32 functions (lgammaf: 6 ulp) and
-// an ld that is off by 8e-6 relative.  False when anything is NaN.
+// an ld that is off by 4e-6 (|ld| + d).  False when anything is NaN.
 __device__ inline bool refused_at(const SMArgs& a, const double* Ltab, int k1, int k2, double n1, double n2, double ld,
                                   float lgm) {
     const int d = a.L.d;
@@ -688,10 +688,19 @@ __device__ inline bool refused_by_factor(const SMArgs& a, const double* Ltab, in
     __syncthreads();
     chol_ldl_blk<float>(A, d, ld, piv, cols, cols + 4 * d, nullptr, 0.f, &s_fail, nullptr, nt, [] { __syncthreads(); });
     if (tid < 32) {
-        float v = 0.f;
-        for (int j = tid; j < d; j += 32) v += logf(piv[j]);
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        const bool r = !s_fail && refused_at(a, Ltab, k1, k2, n1, n2, (double)v, warp_lmvgamma(a, n1 + n2));
+        // the sum of logarithms and that of their magnitudes m: an ulp a logarithm and 9 additions are
+        // below 11 x 2^-24 m, also where the features' units differ so that the logarithms cancel
+        float v = 0.f, m = 0.f;
+        for (int j = tid; j < d; j += 32) {
+            const float t = logf(piv[j]);
+            v += t;
+            m += fabsf(t);
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            v += __shfl_xor_sync(0xffffffffu, v, o);
+            m += __shfl_xor_sync(0xffffffffu, m, o);
+        }
+        const bool r = !s_fail && refused_at(a, Ltab, k1, k2, n1, n2, (double)v - 1e-6 * m, warp_lmvgamma(a, n1 + n2));
         if (tid == 0) s_ref = r;
     }
     __syncthreads();
