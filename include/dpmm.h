@@ -318,7 +318,8 @@ dpmm_status dpmm_get_profile(dpmm_ctx* ctx, int cap, const char** names, int* la
  * in [0, K) and zbar[N] in {0, 1}.  Outputs, device memory of length 2K, 2K x d and
  * 2K x d x d: for sub-cluster slot 2k + h, n_out = count, sx_out = sum of x,
  * sxx_out = sum of x x^T over the points with (z, zbar) = (k, h), in FP64 (per-tile
- * FP32 sums, added to about 48 bits; in FP64 where they leave FP32's range).  Points whose label is outside that range are ignored.
+ * FP32 sums, added with FP64's precision).  Points whose label is outside that range
+ * are ignored.
  * The call is asynchronous on `stream` (a cudaStream_t or NULL).
  *
  * Limits: 1 <= d <= 32, 1 <= K <= 16, N >= 1; anything else returns DPMM_EINVAL

@@ -26,7 +26,8 @@ constexpr int NA_P = 128;      // points per tile
 constexpr int NA_EMAX = 16 * (((NA_DMAX + 4) / 4) * ((NA_DMAX + 4) / 4 + 1) / 2);  // 720 entries
 constexpr int NA_W = 8;        // warps per block
 constexpr int NA_Q = 4;        // tiles whose labels a warp scans at a time
-constexpr int NA_D = 8;        // rows in flight per warp
+constexpr int NA_D = 6;        // rows in flight per warp (8 spill registers at d > 16)
+constexpr int NA_CARRY = 640;  // additions to a sum before its words are made apart again
 constexpr int NA_ROW = 52;     // floats of a staged row: x, then its first d / 2 + 1 values again
 constexpr size_t NA_SCRATCH = (size_t)32 * 2 * NA_KMAX * NA_EMAX;  // doubles
 
@@ -65,27 +66,40 @@ __device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
     return r;
 }
 
-// Two sums, each an FP32 pair: s + c is the sum so far to about 48 bits.
-struct NaPair {
-    f2 s, c;
-    __device__ void zero() { s = c = 0ull; }
-    __device__ void add(f2 a) {  // two-sum: s + a = t + err exactly
-        const f2 t = f2_add(s, a), bb = f2_sub(t, s);
-        c = f2_add(c, f2_add(f2_sub(s, f2_sub(t, bb)), f2_sub(a, bb)));
-        s = t;
+// Knuth's two-sum: a becomes a + b rounded; its error, which is returned, is exact
+__device__ __forceinline__ f2 f2_two_sum(f2& a, f2 b) {
+    const f2 t = f2_add(a, b), bb = f2_sub(t, a);
+    const f2 err = f2_add(f2_sub(a, f2_sub(t, bb)), f2_sub(b, bb));
+    a = t;
+    return err;
+}
+
+// Two sums, each of three FP32 words: the errors of s are added up exactly in c, those of c in e.
+// With NA_CARRY = 640 additions from one carry to the next, |c| <= 641 x 2^-24 S and |e| <= 640 x 641 x
+// 2^-48 S (S: the largest partial sum), so an addition to e loses less than 2^-53 S, which is what
+// one to an FP64 sum may lose.
+struct NaSum {
+    f2 s, c, e;
+    __device__ void zero() { s = c = e = 0ull; }
+    __device__ void add(f2 a) { e = f2_add(e, f2_two_sum(c, f2_two_sum(s, a))); }
+    __device__ void carry() {  // the same sum with |c| <= 2^-24 |s|, |e| <= 2^-24 |c|
+        const f2 t = f2_two_sum(c, e);
+        c = f2_two_sum(s, c);
+        e = f2_two_sum(c, t);
     }
     __device__ double2 value() const {
-        const float2 x = f2_unpack(s), y = f2_unpack(c);
-        return make_double2((double)x.x + (double)y.x, (double)x.y + (double)y.y);
+        const float2 x = f2_unpack(s), y = f2_unpack(c), z = f2_unpack(e);
+        return make_double2((double)x.x + ((double)y.x + (double)z.x), (double)x.y + ((double)y.y + (double)z.y));
     }
     __device__ bool bad() const {
-        const float2 x = f2_unpack(s), y = f2_unpack(c);
-        return !isfinite(x.x) || !isfinite(y.x) || !isfinite(x.y) || !isfinite(y.y);
+        const float2 x = f2_unpack(s), y = f2_unpack(c), z = f2_unpack(e);
+        return !isfinite(x.x) || !isfinite(y.x) || !isfinite(z.x) || !isfinite(x.y) || !isfinite(y.y) || !isfinite(z.y);
     }
 };
 struct NaDouble {
     double2 v;
     __device__ void zero() { v = make_double2(0.0, 0.0); }
+    __device__ void carry() {}
     __device__ void add(f2 a) {
         const float2 x = f2_unpack(a);
         v.x += (double)x.x;
@@ -114,24 +128,30 @@ __host__ __device__ inline int na_entries(int d) { return (d / 2 + 2) * d + 1; }
 // warp in tiles of its own.  A warp scans four tiles' labels by ballots (every slot's block
 // reads them: 5 bytes a point from L2) and then takes its slot's own rows one after another,
 // so X crosses DRAM once: lane j holds x_j, and its partners x_(j + t) come from the row
-// staged in shared memory, eight rows being loaded while eight are added up.
+// staged in shared memory, NA_D rows being loaded while as many are added up.
 // What bounds it is the precision: a tile's points of one slot are summed in FP32 (point q
-// in group q mod W), and the groups' sums are added to about 48 bits.  In FP64 that is one
-// conversion and one add per entry and group on a pipe of two lanes an SM (2.3 ms at
-// d = 32, N = 1e6); as an FP32 pair it is six FP32 adds and one more.  A pair that
-// overflows or meets an infinity or NaN makes the block start over in FP64.
-// Measured at d = 32, K = 16, N = 1e6: 0.29 ms (fmaheavy pipe about 70% busy); 0.46 ms as 4 x 4 register blocks over staged
-// tiles (290 million instructions, half of them loops over tiles of four points); 21.4 ms for
-// 32 blocks that took a tile's 32 slots in turn, two block barriers each.
+// in group q mod W), and the groups' sums are added with the precision of FP64.  On the FP64 pipe
+// that is one conversion and one add per entry and group at two lanes an SM (2.3 ms at d = 32,
+// N = 1e6); as three FP32 words it is 13 FP32 adds.  A sum that overflows or meets an infinity or
+// NaN makes the block start over in FP64.
+// Measured at d = 32, K = 16, N = 1e6: 0.37 ms (0.51 with 8 rows in flight, which spill; 0.27 with two words,
+// 48 bits, whose second loses bits with the number of additions); 0.46 ms with two words as 4 x 4
+// register blocks over staged tiles (290 million instructions, half of them loops over tiles of four
+// points); 25.4 ms for 32 blocks that took a tile's 32 slots in turn, two block barriers each.
 template <int T, typename Acc>  // T: odd, at least d / 2 + 1
 __device__ __forceinline__ bool na_block(const NaArgs& a, float* row, int* list, double* red) {
     constexpr int NP = (T + 1) / 2;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int d = a.d, S = 2 * a.K, s = blockIdx.x, g = blockIdx.y, W = a.W;
     Acc acc[NP];  // t = 2 p and 2 p + 1; the last one's second: sum x_j
+    f2 f[NP];     // the group in hand
 #pragma unroll
-    for (int p = 0; p < NP; ++p) acc[p].zero();
+    for (int p = 0; p < NP; ++p) {
+        acc[p].zero();
+        f[p] = 0ull;
+    }
     unsigned long long count = 0;
+    int since = 0;  // additions since the last carry
     const int wm = 65536 / W + 1;  // n * wm >> 16 = n / W for 0 <= n <= 128, W <= 256
     const int64_t R = (a.N + NA_RANGES - 1) / NA_RANGES;
     const unsigned Tr = (unsigned)((R + NA_P - 1) / NA_P), tiles = NA_RANGES * Tr;  // tiles per range, in all
@@ -181,6 +201,12 @@ __device__ __forceinline__ bool na_block(const NaArgs& a, float* row, int* list,
             n += nu;
         }
         count += n;
+        if (since + n >= NA_CARRY) {  // n <= 512; the last group is added after the loop
+#pragma unroll
+            for (int p = 0; p < NP; ++p) acc[p].carry();
+            since = 0;
+        }
+        since += n;
         __syncwarp();
         float x[NA_D];
         auto fetch = [&](int q0) {
@@ -189,9 +215,6 @@ __device__ __forceinline__ bool na_block(const NaArgs& a, float* row, int* list,
                 x[q] = q0 + q < n ? __ldg(Xb + (int64_t)(list[q0 + q] & 0x7fffffff) * d) : 0.f;
         };
         fetch(0);
-        f2 f[NP];
-#pragma unroll
-        for (int p = 0; p < NP; ++p) f[p] = 0ull;
         for (int q0 = 0; q0 < n; q0 += NA_D) {
             __syncwarp();
 #pragma unroll
@@ -219,9 +242,9 @@ __device__ __forceinline__ bool na_block(const NaArgs& a, float* row, int* list,
                 }
             }
         }
-#pragma unroll
-        for (int p = 0; p < NP; ++p) acc[p].add(f[p]);
     }
+#pragma unroll
+    for (int p = 0; p < NP; ++p) acc[p].add(f[p]);
     bool bad = false;
 #pragma unroll
     for (int p = 0; p < NP; ++p) bad = bad || acc[p].bad();
@@ -257,7 +280,7 @@ __global__ void __launch_bounds__(32 * NA_W, 2) na_partial_kernel(NaArgs a) {
     float* row = (float*)((int*)sm + NA_W * LIST) + (threadIdx.x >> 5) * (NA_D * NA_ROW);
     for (int e = threadIdx.x & 31; e < NA_D * NA_ROW; e += 32) row[e] = 0.f;  // what no feature fills
     __syncwarp();
-    if (na_block<T, NaPair>(a, row, list, (double*)sm)) return;
+    if (na_block<T, NaSum>(a, row, list, (double*)sm)) return;
     for (int e = threadIdx.x & 31; e < NA_D * NA_ROW; e += 32) row[e] = 0.f;
     __syncthreads();
     na_block<T, NaDouble>(a, row, list, (double*)sm);
