@@ -391,6 +391,10 @@ inline bool roomy(size_t bytes, size_t later) {
     size_t free = 0, total = 0;
     return cudaMemGetInfo(&free, &total) == cudaSuccess && free >= bytes + later + ((size_t)1 << 30);
 }
+// what dpmm_stage_data's buffer and dpmm_update_data's copy of pageable values take later on
+inline size_t input_copies(const dpmm_ctx* c) {
+    return 2 * (size_t)c->N * c->d * (c->in_dt == DPMM_F64 ? 8 : c->in_dt == DPMM_BF16 ? 2 : 4);
+}
 cudaError_t tc_prepare(dpmm_ctx* c);
 bool substats_tc_supported(const dpmm_ctx* c);
 cudaError_t substats_tc_prepare(dpmm_ctx* c);

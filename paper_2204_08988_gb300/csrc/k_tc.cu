@@ -716,7 +716,7 @@ namespace dpmm {
 cudaError_t tc_carry_alloc(dpmm_ctx* c) {
     if (c->kind != DPMM_PRIOR_NIW || c->prec != DPMM_PREC_TF32 || !tc_supported(c) || tc_cfg(c).gmax <= 1) return cudaSuccess;
     const size_t full = (size_t)c->N * tc::carry_bytes(tc::HELD);
-    c->tc_held = roomy(full, (size_t)c->N * c->d * 8) ? tc::HELD : 1;  // a copy of the input (FP64 at most) follows
+    c->tc_held = roomy(full, input_copies(c)) ? tc::HELD : 1;
     cudaError_t e = cudaMalloc(&c->tc_carry, (size_t)c->N * tc::carry_bytes(c->tc_held));
     if (e != cudaSuccess) c->tc_carry = nullptr;
     return e;

@@ -747,7 +747,7 @@ static bool x3_screen_alloc(dpmm_ctx* c) {
     if (c->x3_cimg) return true;
     const int64_t ct = (x3_cap(c) + 127) / 128 + x3::MT;
     const size_t cbytes = (size_t)ct * x3_geo(c, nullptr).xtile;
-    if (!roomy((sizeof(float2) + sizeof(int)) * c->N + cbytes, 0)) return false;
+    if (!roomy((sizeof(float2) + sizeof(int)) * c->N + cbytes, input_copies(c))) return false;
     cudaError_t e = cudaMalloc(&c->x3_xn, sizeof(float2) * c->N);
     if (e == cudaSuccess) e = cudaMalloc(&c->x3_list, sizeof(int) * c->N);
     if (e == cudaSuccess && !c->x3_words) e = cudaMalloc(&c->x3_words, 4 * sizeof(int));
