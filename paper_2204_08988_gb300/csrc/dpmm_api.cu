@@ -207,22 +207,47 @@ static dpmm_status upload(dpmm_ctx* c, const void* X, dpmm_dtype dt, int on_devi
     return DPMM_OK;
 }
 
-// What the getters read about a chain, written to page-locked host memory by one kernel: a
-// getter then waits for the stream once (a copy and a wait each for K, the sweep index and the
-// error word took 31 us; this takes 10).
-enum { PUB_K = 0, PUB_ITER, PUB_COUNTERS, PUB_ERR = PUB_COUNTERS + 4, PUB_N };
-__global__ void publish_kernel(const int* dK, const uint32_t* diter, const int* counters, const int* derr, volatile int* out) {
-    const int t = threadIdx.x;
-    if (t < PUB_N) out[t] = t == PUB_K ? *dK : t == PUB_ITER ? (int)diter[0] : t == PUB_ERR ? *derr : counters[t - PUB_COUNTERS];
+// The words that the getters read about a chain lie in one block (dpmm_ctx::words): one copy and
+// one wait (10 us; 31 with a copy and a wait each for K, the sweep index and the error word).
+enum { W_K = 0, W_ITER = 1, W_COUNTERS = 4, W_ERR = 12, W_N = 16 };
+
+// Host memory that the words are copied to: 16 KB for the process, page-locked once (2 us less a
+// getter than pageable memory; page-locking some for every context took 0.2 ms of its life).  A
+// context holds one slot; those beyond W_SLOTS at a time take the caller's stack.  Where the
+// page-locking failed, or went with a device reset, the copies are those to pageable memory.
+constexpr int W_SLOTS = 256;
+static std::mutex g_words_mu;
+alignas(4096) static int g_words[W_SLOTS][W_N];
+static bool g_words_taken[W_SLOTS], g_words_locked = false;
+
+static int* words_take() {
+    std::lock_guard<std::mutex> lk(g_words_mu);
+    if (!g_words_locked) {
+        g_words_locked = true;
+        if (cudaHostRegister(g_words, sizeof(g_words), cudaHostRegisterPortable) != cudaSuccess) cudaGetLastError();
+    }
+    for (int s = 0; s < W_SLOTS; ++s)
+        if (!g_words_taken[s]) {
+            g_words_taken[s] = true;
+            return g_words[s];
+        }
+    return nullptr;
 }
 
-// Waits for the stream's work and fetches the words above into c->pub; *e: the device error
-// word's status (the word is cleared).
-static dpmm_status fetch(dpmm_ctx* c, dpmm_status* e) {
-    publish_kernel<<<1, 32, 0, c->stream>>>(c->dK, c->diter, c->counters, c->derr, c->pub);
-    CK(c, cudaGetLastError());
+static void words_give(int* slot) {
+    if (!slot) return;
+    std::lock_guard<std::mutex> lk(g_words_mu);
+    g_words_taken[(slot - g_words[0]) / W_N] = false;
+}
+
+// Waits for the stream's work and fetches the words; *e: the device error word's status (the word
+// is cleared).
+static dpmm_status fetch(dpmm_ctx* c, int w[W_N], dpmm_status* e) {
+    int* to = c->pub ? c->pub : w;
+    CK(c, cudaMemcpyAsync(to, c->words, sizeof(int) * W_N, cudaMemcpyDeviceToHost, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
-    const int h = c->pub[PUB_ERR];
+    if (to != w) memcpy(w, to, sizeof(int) * W_N);
+    const int h = w[W_ERR];
     *e = DPMM_OK;
     if (h != 0) {
         // cleared on the context's stream, so that the clear is ordered before any later
@@ -236,8 +261,9 @@ static dpmm_status fetch(dpmm_ctx* c, dpmm_status* e) {
 }
 
 static dpmm_status check_derr(dpmm_ctx* c) {
+    int w[W_N];
     dpmm_status e = DPMM_OK;
-    const dpmm_status s = fetch(c, &e);
+    const dpmm_status s = fetch(c, w, &e);
     return s != DPMM_OK ? s : e;
 }
 
@@ -451,11 +477,14 @@ dpmm_status dpmm_create(const dpmm_prior* prior, double alpha, int d, int K_max,
     const size_t S = 3 * (size_t)K_max;
     bool ok = true;
     auto A = [&](auto** p, size_t bytes) { ok = ok && dalloc(p, bytes) == cudaSuccess; };
-    A(&c->dK, sizeof(int));
-    A(&c->diter, 3 * sizeof(uint32_t));  // [sweep index, problem id, point offset]
+    A(&c->words, sizeof(int) * W_N);
+    if (c->words) {
+        c->dK = c->words + W_K;
+        c->diter = (uint32_t*)c->words + W_ITER;  // [sweep index, problem id, point offset]
+        c->counters = c->words + W_COUNTERS;      // 8
+        c->derr = c->words + W_ERR;
+    }
     A(&c->age, sizeof(int) * K_max);
-    A(&c->counters, sizeof(int) * 8);
-    A(&c->derr, sizeof(int));
     A(&c->stats, sizeof(double) * 2 * K_max * c->st.E);
     A(&c->shift_new, sizeof(double) * K_max * d);
     A(&c->shift_stats, sizeof(double) * K_max * d);
@@ -473,7 +502,7 @@ dpmm_status dpmm_create(const dpmm_prior* prior, double alpha, int d, int K_max,
     if (c->kind == DPMM_PRIOR_NIW) A(&c->p_b, sizeof(double) * S * d);
     A(&c->q_logtheta, sizeof(float) * S * d);
     A(&c->cweights, sizeof(double) * K_max);
-    A(&c->eps, sizeof(double) * S * d);
+    A(&c->eps, sizeof(double) * (S * d + 4));  // and what dpmm_get_stats unpacks of a compressed-row cluster
     A(&c->bart, sizeof(double) * S * d);
     A(&c->lgs, sizeof(double) * (S + 1));
     A(&c->retry, sizeof(int) * S);
@@ -512,30 +541,17 @@ dpmm_status dpmm_create(const dpmm_prior* prior, double alpha, int d, int K_max,
     }
     A(&c->Ltab, sizeof(double) * (3 * (size_t)K_max + 3 * ((size_t)K_max * (K_max - 1) / 2) + 1 + 6 * (size_t)K_max));
     A(&c->relabel, sizeof(int) * 4 * K_max);
-    if (c->kind == DPMM_PRIOR_NIW) {
-        A(&c->sm_T, sizeof(float) * (size_t)K_max * d * d);
-        A(&c->sm_xbar, sizeof(double) * (size_t)K_max * (d + 1));
-    }
     A(&c->acc, sizeof(int) * ((size_t)K_max + (size_t)K_max * (K_max - 1) / 2 + 1));
     A(&c->center, sizeof(double) * (2 * (size_t)d + (size_t)d * d));
-    {  // the getters' buffers: up to 4 MB of unpacked statistics, at least one cluster's
-        const size_t per = sizeof(double) * unpack_doubles(c->kind, d);
-        c->unpack_bytes = std::max(per, std::min(per * K_max, (size_t)4 << 20));
-        A(&c->unpack, c->unpack_bytes);
-        ok = ok && cudaHostAlloc((void**)&c->pub, sizeof(int) * 16, cudaHostAllocPortable) == cudaSuccess;
-    }
     if (!ok) {
         cudaGetLastError();  // the failed allocation's error is not left for a later call to report
         dpmm_destroy(c);
         return DPMM_ENOMEM;
     }
-    cudaMemset(c->derr, 0, sizeof(int));
-    cudaMemset(c->diter, 0, 3 * sizeof(uint32_t));
     cudaMemset(c->retry, 0, sizeof(int) * S);
-    cudaMemset(c->counters, 0, sizeof(int) * 8);
     cudaMemset(c->p_logw, 0, sizeof(double) * S);
-    cudaMemset(c->dK, 0, sizeof(int));
     cudaMemset(c->center, 0, sizeof(double) * (2 * (size_t)d + (size_t)d * d));
+    c->pub = words_take();
     // the memsets above run on the legacy stream; the context's stream may not wait for it
     if (cudaDeviceSynchronize() != cudaSuccess) {
         dpmm_destroy(c);
@@ -549,15 +565,15 @@ void dpmm_destroy(dpmm_ctx* c) {
     if (!c) return;
     if (c->stream) cudaStreamSynchronize(c->stream);
     free_data(c);
-    void* ps[] = {c->dK, c->diter, c->age, c->counters, c->derr, c->stats, c->shift_new, c->shift_stats,
+    void* ps[] = {c->words, c->age, c->stats, c->shift_new, c->shift_stats,
                   c->shift32, c->p_logw, c->p_mu, c->p_W, c->p_logdetW, c->p_c, c->p_logtheta, c->q_mu,
                   c->q_W, c->q_c, c->q_b, c->q_logtheta, c->cweights, c->tot, c->records, c->Ltab,
-                  c->relabel, c->acc, c->sm_T, c->sm_xbar, c->center, c->tc_img, c->tcs_img, c->tc_flag, c->dbg_scores, c->eps, c->bart, c->lgs, c->retry, c->x3_fimg, c->x3_kn, c->x3_words,
+                  c->relabel, c->acc, c->center, c->tc_img, c->tcs_img, c->tc_flag, c->dbg_scores, c->eps, c->bart, c->lgs, c->retry, c->x3_fimg, c->x3_kn, c->x3_words,
                   c->sp_cc, c->sp_ltT, c->sp_ct, c->sp_lgt, c->sp_lgb, c->sp_part, c->shard_scratch, c->p_b, c->mcnt,
-                  c->stage, c->unpack};
+                  c->stage};
     if (c->cstream) cudaStreamSynchronize(c->cstream);
     for (void* p : ps) dfree(p);
-    if (c->pub) cudaFreeHost(c->pub);
+    words_give(c->pub);
     if (c->ev_copied) cudaEventDestroy(c->ev_copied);
     if (c->ev_free) cudaEventDestroy(c->ev_free);
     if (c->cstream) cudaStreamDestroy(c->cstream);
@@ -1190,11 +1206,12 @@ dpmm_status dpmm_sweep_sharded(dpmm_ctx* const* sh, int G, int iters, uint64_t s
 
 dpmm_status dpmm_get_info(dpmm_ctx* c, int* K, uint32_t* iter) {
     if (!c) return DPMM_EINVAL;
+    int w[W_N];
     dpmm_status e = DPMM_OK;
-    const dpmm_status s = fetch(c, &e);
+    const dpmm_status s = fetch(c, w, &e);
     if (s != DPMM_OK) return s;
-    if (K) *K = c->pub[PUB_K];
-    if (iter) *iter = (uint32_t)c->pub[PUB_ITER];
+    if (K) *K = w[W_K];
+    if (iter) *iter = (uint32_t)w[W_ITER];
     return e;
 }
 
@@ -1208,14 +1225,16 @@ dpmm_status dpmm_get_labels(dpmm_ctx* c, int32_t* z, uint8_t* zbar) {
 
 dpmm_status dpmm_get_counters(dpmm_ctx* c, int out[4]) {
     if (!c || !out) return DPMM_EINVAL;
+    int w[W_N];
     dpmm_status e = DPMM_OK;
-    const dpmm_status s = fetch(c, &e);
+    const dpmm_status s = fetch(c, w, &e);
     if (s != DPMM_OK) return s;
-    for (int q = 0; q < 4; ++q) out[q] = c->pub[PUB_COUNTERS + q];
+    for (int q = 0; q < 4; ++q) out[q] = w[W_COUNTERS + q];
     return e;
 }
 
-// The table is unpacked on the device, as many clusters at a time as c->unpack holds, and
+// The table is unpacked on the device, into scratch that a sweep writes before it reads it (the ranges'
+// records; for compressed rows, which have none, eps), as many clusters at a time as that holds, and
 // copied into the caller's arrays (K = 60, d = 32: 98 us; 356 us with the packed table copied
 // and unpacked on the host).
 dpmm_status dpmm_get_stats(dpmm_ctx* c, int* Kout, int64_t* n, double* sx, double* sxx, double* weights) {
@@ -1223,27 +1242,40 @@ dpmm_status dpmm_get_stats(dpmm_ctx* c, int* Kout, int64_t* n, double* sx, doubl
     if (!c->X) return fail(c, DPMM_ESTATE, "no data");
     const int d = c->d, gaussian = c->kind == DPMM_PRIOR_NIW && sxx;
     const size_t per = unpack_doubles(c->kind, d);
-    const int C = (int)std::min<size_t>(c->K_max, c->unpack_bytes / sizeof(double) / per);
-    int K = 0;
+    double* const buf = c->sparse ? c->eps : c->records;
+    const size_t room = c->sparse ? 3 * (size_t)c->K_max * d + 4 : c->records_bytes / sizeof(double);
+    const int C = (int)std::min<size_t>(c->K_max, room / per);
+    int K = 0, dev = c->device;
+    cudaGetDevice(&dev);  // the caller's current device may be another one
+    const struct Device {
+        int back;
+        Device(int own, int cur) : back(own != cur ? cur : -1) {
+            if (back >= 0) cudaSetDevice(own);
+        }
+        ~Device() {
+            if (back >= 0) cudaSetDevice(back);
+        }
+    } on(c->device, dev);
     std::vector<double> head;
     dpmm_status e = DPMM_OK;
     for (int k0 = 0; k0 == 0 || k0 < K; k0 += C) {
         unpack_kernel<<<dim3(3, C), 256, (gaussian ? 2 : 0) * sizeof(double) * d, c->stream>>>(
-            c->stats, c->st, c->shift_stats, c->center, c->cweights, c->dK, gaussian, k0, C, c->unpack);
+            c->stats, c->st, c->shift_stats, c->center, c->cweights, c->dK, gaussian, k0, C, buf);
         CK(c, cudaGetLastError());
         if (k0 == 0) {
-            const dpmm_status s = fetch(c, &e);
+            int w[W_N];
+            const dpmm_status s = fetch(c, w, &e);
             if (s != DPMM_OK) return s;
-            K = c->pub[PUB_K];
+            K = w[W_K];
         }
         const size_t m = (size_t)std::min(C, K - k0);
         if (m == 0) break;
         const size_t at = 4 * (size_t)C;  // counts and weights, then the sums
         head.resize(at);
-        CK(c, cudaMemcpyAsync(head.data(), c->unpack, sizeof(double) * at, cudaMemcpyDeviceToHost, c->stream));
-        if (sx) CK(c, cudaMemcpyAsync(sx + (size_t)3 * k0 * d, c->unpack + at, sizeof(double) * 3 * m * d, cudaMemcpyDeviceToHost, c->stream));
+        CK(c, cudaMemcpyAsync(head.data(), buf, sizeof(double) * at, cudaMemcpyDeviceToHost, c->stream));
+        if (sx) CK(c, cudaMemcpyAsync(sx + (size_t)3 * k0 * d, buf + at, sizeof(double) * 3 * m * d, cudaMemcpyDeviceToHost, c->stream));
         if (gaussian)
-            CK(c, cudaMemcpyAsync(sxx + (size_t)3 * k0 * d * d, c->unpack + at + (size_t)3 * C * d, sizeof(double) * 3 * m * d * d,
+            CK(c, cudaMemcpyAsync(sxx + (size_t)3 * k0 * d * d, buf + at + (size_t)3 * C * d, sizeof(double) * 3 * m * d * d,
                                   cudaMemcpyDeviceToHost, c->stream));
         CK(c, cudaStreamSynchronize(c->stream));
         if (n) memcpy(n + 3 * k0, head.data(), sizeof(int64_t) * 3 * m);

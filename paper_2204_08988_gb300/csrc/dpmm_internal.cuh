@@ -246,6 +246,7 @@ struct dpmm_ctx {
     // chain state
     int32_t* z = nullptr;
     uint8_t* zbar = nullptr;
+    int* words = nullptr;     // device: the block that holds dK, diter, counters and derr
     int* dK = nullptr;        // device: current K
     uint32_t* diter = nullptr;// device: [sweep counter, problem id, point offset] (Philox words c1, c3; c0 offset)
     int* age = nullptr;       // device, K_max
@@ -292,7 +293,8 @@ struct dpmm_ctx {
     bool sorted = false;     // idx holds a permutation of the points (a sort has run on these data)
     int G2 = 0;              // most ranges of the sub-label/statistics step (records capacity)
     int Gr = 1;              // ranges used for the current data: about one per 512 points, at most G2
-    double* records = nullptr;  // (G2 + K_max) x 2 x E
+    double* records = nullptr;  // (G2 + K_max) x 2 x E; between two statistics steps, scratch: what the merge
+                                // bounds keep of every cluster, dpmm_get_stats' unpacked statistics
     size_t records_bytes = 0;
 
     // split/merge scratch
@@ -301,8 +303,6 @@ struct dpmm_ctx {
                              // pair lgamma(n) and lgamma(alpha + n) (K_max (K_max - 1))
     int* relabel = nullptr;  // 4 K_max
     int* acc = nullptr;      // K_max + K_max (K_max - 1)/2 accept flags of the split/merge proposals
-    float* sm_T = nullptr;     // NIW: K_max x d x d, Psi0 / 2 + scatter of every cluster (FP32)
-    double* sm_xbar = nullptr; // NIW: K_max x d cluster means, then K_max log determinants of sm_T
 
     // tensor-core path
     int* tc_flag = nullptr;        // device: 1 when K did not fit the tensor-core kernel
@@ -323,10 +323,7 @@ struct dpmm_ctx {
     double* sp_lgb = nullptr;      // lgamma(beta_j)
     void* sp_part = nullptr;       // 3 K_max x ceil(d / 2048) (max, sum exp) of the FP32 theta draws
 
-    // getters: unpacked statistics (device), the chain's words (page-locked host memory)
-    double* unpack = nullptr;
-    size_t unpack_bytes = 0;
-    int* pub = nullptr;
+    int* pub = nullptr;  // getters: where the words are copied to on the host (null: nowhere of its own)
 
     // point-sharded chains: this context's first point in the whole data set
     int64_t poff = 0;

@@ -881,9 +881,10 @@ static SMArgs sm_args(dpmm_ctx* c) {
         }
         a.lg_sum_beta = std::lgamma(a.sum_beta);
     }
-    a.T32 = c->sm_T;
-    a.xbar = c->sm_xbar;
-    a.ldT = c->sm_xbar ? c->sm_xbar + (size_t)c->K_max * c->d : nullptr;
+    // in the ranges' records, which have been added up: 8 (d + 1) + 4 d^2 of their 16 E bytes a cluster
+    a.xbar = c->records;
+    a.ldT = a.xbar + (size_t)c->K_max * c->d;
+    a.T32 = (float*)(a.ldT + c->K_max);
     a.stage = 0;
     a.exact = 0;
     a.kind = c->kind;
