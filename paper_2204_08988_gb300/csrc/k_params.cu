@@ -219,7 +219,7 @@ struct NiwPrior {
 // (launched with retry set, it takes only the flagged slots).
 // Psi_n (lower triangle, with the diagonal) and W (upper triangle, with the diagonal) share one
 // array of rows of ld T: W's entry (r, c) sits at column c + 1, so that W is in shared memory in
-// FP64 too up to d = 156 (d = 128, 192 slots: 970 us).
+// FP64 too up to d = 153 (d = 128, 192 slots: 970 us).
 // Dynamic shared memory: (E doubles when staged) + (d * ld + 12 d) T (13 d + 2 in FP32).
 __device__ inline float log_t(float x) { return logf(x); }
 __device__ inline double log_t(double x) { return log(x); }
@@ -664,7 +664,8 @@ cudaError_t launch_params(dpmm_ctx* c, uint64_t seed) {
         };
         int st64, w64, st32, w32;
         const size_t sm64 = plan(8, st64, w64), sm32 = plan(4, st32, w32);
-        // FP32 up to the d whose matrices and statistics fit 200 KB unpacked (d <= 125), FP64 above
+        // FP32 where the matrices, unpacked, and the statistics, if both fit, are within 200 KB (d <= 127, and
+        // 156 and 157, whose statistics do not fit beside one matrix), FP64 elsewhere
         const size_t base = 4 * ((size_t)c->d * (c->d | 1) + 11 * (size_t)c->d), sq = 4 * (size_t)c->d * c->d;
         const bool fp32 = c->prec != DPMM_PREC_FP64_PLAIN && w32 &&
                           base + (base + 8 * E <= 200 * 1024 ? 8 * E : 0) + sq <= 200 * 1024;
