@@ -346,7 +346,6 @@ struct Niw64 {
     const int* dK;
     const uint32_t* diter;
     uint64_t seed;
-    const int* gate;
     int32_t* z;
 };
 
@@ -356,7 +355,6 @@ struct Niw64 {
 // last columns of W, mu - mu_0).
 template <bool VEC>  // VEC: d is a multiple of 4, rows of the FP32 W are 16-byte aligned
 __global__ void __launch_bounds__(128) labels_niw64_kernel(Niw64 a) {
-    if (a.gate && *a.gate == 0) return;
     extern __shared__ __align__(16) unsigned char smraw[];
     const int K = *a.dK, d = a.d, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, ld = nt + 1;
     double* sd = (double*)smraw + tid;                    // x - mu of the cluster in hand, FP64
@@ -2217,7 +2215,7 @@ static cudaError_t labels_simt_t(dpmm_ctx* c, uint64_t seed, const int* gate) {
 
 // Gaussian FP64 labels without the score hook.  Blocks of 32 to 128 points: the most that
 // still give every SM two blocks.
-static cudaError_t labels_niw64(dpmm_ctx* c, uint64_t seed, const int* gate) {
+static cudaError_t labels_niw64(dpmm_ctx* c, uint64_t seed) {
     const int d = c->d;
     const size_t per = ((size_t)d * d + d + 1) * sizeof(double);  // d too large for labels_simt_kernel: refused here too
     if ((size_t)32 * (d + 1) * sizeof(double) + per > 200 * 1024) return cudaErrorInvalidValue;
@@ -2228,10 +2226,9 @@ static cudaError_t labels_niw64(dpmm_ctx* c, uint64_t seed, const int* gate) {
     auto kern = d % 4 == 0 ? labels_niw64_kernel<true> : labels_niw64_kernel<false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(TB));
     if (e != cudaSuccess) return e;
-    const int64_t tiles = (c->N + TB - 1) / TB;
-    const int grid = (int)(gate ? std::min<int64_t>(tiles, (int64_t)c->num_sms) : tiles);
+    const int grid = (int)((c->N + TB - 1) / TB);
     Niw64 a{d, c->xs, c->N, (const double*)c->X, c->p_W, c->p_mu, c->p_c, c->q_W, c->q_mu, c->q_b,
-            c->q_c, c->sorted ? c->idx : nullptr, c->dK, c->diter, seed, gate, c->z};
+            c->q_c, c->sorted ? c->idx : nullptr, c->dK, c->diter, seed, c->z};
     kern<<<grid, TB, bytes(TB), c->stream>>>(a);
     return cudaGetLastError();
 }
@@ -2270,7 +2267,7 @@ cudaError_t launch_labels_simt_gated(dpmm_ctx* c, uint64_t seed, const int* gate
         else
             e = c->d <= 2 ? labels_small_t<float, 2>(c, seed) : c->d <= 4 ? labels_small_t<float, 4>(c, seed)
               : c->d <= 8 ? labels_small_t<float, 8>(c, seed) : labels_small_t<float, 16>(c, seed);
-    } else if (c->kind == DPMM_PRIOR_NIW && c->prec == DPMM_PREC_FP64_PLAIN && !c->dbg_scores) e = labels_niw64(c, seed, gate);
+    } else if (c->kind == DPMM_PRIOR_NIW && c->prec == DPMM_PREC_FP64_PLAIN && !c->dbg_scores) e = labels_niw64(c, seed);
     else if (c->prec == DPMM_PREC_FP64_PLAIN) e = labels_simt_t<double, double>(c, seed, gate);
     else if (c->xdt == 2) e = labels_simt_t<float, __nv_bfloat16>(c, seed, gate);
     else e = labels_simt_t<float, float>(c, seed, gate);
