@@ -1,11 +1,14 @@
 // k_sweep.cu -- the label step and the sufficient statistics (Sec. 4.1 steps (e),
 // (f); Sec. 4.4 "updating the sufficient statistics" in three steps).
 //
-//   labels_simt  : z_i = argmax_k [log pi_k + log f(x_i; theta_k) + G_ik] on CUDA
-//                  cores (FP64 parity path, FP32 for small d), one thread per point,
-//                  cluster parameters staged in shared memory and read by broadcast.
-//   hist/scan/scatter : stable counting sort of the points by cluster (tiles of 256
-//                  points), so that the next kernel sees each cluster as one run.
+//   labels       : z_i = argmax_k [log pi_k + log f(x_i; theta_k) + G_ik] on CUDA cores.
+//                  labels_small: Gaussian, d <= 8 (FP64) or 16 (FP32), all clusters'
+//                  parameters in shared memory.  labels_niw64: Gaussian FP64, scores
+//                  enclosed in FP32 first.  labels_simt: what is left (FP32 at larger d or
+//                  K_max, multinomial data, every score for the score hook), one thread
+//                  per point, parameters staged in chunks and read by broadcast.
+//   hist/scan/scatter : stable counting sort of the points by cluster (tiles of
+//                  SORT_TILE points), so that the next kernel sees each cluster as one run.
 //   substats     : per sorted run, z-bar_i from the two sub-clusters of z_i, then the
 //                  per-sub-cluster sums of xt xt^T (xt = [x - shift_k, 1]) as 4x4
 //                  register blocks, one partial record per (CTA, cluster) run.
@@ -2233,7 +2236,9 @@ static cudaError_t labels_niw64(dpmm_ctx* c, uint64_t seed) {
     return cudaGetLastError();
 }
 
-// labels_small_kernel where it applies: every cluster's padded parameters in 100 KB
+// labels_small_kernel where it applies: the padded parameters of K_max clusters in 100 KB, two blocks to
+// an SM (the launch does not know K).  Beyond (FP32: K_max 93 at d > 8, 350 at d > 4; FP64: 175 at
+// d > 4) the kernels of larger d take over, which stage clusters in turn.
 template <typename T, int DV>
 static cudaError_t labels_small_t(dpmm_ctx* c, uint64_t seed) {
     const size_t smem = (size_t)c->K_max * (DV * DV + DV + 1) * sizeof(T);

@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(STHREADS, 1) x3_screen_kernel(ScreenArgs a) {
                         Lb[j] = L;
                         Ub[j] = U;
                         kb[j] = k;
-                    } else if (!(U <= U2[j])) {  // a NaN stays and leaves the point open
+                    } else if (!(U <= U2[j])) {  // NaN only where q is, and then the full score too: no contender
                         U2[j] = U;
                     }
                 }
