@@ -157,6 +157,10 @@ __device__ inline float gumbel_approx(uint32_t a, uint32_t b) {
     return -logf(e);
 }
 
+// Two values s + G cannot be told apart by approximate G when they are this close: G's errors, and the
+// rounding of the sums (size: their magnitude), which makes equals of them where s is large.
+__device__ inline double approx_margin(double size) { return 4 * GUMBEL_APPROX + 1e-15 * size; }
+
 template <typename T>
 __device__ inline T gmin();  // below every Gumbel value of the precision
 template <>
@@ -282,7 +286,7 @@ __global__ void __launch_bounds__(256) labels_small_kernel(int d, int xs, int64_
             };
             reduce();
             if constexpr (sizeof(T) == 8) {
-                const T cut = vb - 4 * GUMBEL_APPROX;
+                const T cut = vb - approx_margin(fabs(vb));
                 const bool near = need && vs >= cut;
                 if (__any_sync(0xffffffffu, near)) {
                     const int keep = kv;
@@ -634,15 +638,16 @@ __global__ void __launch_bounds__(128) labels_niw64_kernel(Niw64 a) {
                 cu[e * nt] = g;
                 vmax = fmax(vmax, csc[e * nt] + (double)g);
             }
+            const double cut = vmax - approx_margin(fabs(vmax));
             int m = 0;  // the contenders that the approximation cannot tell from the best
             for (int e = 0; e < nc; ++e)
-                if (csc[e * nt] + (double)cu[e * nt] >= vmax - 4 * GUMBEL_APPROX) {
+                if (csc[e * nt] + (double)cu[e * nt] >= cut) {
                     csc[m * nt] = csc[e * nt];
                     ck[m * nt] = ck[e * nt];
                     ++m;
                 }
             nc = m;
-            if (nc == 1 && !(drawn && vb >= vmax - 4 * GUMBEL_APPROX)) kb = ck[0];
+            if (nc == 1 && !(drawn && vb >= cut)) kb = ck[0];
             else draw_all();
         }
         if (live) a.z[i] = kb;
@@ -925,7 +930,7 @@ __global__ void __launch_bounds__(MAXT) substats_kernel(SubArgs<T> a) {
                 bool near = true;  // FP64: an FP32 Gumbel difference decides where it can
                 if constexpr (sizeof(T) == 8) {
                     const T diff = (sr - sl) + (T)(gumbel_approx(w[2], w[3]) - gumbel_approx(w[0], w[1]));
-                    near = !(fabs(diff) > 4 * GUMBEL_APPROX);
+                    near = !(fabs(diff) > approx_margin(fabs(sl) + fabs(sr)));
                     h = diff > 0 ? 1 : 0;
                 }
                 if (near) h = sr + gumbel_of<T>(w[2], w[3]) > sl + gumbel_of<T>(w[0], w[1]) ? 1 : 0;
@@ -1164,7 +1169,7 @@ __global__ void __launch_bounds__(MAXT) substats_niw64_kernel(Sub64 b) {
                     const double sl = a.pv.c[3 * k + 1] - 0.5 * q0, sr = a.pv.c[3 * k + 2] - 0.5 * q1;
                     const double diff = (sr - sl) + (double)(gumbel_approx(w[2], w[3]) - gumbel_approx(w[0], w[1]));
                     int h = diff > 0 ? 1 : 0;
-                    if (!(fabs(diff) > 4 * GUMBEL_APPROX))
+                    if (!(fabs(diff) > approx_margin(fabs(sl) + fabs(sr))))
                         h = sr + gumbel_of<double>(w[2], w[3]) > sl + gumbel_of<double>(w[0], w[1]) ? 1 : 0;
                     a.zbar[i] = (uint8_t)h;
                     hq[p] = (unsigned char)h;
