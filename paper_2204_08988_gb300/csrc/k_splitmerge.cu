@@ -53,12 +53,6 @@ __device__ inline double smv(const SMArgs& a, int k, int h, int j, int l) {
     return a.stats[(size_t)(2 * k) * a.L.E + e] + a.stats[(size_t)(2 * k + 1) * a.L.E + e];
 }
 
-__device__ inline double lmvgamma(double x, int d) {
-    double s = 0.25 * d * (d - 1) * log(M_PI);
-    for (int j = 1; j <= d; ++j) s += lgamma(x + 0.5 * (1 - j));
-    return s;
-}
-
 // per-slot lgamma table after the log marginals: lg[2 s] = lgamma(n_s),
 // lg[2 s + 1] = lgamma(alpha / 2 + n_s)
 __host__ __device__ inline size_t lg_offset(int K_max) { return 3 * (size_t)K_max + (size_t)K_max * (K_max - 1) / 2 + 1; }

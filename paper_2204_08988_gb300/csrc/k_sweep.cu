@@ -2342,10 +2342,6 @@ static SubCfg sub_cfg_f32(const dpmm_ctx* c, int DV) {
     return q;
 }
 
-size_t substats_smem(const dpmm_ctx* c) {
-    return c->prec == DPMM_PREC_FP64_PLAIN ? sub_cfg<double>(c).smem : sub_cfg<float>(c).smem;
-}
-
 template <typename T, typename XT>
 static cudaError_t substats_t(dpmm_ctx* c, uint64_t seed, int draw, const int* gate) {
     SubCfg q = sub_cfg<T>(c);
