@@ -565,8 +565,23 @@ __global__ void derive_kernel(int kind, int d, int tf32, int fp64, const int* dK
                               float* shift32) {
     const int K = *dK;
     const int s = blockIdx.x;
-    if (s >= 3 * K) return;
     const int tid = threadIdx.x, nt = blockDim.x;
+    if (fp64 && kind == DPMM_PRIOR_NIW) {
+        // for the FP32 enclosures of the FP64 label step: mu - mu_0 and its norm, of the slots beyond K
+        // too, whose last parameters a later label step without the parameter step may use (K grows by
+        // splits): mu_0 has changed for them as well
+        for (int j = tid; j < d; j += nt) q_mu[(size_t)s * d + j] = (float)(p_mu[(size_t)s * d + j] - p_mu[j]);
+        if (tid < 32) {
+            float n2 = 0.f;
+            for (int j = tid; j < d; j += 32) {
+                const float m = (float)(p_mu[(size_t)s * d + j] - p_mu[j]);
+                n2 = fmaf(m, m, n2);
+            }
+            for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+            if (tid == 0) q_c[s] = sqrtf(n2);
+        }
+    }
+    if (s >= 3 * K) return;
     if (kind == DPMM_PRIOR_NIW) {
         const double* W = p_W + (size_t)s * d * d;
         const double* mu = p_mu + (size_t)s * d;
@@ -584,8 +599,7 @@ __global__ void derive_kernel(int kind, int d, int tf32, int fp64, const int* dK
             }
         }
         for (int j = tid; j < d; j += nt) {
-            if (fp64) {  // for the FP32 enclosures of the FP64 label step: mu - mu_0 and ||W_j||
-                q_mu[(size_t)s * d + j] = (float)(mu[j] - p_mu[j]);
+            if (fp64) {  // ||W_j||
                 float n2 = 0.f;
 #pragma unroll 8
                 for (int l = 0; l < d; ++l) {
@@ -618,15 +632,6 @@ __global__ void derive_kernel(int kind, int d, int tf32, int fp64, const int* dK
         for (int j = j0 + tid; j < j1; j += nt) q_logtheta[(size_t)s * d + j] = (float)p_logtheta[(size_t)s * d + j];
     }
     if (tid == 0 && blockIdx.y == 0 && !fp64) q_c[s] = (float)p_c[s];
-    if (fp64 && kind == DPMM_PRIOR_NIW && tid < 32) {  // ||mu - mu_0||
-        float n2 = 0.f;
-        for (int j = tid; j < d; j += 32) {
-            const float m = (float)(p_mu[(size_t)s * d + j] - p_mu[j]);
-            n2 = fmaf(m, m, n2);
-        }
-        for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
-        if (tid == 0) q_c[s] = sqrtf(n2);
-    }
 }
 
 static StatView make_sv(dpmm_ctx* c) { return StatView{c->stats, c->st}; }
