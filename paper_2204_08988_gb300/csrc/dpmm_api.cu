@@ -568,7 +568,7 @@ void dpmm_destroy(dpmm_ctx* c) {
     void* ps[] = {c->words, c->age, c->stats, c->shift_new, c->shift_stats,
                   c->shift32, c->p_logw, c->p_mu, c->p_W, c->p_logdetW, c->p_c, c->p_logtheta, c->q_mu,
                   c->q_W, c->q_c, c->q_b, c->q_logtheta, c->cweights, c->tot, c->records, c->Ltab,
-                  c->relabel, c->acc, c->center, c->tc_img, c->tcs_img, c->tc_flag, c->dbg_scores, c->eps, c->bart, c->lgs, c->retry, c->x3_fimg, c->x3_kn, c->x3_words,
+                  c->relabel, c->acc, c->center, c->tc_img, c->tcs_img, c->tc_flag, c->eps, c->bart, c->lgs, c->retry, c->x3_fimg, c->x3_kn, c->x3_words,
                   c->sp_cc, c->sp_ltT, c->sp_ct, c->sp_lgt, c->sp_lgb, c->sp_part, c->shard_scratch, c->p_b, c->mcnt,
                   c->stage};
     if (c->cstream) cudaStreamSynchronize(c->cstream);
@@ -1403,24 +1403,34 @@ dpmm_status dpmm_label_scores(dpmm_ctx* c, double* scores) {
     CK(c, cudaMemcpyAsync(&K, c->dK, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
     const size_t bytes = sizeof(double) * (size_t)c->N * K;
-    CK(c, cudaMalloc(&c->dbg_scores, bytes));
     // the label kernel of this precision with the current parameters; the labels it
-    // draws are put back afterwards
+    // draws are put back afterwards.  Whatever fails, the hook is off again on return: a
+    // sweep would fill it for its own K.
+    double* out = nullptr;
     int32_t* zkeep = nullptr;
-    CK(c, cudaMalloc(&zkeep, sizeof(int32_t) * c->N));
-    CK(c, cudaMemcpyAsync(zkeep, c->z, sizeof(int32_t) * c->N, cudaMemcpyDeviceToDevice, c->stream));
-    const bool tc = c->prec == DPMM_PREC_TF32 || c->prec == DPMM_PREC_BF16;
-    cudaError_t e = c->sparse                   ? launch_sparse(c, c->seed, 3, nullptr)
-                    : c->prec == DPMM_PREC_BF16X3 ? launch_labels_x3(c, c->seed)
-                    : tc                        ? launch_labels_tc(c, c->seed)
-                                                : launch_labels_simt(c, c->seed);
-    CK(c, e);
-    CK(c, cudaMemcpyAsync(scores, c->dbg_scores, bytes, cudaMemcpyDeviceToHost, c->stream));
-    CK(c, cudaMemcpyAsync(c->z, zkeep, sizeof(int32_t) * c->N, cudaMemcpyDeviceToDevice, c->stream));
-    CK(c, cudaStreamSynchronize(c->stream));
+    cudaError_t e = cudaMalloc(&out, bytes);
+    if (e == cudaSuccess) e = cudaMalloc(&zkeep, sizeof(int32_t) * c->N);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(zkeep, c->z, sizeof(int32_t) * c->N, cudaMemcpyDeviceToDevice, c->stream);
+    if (e == cudaSuccess) {
+        const bool tc = c->prec == DPMM_PREC_TF32 || c->prec == DPMM_PREC_BF16;
+        c->dbg_scores = out;
+        e = c->sparse                     ? launch_sparse(c, c->seed, 3, nullptr)
+            : c->prec == DPMM_PREC_BF16X3 ? launch_labels_x3(c, c->seed)
+            : tc                          ? launch_labels_tc(c, c->seed)
+                                          : launch_labels_simt(c, c->seed);
+        c->dbg_scores = nullptr;
+        const cudaError_t back =
+            cudaMemcpyAsync(c->z, zkeep, sizeof(int32_t) * c->N, cudaMemcpyDeviceToDevice, c->stream);
+        if (e == cudaSuccess) e = back;
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(scores, out, bytes, cudaMemcpyDeviceToHost, c->stream);
+    const cudaError_t done = cudaStreamSynchronize(c->stream);
+    if (e == cudaSuccess) e = done;
     cudaFree(zkeep);
-    cudaFree(c->dbg_scores);
-    c->dbg_scores = nullptr;
+    cudaFree(out);
+    if (e != cudaSuccess) cudaGetLastError();  // the error is this call's, not a later one's
+    CK(c, e);
     return check_derr(c);
 }
 
